@@ -138,8 +138,8 @@ struct GroupWs {
   float* zy;         // [Tpad] target logits
   float* pyb;        // [Tpad] the targets' bf16 exchange-tile entries
   float* nll;        // [Tpad] per-row loss terms
-  float* part_s;     // [g_max, Tpad] per-member partial sums
-  float* part_m;     // [g_max, Tpad] per-member partial maxima
+  float* part_s;     // [2 g_max, Tpad] partial sums per member and column half
+  float* part_m;     // [2 g_max, Tpad] partial maxima
   void* ring;        // group_ring_bytes(T, d, V)
   uint32_t* outer;   // [2 rt] pass-A group barriers (first launch, redo launch)
   uint32_t* redo;    // [1 + rt] redo list
@@ -184,8 +184,7 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
                           int32_t d, int32_t V, const GroupArgs& a, int c_base, int c_end,
                           uint32_t* ring_ctr);
 // The divergence gradient on chip: d_h_s = G . W_s with G from both heads'
-// logits (recomputed tile by tile by groups of CTA pairs, 128-wide vocabulary
-// tiles) and the value sweep's kl, lse_s, lse_t; ctr (ctr_words) is zeroed here.
+// logits (recomputed tile by tile by groups of CTA pairs) and the value sweep's kl, lse_s, lse_t; ctr (ctr_words) is zeroed here.
 olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct, const void* W_s,
                                   int32_t d_s, const void* W_t, int32_t d_t, const int32_t* rows,
                                   const int32_t* n_rows, int32_t T, int32_t V, float inv_tau,

@@ -43,9 +43,10 @@
 //   Divergence mode (GM_KL: the gradient of OPD's per-token KL, Section 1,
 //   after the value sweep of lmhead_kl.cu has given KL and both heads' lse):
 //     the pass A layout with two products per Z job, the student's (K = d_s)
-//     and the teacher's (K = d_t) logits of a 128-column vocabulary tile in
-//     the two halves of the 256-column Z accumulator; the epilogue forms the
-//     exact G (reverse: g inv_tau p_s ((z_s - z_t) - (lse_s - lse_t) - KL),
+//     and then the teacher's (K = d_t) logits of a 256-column vocabulary tile
+//     in the Z accumulator, half of the previous round's accumulation between
+//     them; the epilogue holds the student's logits in registers (128 a
+//     thread) until the teacher's arrive and forms the exact G (reverse: g inv_tau p_s ((z_s - z_t) - (lse_s - lse_t) - KL),
 //     forward: g inv_tau (p_s - p_t)) and the members accumulate
 //     d_h_s = G . W_s.
 //
@@ -78,7 +79,19 @@
 // TMEM columns).  Waits between members go through global release/acquire
 // counters: a slot's `ready` count (tile written) and `cons` count (tile
 // copied by all g members); the producer warp checks a whole round's ready
-// flags at once and a signal warp posts the cons counts.  Every dependency
+// flags at once and a signal warp posts the cons counts.  Eight
+// epilogue warps, two per TMEM lane quadrant with half of a tile's columns
+// each, stage their bf16 values in shared memory and move them to the ring
+// with 4 KB bulk stores, one `ready` count a warp; a finished output
+// accumulator is taken into registers (up to 128 a thread) and handed back
+// before it is converted and stored.  With four warps that stored 16-byte
+// pieces from registers and held the accumulator until its rows were stored,
+// the training step took 3.93 ms against 3.73 ms now (1024 masked rows,
+// d = 4096, V = 151936: outer tiles of pass B last 4 inner tiles) and
+// 4.48 -> 4.04 ms with 1677 rows, d = 2560, V = 100003, fp32 gradients; the
+// divergence with two N = 128 products side by side in the Z accumulator
+// (60 % of the tensor rate) 21.8 against 18.6 ms (4096 rows, d_s = 4096,
+// d_t = 5120).  Every dependency
 // points to a tile of an earlier round, every CTA is resident at once (the
 // grid is one CTA per SM; the host checks that the GPU holds all its
 // clusters), and every wait is bounded (OLIVE_ERR_TIMEOUT on expiry).  A
@@ -107,11 +120,20 @@ constexpr int kSB = kBM * kBK * 2;   // B operand: this CTA's half of N (<= 128)
 constexpr int kStageBytes = kSA + kSB;
 constexpr int kXSlice = kSA;         // one 128 x 64 K-slice of an exchange tile
 constexpr int kXTile = 4 * kXSlice;  // 128 x 256 bf16 (64 KB)
-constexpr int kEpi = 128;            // epilogue threads: one accumulator row each
-constexpr int kProducerWarp = 4;
-constexpr int kMmaWarp = 5;
-constexpr int kSignalWarp = 6;       // posts the members' "tile copied" counts
-constexpr int kThreads = 224;
+constexpr int kWarpSlice = kXSlice / 4;  // an epilogue warp's 32 rows of a slice (4 KB, contiguous)
+constexpr int kEpiWarps = 8;         // two per TMEM lane quadrant, half of a tile's columns each
+constexpr int kEpi = 32 * kEpiWarps; // epilogue threads: two per accumulator row
+constexpr int kProducerWarp = kEpiWarps;
+constexpr int kMmaWarp = kEpiWarps + 1;
+constexpr int kSignalWarp = kEpiWarps + 2;  // posts the members' "tile copied" counts
+constexpr int kThreads = 32 * (kEpiWarps + 4);  // three whole warpgroups (warp 11 idles)
+// Registers a thread: 168 at launch (65536 / 384 threads); the warpgroup of
+// the producer, MMA and signal warps hands most of its share to the two of
+// the epilogue, whose 128 held accumulator values otherwise spill (the L1 left
+// beside 227 KB of shared memory is too small for 384 stacks: spilled, a
+// 32-column block took ~5500 cycles).  2 x 216 + 72 = 3 x 168.
+constexpr int kEpiRegs = 216;
+constexpr int kOtherRegs = 72;
 constexpr int kStatusTimeoutBit = 1 << OLIVE_ERR_TIMEOUT;
 constexpr float kRefMax = 64.f;
 constexpr int kMetaBytes = kZN * 8;  // pass B: lse2 and target of the tile's 256 rows
@@ -130,8 +152,8 @@ enum GMode : int { GM_REF = 0, GM_A = 1, GM_B = 2, GM_KL = 3 };
 // GM_B:          za = W {64 x 128},  zb = hc {64 x 128}, xb = hc {64 x 64}
 // xa: the ring, [slices x 128 rows] of 64 bf16, unswizzled {64 x 128} boxes
 // (a slice is stored already swizzled, so the copy is linear)
-// GM_KL:         za = hc_s {64 x 128}, zb = W_s {64 x 64}, za2 = hc_t {64 x 128},
-//                zb2 = W_t {64 x 64}, xb = W_s {64 x 64} (128-wide vocabulary tiles)
+// GM_KL:         za = hc_s {64 x 128}, zb = W_s {64 x 128}, za2 = hc_t {64 x 128},
+//                zb2 = W_t {64 x 128}, xb = W_s {64 x 64}
 struct GroupMaps {
   CUtensorMap za, zb, xb, xa, za2, zb2;
 };
@@ -157,8 +179,8 @@ struct GroupParams {
   const float* lse_in;      // [T] natural lse per packed row (GM_A lse_known, GM_B)
   float* rref;              // [Tpad] base-2 reference per compact row (GM_REF writes)
   float* rmax;              // [Tpad] base-2 row maximum (GM_A writes for redo rows)
-  float* part_s;            // [g][Tpad] per-member sums of 2^(x - R)
-  float* part_m;            // [g][Tpad] per-member maxima (base 2)
+  float* part_s;            // [2 g][Tpad] sums of 2^(x - R) per member and column half
+  float* part_m;            // [2 g][Tpad] the logits' maxima (base 2)
   float* zy;                // [Tpad] target logit z_y (natural units)
   float* pyb;               // [Tpad] P'_y as rounded to bf16 in the exchange tile
   float* logp;              // [T]
@@ -174,7 +196,6 @@ struct GroupParams {
   int32_t out_dtype;
   int64_t ring_tiles;       // exchange tiles the ring holds (debug checks)
   int32_t part_groups;      // rows of part_s / part_m (debug checks)
-  int32_t zn;               // width of an inner vocabulary tile: 256 (CE), 128 (GM_KL)
   // GM_KL (divergence gradient): per compact row the lse of both heads from the
   // value sweep, per packed row the KL and the weights g_t
   int32_t d2;               // teacher width
@@ -201,7 +222,6 @@ struct GSched {
   int nacc;   // N of the accumulation MMA (cw rounded up to 16)
   int b0;     // first column of this CTA's half of B
   int kcount; // inner extent: V (pass A) or n (pass B)
-  int zn;     // inner tile width
   int nk2;    // 64-wide K steps of a Z job's second product (GM_KL: the teacher)
   float coef;
 };
@@ -223,10 +243,9 @@ __device__ GSched make_gsched(const GroupParams& p) {
   } else {
     s.no = (p.mode == GM_A && p.redo) ? static_cast<int>(min(p.redo_list[0], static_cast<uint32_t>(rt))) : rt;
     s.ph = rt;
-    s.ni = p.mode == GM_REF ? 1 : (p.V + p.zn - 1) / p.zn;
+    s.ni = p.mode == GM_REF ? 1 : (p.V + kZN - 1) / kZN;
     s.kcount = p.V;
   }
-  s.zn = p.zn;
   s.nk = (p.d + kBK - 1) / kBK;
   s.nk2 = p.mode == GM_KL ? (p.d2 + kBK - 1) / kBK : 0;
   const int pair = blockIdx.x >> 1;
@@ -265,7 +284,7 @@ __device__ __forceinline__ int outer_of(const GroupParams& p, const GSched& s, i
   return (p.mode == GM_A && p.redo) ? static_cast<int>(p.redo_list[1 + k]) : k;
 }
 __device__ __forceinline__ int kvalid_of(const GSched& s, int k) {
-  return min(s.zn, s.kcount - k * s.zn);
+  return min(kZN, s.kcount - k * kZN);
 }
 // 64-wide K slices of inner tile k that hold valid columns
 __device__ __forceinline__ int slices_of(const GSched& s, int k) {
@@ -278,12 +297,27 @@ __device__ __forceinline__ bool member_has_job(const GSched& s, int g, int i) {
   return first < lo + s.ni;
 }
 
-// byte offset of 16-byte chunk c (0..7) of row r in K-slice sl of an exchange
-// tile: the 128-byte-swizzled K-major layout a TMA load of a 64 x 128 box
-// produces (row r at r * 128, chunk c at position c ^ (r & 7)), so a linear
-// copy of a slice to a 1024-byte-aligned stage is a valid UMMA operand
-__device__ __forceinline__ uint32_t img_off(int r, int sl, int c) {
-  return static_cast<uint32_t>(sl * kXSlice + (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4));
+// Where a round's accumulation [e_lo, e_end) pauses for the second Z product.
+// The divergence's two products share the 256-column Z accumulator one after
+// the other: half of the previous round's tiles are accumulated between them,
+// which is when the epilogue takes the student's logits into registers.  It
+// pauses no later than before a tile that opens an outer tile: that tile
+// needs the accumulator which the epilogue hands back only after it has had
+// the teacher's logits.
+template <int kMode>
+__device__ __forceinline__ int split_point(const GSched& s, int e_lo, int e_end) {
+  if (kMode != GM_KL || e_lo == e_end) return e_end;
+  const int opens = (e_lo / s.ni + 1) * s.ni;  // first tile after e_lo with k = 0
+  return min(e_lo + (e_end - e_lo + 1) / 2, opens);
+}
+
+// byte offset of row r (a multiple of 8) of K-slice sl in an exchange tile.
+// The image is the 128-byte-swizzled K-major layout a TMA load of a 64 x 128
+// box produces (row r at r * 128, its 16-byte chunk c at position c ^ (r & 7)),
+// so a linear copy of a slice to a 1024-byte-aligned stage is a valid UMMA
+// operand.
+__device__ __forceinline__ uint32_t img_off(int r, int sl) {
+  return static_cast<uint32_t>(sl * kXSlice + r * 128);
 }
 
 __device__ __forceinline__ void store_out32(void* base, size_t off, int dtype, int n_valid,
@@ -315,16 +349,18 @@ __device__ __forceinline__ void store_out32(void* base, size_t off, int dtype, i
   }
 }
 
-// 32 fp32 values -> four 16-byte chunks of row r of the exchange image
-__device__ __forceinline__ void store_img32(uint8_t* img, int r, int h, const float (&v)[32]) {
-  const int sl = h >> 1;
-  const int c0 = (h & 1) * 4;
+// 32 fp32 values (the slice's first or last 32 columns) -> four 16-byte
+// chunks of this lane's row in the warp's staging copy of a slice: 32 rows of
+// 128 bytes in the same swizzled order as the exchange image (img_off), so
+// one 4 KB bulk store moves them.  A quarter warp's 8 lanes hit 8 different
+// 16-byte columns: no bank conflicts.
+__device__ __forceinline__ void stage32(uint32_t stage, int lane, int h, const float (&v)[32]) {
+  const uint32_t row = stage + static_cast<uint32_t>((lane >> 3) * 1024 + (lane & 7) * 128);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint4 u = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                               pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
-    *reinterpret_cast<uint4*>(img + img_off(r, sl, c0 + q)) = u;
-  }
+  for (int q = 0; q < 4; ++q)
+    st_shared_v4(row + ((((h & 1) * 4 + q) ^ (lane & 7)) << 4),
+                 make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
+                            pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7])));
 }
 
 // per-row values of pass A (and GM_REF) for compact row rc
@@ -357,7 +393,8 @@ __device__ __forceinline__ RowA load_row_a(const GroupParams& p, const GSched& s
 }
 
 // All lanes of a warp: wait until the exchange tiles [e_lo, e_end) of a
-// round are written (ready[e mod R] > e / R), lane i checking tiles i, i+32,
+// round are written (every epilogue warp of their member has posted
+// ready[e mod R] e / R + 1 times), lane i checking tiles i, i+32,
 // ...  Returns the warp's common decision (false: limit ran out or abort).
 __device__ bool wait_round_ready(const uint32_t* ready, int R, int e_lo, int e_end, int lane,
                                  const WaitCtl& ctl) {
@@ -365,7 +402,7 @@ __device__ bool wait_round_ready(const uint32_t* ready, int R, int e_lo, int e_e
   while (true) {
     bool mine = true;
     for (int e = e_lo + lane; e < e_end; e += 32)
-      mine = mine && ld_acquire(ready + e % R) >= static_cast<uint32_t>(e / R + 1);
+      mine = mine && ld_acquire(ready + e % R) >= static_cast<uint32_t>(kEpiWarps * (e / R + 1));
     if (__all_sync(0xffffffffu, mine)) return true;
     bool stop = *ctl.abort != 0;
     if (!stop && global_timer_ns() - t0 > ctl.limit_ns) {
@@ -392,16 +429,17 @@ __device__ void pace_wait(const uint32_t* pace, int ngroups, int need, int lane)
   }
 }
 
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
     lmhead_group_kernel(const __grid_constant__ GroupMaps maps, const GroupParams p) {
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* gbase = smem_raw + (base - raw);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const uint32_t base = smem_u32(smem_raw);
+  uint8_t* gbase = smem_raw;
 
   // the same layout in both CTAs of a pair: the MMA reads both at these offsets
   const uint32_t stages = base;
-  const uint32_t bar0 = base + kStages * kStageBytes;
+  const uint32_t stage_out = base + kStages * kStageBytes;  // the epilogue warps' staging
+  const uint32_t bar0 = stage_out + kEpiWarps * kWarpSlice;
   auto full_bar = [&](int st) { return bar0 + 8u * st; };
   auto empty_bar = [&](int st) { return bar0 + 8u * (kStages + st); };
   const uint32_t zfull = bar0 + 8u * (2 * kStages);
@@ -409,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t ofull = zfull + 16;
   const uint32_t oempty = zfull + 24;
   const uint32_t drain = zfull + 32;
-  uint8_t* misc = gbase + kStages * kStageBytes + 8 * (2 * kStages + 5);
+  uint8_t* misc = gbase + kStages * kStageBytes + kEpiWarps * kWarpSlice + 8 * (2 * kStages + 5);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
   volatile uint32_t* copied = reinterpret_cast<volatile uint32_t*>(misc + 8);  // tiles copied
@@ -427,9 +465,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(empty_bar(st), 1);  // the even CTA's MMA commit (multicast)
     }
     mbar_init(zfull, 1);
-    mbar_init(zempty, 8);           // the four epilogue warps of both CTAs
+    mbar_init(zempty, 2 * kEpiWarps);  // the epilogue warps of both CTAs
     mbar_init(ofull, 1);
-    mbar_init(oempty, 8);
+    mbar_init(oempty, 2 * kEpiWarps);
     mbar_init(drain, 1);
     *abort_flag = 0;
     *copied = 0;
@@ -453,235 +491,287 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
 
   const uint32_t tmem_base = *tmem_slot;
-  const GSched s = *sched_smem;
+  // (read from shared memory where it is used: the epilogue needs its registers)
+  const GSched& s = *sched_smem;
   const WaitCtl ctl{abort_flag, p.wait_limit_ns};
   const int g = p.g;
-  const bool consume = p.mode != GM_REF;
+  constexpr bool consume = kMode != GM_REF;
   const int nr = (s.E + g - 1) / g;  // rounds
   const size_t ring0 = static_cast<size_t>(s.q) * p.R;
 
-  if (warp == kProducerWarp) {
-    // lane 0 issues every copy (this CTA's 128 rows of A and its half of B;
-    // completion counted on the even CTA's full barrier, whose producer
-    // announces both CTAs' bytes: the odd CTA's copies may land first, the
-    // transaction count then dips below zero within the phase, which mbarriers
-    // allow; no phase can mix with the next, since a CTA refills a stage only
-    // after the MMAs that read it have committed); the whole warp checks the
-    // `ready` flags of a round's g exchange tiles at once
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    const bool paced = consume && p.ngroups > 2;
-    // the streamed operand of a Z job (W rows in pass A, hc rows in pass B)
-    // is read again by the accumulation a round later: keep it in the L2
-    // ahead of other lines (ncu at 16384 rows: DRAM reads 196 -> 149 GB per
-    // call, time level)
-    const uint64_t keep = l2_policy_evict_last();
-    for (int r = 0; ok && r <= nr; ++r) {
-      const int j = r * g + s.m;
-      if (paced && r < nr) {
-        pace_wait(p.pace, p.ngroups, r - kPaceLag, lane);
-        if (s.m == 0 && lane == 0)
-          *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = static_cast<uint32_t>(r + 1);
-      }
-      if (r < nr && j < s.E) {
-        if (lane == 0) {
+  if (warp >= kEpiWarps) {
+    regs_dec<kOtherRegs>();
+    if (warp == kProducerWarp) {
+      // lane 0 issues every copy (this CTA's 128 rows of A and its half of B;
+      // completion counted on the even CTA's full barrier, whose producer
+      // announces both CTAs' bytes: the odd CTA's copies may land first, the
+      // transaction count then dips below zero within the phase, which mbarriers
+      // allow; no phase can mix with the next, since a CTA refills a stage only
+      // after the MMAs that read it have committed); the whole warp checks the
+      // `ready` flags of a round's g exchange tiles at once
+      const GSched s = *sched_smem;
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      const bool paced = consume && p.ngroups > 2;
+      // the streamed operand of a Z job (W rows in pass A, hc rows in pass B)
+      // is read again by the accumulation a round later: keep it in the L2
+      // ahead of other lines (ncu at 16384 rows: DRAM reads 196 -> 149 GB per
+      // call, time level)
+      const uint64_t keep = l2_policy_evict_last();
+      for (int r = 0; ok && r <= nr; ++r) {
+        const int j = r * g + s.m;
+        if (paced && r < nr) {
+          pace_wait(p.pace, p.ngroups, r - kPaceLag, lane);
+          if (s.m == 0 && lane == 0)
+            *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = static_cast<uint32_t>(r + 1);
+        }
+        const bool job = r < nr && j < s.E;
+        // a Z product: za x zb, or GM_KL's teacher za2 x zb2; the B rows are this
+        // CTA's half of the 256-wide vocabulary (or row) tile
+        auto load_z = [&](bool second) {
           const int o = outer_of(p, s, j / s.ni);
           const int k = j % s.ni;
-          // K steps [0, nk): the (first) product, za x zb; [nk, nk + nk2):
-          // GM_KL's teacher product, za2 x zb2; B rows of this CTA's half of
-          // the zn-wide vocabulary (or row) tile
-          const int half = s.zn / 2;
-          const uint32_t zbytes = 2 * (kSA + half * kBK * 2);
-          for (int ks = 0; ks < s.nk + s.nk2; ++ks) {
+          const int steps = second ? s.nk2 : s.nk;
+          for (int ks = 0; ok && ks < steps; ++ks) {
             if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
             const uint32_t sA = stages + stage * kStageBytes;
             const uint32_t fb = map_shared(full_bar(stage), 0);
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), zbytes);
-            const bool second = ks >= s.nk;
-            const int kx = (second ? ks - s.nk : ks) * kBK;
+            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kStageBytes);
             // (a skipped copy leaves its stage short: the MMA's wait then runs
             // out and the call reports OLIVE_ERR_TIMEOUT as well)
             if (OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph && k >= 0 && k < s.ni)) {
-              tma_load_2d_pair(sA, second ? &maps.za2 : &maps.za, fb, kx, o * kBM);
-              tma_load_2d_pair_hint(sA + kSA, second ? &maps.zb2 : &maps.zb, fb, kx,
-                                    k * s.zn + static_cast<int>(rank) * half, keep);
+              tma_load_2d_pair(sA, second ? &maps.za2 : &maps.za, fb, ks * kBK, o * kBM);
+              tma_load_2d_pair_hint(sA + kSA, second ? &maps.zb2 : &maps.zb, fb, ks * kBK,
+                                    k * kZN + static_cast<int>(rank) * (kZN / 2), keep);
             }
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
+        };
+        auto load_tiles = [&](int e_from, int e_to) {
+          for (int e = e_from; ok && e < e_to; ++e) {
+            const int slot = e % p.R;
+            const int k = e % s.ni;
+            const int nsl = slices_of(s, k);
+            for (int sl = 0; sl < nsl; ++sl) {
+              if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
+              const uint32_t sA = stages + stage * kStageBytes;
+              const uint32_t fb = map_shared(full_bar(stage), 0);
+              if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * (kXSlice + s.nbox * 8192));
+              // TMA x coordinates must be 16-byte aligned (8 bf16)
+              if (OLIVE_DCHECK(p.dev_status, static_cast<int64_t>(ring0 + slot) < p.ring_tiles &&
+                                                 s.b0 % 8 == 0 && s.b0 >= 0 && s.b0 < p.d + 64)) {
+                tma_load_2d_pair(sA, &maps.xa, fb, 0, static_cast<int>(((ring0 + slot) * 4 + sl) * kBM));
+                for (int b = 0; b < s.nbox; ++b)
+                  tma_load_2d_pair(sA + kSA + b * 8192, &maps.xb, fb, s.b0 + 64 * b, k * kZN + sl * kBK);
+              }
+              if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            }
+          }
+        };
+        if (job && lane == 0) load_z(false);
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok || !consume) continue;
+        const int e_lo = r > 0 ? (r - 1) * g : 0;
+        const int e_end = r > 0 ? min(r * g, s.E) : 0;
+        if (r > 0) {
+          ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
+          if (!ok) break;
+        }
+        if (lane == 0) {
+          fence_proxy_async_global();
+          const int e_mid = split_point<kMode>(s, e_lo, e_end);
+          load_tiles(e_lo, e_mid);
+          if (kMode == GM_KL && job) load_z(true);
+          load_tiles(e_mid, e_end);
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
-      if (!ok || !consume || r == 0) continue;
-      const int e_lo = (r - 1) * g;
-      const int e_end = min(r * g, s.E);
-      ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
-      if (!ok) break;
-      if (lane == 0) {
-        fence_proxy_async_global();
-        for (int e = e_lo; ok && e < e_end; ++e) {
-          const int slot = e % p.R;
-          const int k = e % s.ni;
-          const int nsl = slices_of(s, k);
-          for (int sl = 0; sl < nsl; ++sl) {
-            if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
-            const uint32_t sA = stages + stage * kStageBytes;
-            const uint32_t fb = map_shared(full_bar(stage), 0);
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * (kXSlice + s.nbox * 8192));
-            // TMA x coordinates must be 16-byte aligned (8 bf16)
-            if (OLIVE_DCHECK(p.dev_status, static_cast<int64_t>(ring0 + slot) < p.ring_tiles &&
-                                               s.b0 % 8 == 0 && s.b0 >= 0 && s.b0 < p.d + 64)) {
-              tma_load_2d_pair(sA, &maps.xa, fb, 0, static_cast<int>(((ring0 + slot) * 4 + sl) * kBM));
-              for (int b = 0; b < s.nbox; ++b)
-                tma_load_2d_pair(sA + kSA + b * 8192, &maps.xb, fb, s.b0 + 64 * b, k * s.zn + sl * kBK);
+      if (paced && s.m == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = kPaceDone;
+      if (!ok && lane == 0) {
+        // let copies already issued land before the CTA retires
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
+      }
+      __syncwarp();
+    } else if (warp == kSignalWarp) {
+      // for every exchange tile, in order, once the pair's MMA thread has seen
+      // all its slices land: one release increment of the slot's `cons` count
+      if (lane == 0 && consume) {
+        uint32_t sent = 0;
+        const uint32_t total = static_cast<uint32_t>(s.E);
+        uint64_t last = global_timer_ns();
+        while (sent < total) {
+          const uint32_t c = *copied;
+          if (c > sent) {
+            for (; sent < c; ++sent) red_release_add(p.cons + ring0 + sent % p.R, 1u);
+            last = global_timer_ns();
+            continue;
+          }
+          if (*abort_flag) break;
+          nanosleep_ns(100);
+          if (global_timer_ns() - last > p.wait_limit_ns) {
+            *abort_flag = 1;
+            break;
+          }
+        }
+      }
+      __syncwarp();
+    } else if (warp == kMmaWarp) {
+      // the even CTA's lane 0 issues the pair's MMAs (M = 256: 128 rows in each
+      // CTA's TMEM); the odd CTA's MMA warp only holds its TMEM allocation
+      if (lane == 0 && rank == 0) {
+        const GSched s = *sched_smem;
+        const uint32_t zacc = tmem_base;
+        const uint32_t oacc = tmem_base + 256;
+        const uint32_t idz = idesc_bf16(2 * kBM, kZN, false, false);
+        const uint32_t idx = idesc_bf16(2 * kBM, s.nacc, false, true);
+        const uint32_t copied_peer = map_shared(smem_u32(const_cast<uint32_t*>(copied)), 1);
+        int stage = 0;
+        uint32_t phase = 0, zph = 0, oph = 0;
+        bool ok = true;
+        for (int r = 0; ok && r <= nr; ++r) {
+          const int j = r * g + s.m;
+          const bool job = r < nr && j < s.E;
+          auto z_product = [&](int steps) {
+            if (!mbar_wait(zempty, zph ^ 1u, ctl)) { ok = false; return; }
+            tc_fence_after();
+            for (int ks = 0; ks < steps; ++ks) {
+              if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; return; }
+              tc_fence_after();
+              const uint32_t sA = stages + stage * kStageBytes;
+              const uint32_t sB = sA + kSA;
+#pragma unroll
+              for (int kk = 0; kk < kBK / 16; ++kk)
+                umma_bf16_pair(zacc, sdesc_sw128(sA + kk * 32, 16, 1024), sdesc_sw128(sB + kk * 32, 16, 1024),
+                               idz, (ks > 0 || kk > 0) ? 1u : 0u);
+              umma_commit_pair(empty_bar(stage));
+              if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
-          }
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-    }
-    if (paced && s.m == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = kPaceDone;
-    if (!ok && lane == 0) {
-      // let copies already issued land before the CTA retires
-      const uint64_t t0 = global_timer_ns();
-      while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
-    }
-    __syncwarp();
-  } else if (warp == kSignalWarp) {
-    // for every exchange tile, in order, once the pair's MMA thread has seen
-    // all its slices land: one release increment of the slot's `cons` count
-    if (lane == 0 && consume) {
-      uint32_t sent = 0;
-      const uint32_t total = static_cast<uint32_t>(s.E);
-      uint64_t last = global_timer_ns();
-      while (sent < total) {
-        const uint32_t c = *copied;
-        if (c > sent) {
-          for (; sent < c; ++sent) red_release_add(p.cons + ring0 + sent % p.R, 1u);
-          last = global_timer_ns();
-          continue;
-        }
-        if (*abort_flag) break;
-        nanosleep_ns(100);
-        if (global_timer_ns() - last > p.wait_limit_ns) {
-          *abort_flag = 1;
-          break;
-        }
-      }
-    }
-    __syncwarp();
-  } else if (warp == kMmaWarp) {
-    // the even CTA's lane 0 issues the pair's MMAs (M = 256: 128 rows in each
-    // CTA's TMEM); the odd CTA's MMA warp only holds its TMEM allocation
-    if (lane == 0 && rank == 0) {
-      const uint32_t zacc = tmem_base;
-      const uint32_t oacc = tmem_base + 256;
-      const uint32_t idz = idesc_bf16(2 * kBM, s.zn, false, false);
-      const uint32_t idx = idesc_bf16(2 * kBM, s.nacc, false, true);
-      const uint32_t copied_peer = map_shared(smem_u32(const_cast<uint32_t*>(copied)), 1);
-      int stage = 0;
-      uint32_t phase = 0, zph = 0, oph = 0;
-      bool ok = true;
-      for (int r = 0; ok && r <= nr; ++r) {
-        const int j = r * g + s.m;
-        if (r < nr && j < s.E) {
-          if (!mbar_wait(zempty, zph ^ 1u, ctl)) { ok = false; break; }
-          tc_fence_after();
-          for (int ks = 0; ks < s.nk + s.nk2; ++ks) {
-            if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t sA = stages + stage * kStageBytes;
-            const uint32_t sB = sA + kSA;
-            // GM_KL: the teacher's product goes to the next zn columns
-            const bool second = ks >= s.nk;
-            const uint32_t dz = second ? zacc + static_cast<uint32_t>(s.zn) : zacc;
-            const int kl = second ? ks - s.nk : ks;
+            umma_commit_pair(zfull);
+            zph ^= 1u;
+          };
+          auto accumulate = [&](int e_from, int e_to) {
+            for (int e = e_from; ok && e < e_to; ++e) {
+              const int k = e % s.ni;
+              if (k == 0) {
+                if (!mbar_wait(oempty, oph ^ 1u, ctl)) { ok = false; break; }
+                tc_fence_after();
+              }
+              const int nsl = slices_of(s, k);
+              for (int sl = 0; sl < nsl; ++sl) {
+                if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
+                tc_fence_after();
+                const uint32_t sA = stages + stage * kStageBytes;
+                const uint32_t sB = sA + kSA;
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk)
-              umma_bf16_pair(dz, sdesc_sw128(sA + kk * 32, 16, 1024), sdesc_sw128(sB + kk * 32, 16, 1024),
-                             idz, (kl > 0 || kk > 0) ? 1u : 0u);
-            umma_commit_pair(empty_bar(stage));
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
-          }
-          if (!ok) break;
-          umma_commit_pair(zfull);
-          zph ^= 1u;
+                for (int kk = 0; kk < kBK / 16; ++kk)
+                  umma_bf16_pair(oacc, sdesc_sw128(sA + kk * 32, 16, 1024),
+                                 sdesc_sw128(sB + kk * 2048, 8192, 1024), idx,
+                                 (k > 0 || sl > 0 || kk > 0) ? 1u : 0u);
+                umma_commit_pair(empty_bar(stage));
+                if (++stage == kStages) { stage = 0; phase ^= 1u; }
+              }
+              if (!ok) break;
+              // every slice of tile e has landed in both CTAs: their signal warps
+              // tell the two groups (a slot may be rewritten once all of its
+              // group's members have said so)
+              *copied = static_cast<uint32_t>(e + 1);
+              st_shared_cluster(copied_peer, static_cast<uint32_t>(e + 1));
+              if (k == s.ni - 1) {
+                umma_commit_pair(ofull);
+                oph ^= 1u;
+              }
+            }
+          };
+          if (job) z_product(s.nk);
+          if (!ok || !consume) continue;
+          const int e_lo = r > 0 ? (r - 1) * g : 0;
+          const int e_end = r > 0 ? min(r * g, s.E) : 0;
+          const int e_mid = split_point<kMode>(s, e_lo, e_end);
+          accumulate(e_lo, e_mid);
+          if (kMode == GM_KL && ok && job) z_product(s.nk2);
+          if (ok) accumulate(e_mid, e_end);
         }
-        if (!consume || r == 0) continue;
-        const int e_end = min(r * g, s.E);
-        for (int e = (r - 1) * g; ok && e < e_end; ++e) {
-          const int k = e % s.ni;
-          if (k == 0) {
-            if (!mbar_wait(oempty, oph ^ 1u, ctl)) { ok = false; break; }
-            tc_fence_after();
-          }
-          const int nsl = slices_of(s, k);
-          for (int sl = 0; sl < nsl; ++sl) {
-            if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
-            tc_fence_after();
-            const uint32_t sA = stages + stage * kStageBytes;
-            const uint32_t sB = sA + kSA;
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk)
-              umma_bf16_pair(oacc, sdesc_sw128(sA + kk * 32, 16, 1024),
-                             sdesc_sw128(sB + kk * 2048, 8192, 1024), idx,
-                             (k > 0 || sl > 0 || kk > 0) ? 1u : 0u);
-            umma_commit_pair(empty_bar(stage));
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
-          }
-          if (!ok) break;
-          // every slice of tile e has landed in both CTAs: their signal warps
-          // tell the two groups (a slot may be rewritten once all of its
-          // group's members have said so)
-          *copied = static_cast<uint32_t>(e + 1);
-          st_shared_cluster(copied_peer, static_cast<uint32_t>(e + 1));
-          if (k == s.ni - 1) {
-            umma_commit_pair(ofull);
-            oph ^= 1u;
-          }
-        }
+        // arrives once every MMA issued above has completed (bounded wait that
+        // ignores the abort flag: it only waits for work already in flight)
+        umma_commit_pair(drain);
+        volatile int keep_waiting = 0;
+        const uint64_t floor_ns = 200ull * 1000 * 1000;
+        const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
+        mbar_wait(drain, 0, own);
       }
-      // arrives once every MMA issued above has completed (bounded wait that
-      // ignores the abort flag: it only waits for work already in flight)
-      umma_commit_pair(drain);
-      volatile int keep_waiting = 0;
-      const uint64_t floor_ns = 200ull * 1000 * 1000;
-      const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
-      mbar_wait(drain, 0, own);
+      __syncwarp();
     }
-    __syncwarp();
   } else {
-    // epilogue warps 0..3: thread = accumulator row = TMEM lane
-    const int row = warp * 32 + lane;
-    const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+    regs_inc<kEpiRegs>();
+    // epilogue warps 0..7: the two warps of a TMEM lane quadrant share its 32
+    // accumulator rows (thread = row), `half` choosing the columns: the first
+    // or last 128 of a Z tile, the first or last 32-column blocks of the
+    // member's output chunk
+    const int half = warp >> 2;
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     uint8_t* ring_bytes = reinterpret_cast<uint8_t*>(p.ring);
     // the even CTA's MMA thread waits until both CTAs' epilogues are done with
     // an accumulator: one arrival per epilogue warp on its barriers
     const uint32_t zempty_lead = map_shared(zempty, 0);
     const uint32_t oempty_lead = map_shared(oempty, 0);
     const uint32_t zaddr = lane_addr;
-    const uint32_t oaddr = lane_addr + 256;
+    const uint32_t staging = stage_out + warp * kWarpSlice;
+    // this thread's output columns [ob, oe) of the chunk
+    const int oblocks = (s.cw + 31) / 32;
+    const int ob = half ? (oblocks + 1) / 2 * 32 : 0;
+    const int oe = half ? s.cw : min(s.cw, (oblocks + 1) / 2 * 32);
+    const uint32_t oaddr = lane_addr + 256 + ob;
     uint32_t zph = 0, oph = 0;
     bool ok = true;
     const size_t Tpad = static_cast<size_t>((p.T + kBM - 1) / kBM) * kBM;
 
-    if (p.mode == GM_B && s.ni == 0) {
-      // no masked rows: dW is zero on this member's columns of its outer tiles
-      float zero[32];
+    // The finished output accumulator: every value into registers first, then
+    // the accumulator is handed back, so that the next outer tile's MMAs run
+    // while this one is scaled, converted and stored.  (Holding it until the
+    // stores were issued left the tensor pipe idle for most of every outer
+    // tile's epilogue, which shows where outer tiles are short: pass B at few
+    // masked rows.)
+    // (acc is declared where it is used: held across the loop it would cost
+    // its 128 registers everywhere)
+    auto take_output = [&](float(&acc)[4][32]) -> bool {
+      if (!named_bar_and(1, kEpi, mbar_wait(ofull, oph, ctl))) return false;
+      oph ^= 1u;
+      tc_fence_after();
 #pragma unroll
-      for (int k = 0; k < 32; ++k) zero[k] = 0.f;
+      for (int b = 0; b < 4; ++b)  // (columns past oe are read and not stored)
+        tmem_ld_32x32b_x32(oaddr + 32 * b, reinterpret_cast<uint32_t(&)[32]>(acc[b]));
+      tmem_ld_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(oempty_lead);
+      return true;
+    };
+    // acc -> output row t (a packed row or vocabulary row), stored as is
+    auto store_output = [&](int t, const float(&acc)[4][32]) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int c = ob + 32 * b;
+        if (c < oe && OLIVE_DCHECK(p.dev_status, s.c0 + min(c + 32, oe) <= p.d))
+          store_out32(p.out, static_cast<size_t>(t) * p.d + s.c0 + c, p.out_dtype, min(32, oe - c), acc[b]);
+      }
+    };
+
+    if (kMode == GM_B && s.ni == 0) {
+      // no masked rows: dW is zero on this member's columns of its outer tiles
+      float acc[4][32] = {};
       for (int i = 0; i < s.myo; ++i) {
         const int v = outer_of(p, s, i) * kBM + row;
-        if (v >= p.V) continue;
-        for (int c = 0; c < s.cw; c += 32)
-          store_out32(p.out, static_cast<size_t>(v) * p.d + s.c0 + c, p.out_dtype, min(32, s.cw - c), zero);
+        if (v < p.V) store_output(v, acc);
       }
     }
 
     int cur_o = -1;             // pass A: the outer tile of the running partials
     RowA ra{false, -1, -1, 0.f};
-    float run_s = 0.f, run_m = -INFINITY;
+    float run_s = 0.f, run_m = -INFINITY;  // of 2^(x - R) and of x - R
+    const float s_coef = s.coef;
     for (int r = 0; ok && r <= nr; ++r) {
       const int j = r * g + s.m;
       if (r < nr && j < s.E) {
@@ -693,16 +783,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int kv = kvalid_of(s, k);
         // 32-column blocks to read: every block of the slices the members
         // copy, so columns >= kv are written as zeros, never left stale
-        const int hend = 2 * slices_of(s, k);
-        if (consume) {
-          // the slot's previous tile must have been copied by every member
-          const bool free_ok =
-              threadIdx.x == 0
-                  ? wait_counter(p.cons + ring0 + slot, static_cast<uint32_t>(g * (j / p.R)), ctl)
-                  : true;
-          if (!named_bar_and(1, kEpi, free_ok)) { ok = false; break; }
+        const int hlast = 2 * slices_of(s, k);
+        const int hbeg = half * (kZN / 64);
+        const int hend = min(hlast, hbeg + kZN / 64);
+        // the slot's previous tile must have been copied by every member
+        bool go = true;
+        if (consume && lane == 0) {
+          go = wait_counter(p.cons + ring0 + slot, static_cast<uint32_t>(g * (j / p.R)), ctl);
+          fence_proxy_async_global();
         }
-        if (p.mode == GM_B) {
+        if (kMode == GM_B) {
           // lse2 and target of the tile's 256 masked rows (+inf / -1 beyond n)
           for (int c = threadIdx.x; c < kZN; c += kEpi) {
             const int rc = k * kZN + c;
@@ -719,35 +809,94 @@ __global__ void __launch_bounds__(kThreads, 1)
             meta_y[c] = yy;
           }
         }
-        if (!named_bar_and(1, kEpi, mbar_wait(zfull, zph, ctl))) { ok = false; break; }
+        if (!named_bar_and(1, kEpi, go && mbar_wait(zfull, zph, ctl))) { ok = false; break; }
         zph ^= 1u;
         tc_fence_after();
         uint8_t* img = ring_bytes + (ring0 + slot) * static_cast<size_t>(kXTile);
         if (!OLIVE_DCHECK(p.dev_status, !consume || static_cast<int64_t>(ring0 + slot) < p.ring_tiles))
           img = nullptr;
-        if (p.mode == GM_B) {
+        // Two 32-column blocks at a time make a slice of this warp's 32 rows,
+        // staged in shared memory and moved to the ring by one bulk store
+        // (4 KB of whole lines).  `put` stages a block once the previous
+        // slice's copy has read the staging area, and starts the copy after
+        // the second block.  (Storing the 16-byte chunks straight from the
+        // registers writes half sectors of 32 different lines per
+        // instruction, and needed a device-wide fence by every thread of the
+        // epilogue per tile; the bulk stores need one by each warp's lane 0.)
+        auto put = [&](int h, const float (&v)[32]) {
+          if (!(h & 1)) {
+            if (lane == 0) bulk_wait_read();
+            __syncwarp();
+          }
+          stage32(staging, lane, h, v);
+          if (h & 1) {
+            fence_proxy_async_shared();
+            __syncwarp();
+            if (lane == 0 && img) {
+              bulk_store(img + img_off((warp & 3) * 32, h >> 1), staging, kWarpSlice);
+              bulk_commit();
+            }
+          }
+        };
+        // the accumulator goes back to the MMA thread once its last block is
+        // in registers
+        auto drained = [&](int h) {
+          if (h + 1 < hend) return;
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(zempty_lead);
+        };
+        if (kMode != GM_KL && hbeg >= hend) drained(hend);  // no valid column in this half
+        if (kMode == GM_B) {
           const int v = o * kBM + row;
+          // does any of this half's columns have its target in the outer tile?
+          bool hit = false;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            hit = hit || static_cast<uint32_t>(meta_y[half * 128 + q * 32 + lane] - o * kBM) < kBM;
+          hit = __any_sync(0xffffffffu, hit);
 #pragma unroll 1
-          for (int h = 0; h < hend; ++h) {
+          for (int h = hbeg; h < hend; ++h) {
             uint32_t a[32];
             tmem_ld_32x32b_x32(zaddr + h * 32, a);
             tmem_ld_wait();
+            drained(h);
             float gv[32];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int col = h * 32 + c;
-              const float xl = fmaf(__uint_as_float(a[c]), p.scale2, -meta_l[col]);
+            for (int c = 0; c < 32; ++c)
+              gv[c] = s_coef * fast_exp2(fmaf(__uint_as_float(a[c]), p.scale2, -meta_l[h * 32 + c]));
+            if (hit) {
               // the target entry p - 1 from expm1, exact where p is near 1
-              const float pm = meta_y[col] == v ? expm1f(xl * kLn2) : fast_exp2(xl);
-              gv[c] = col < kv ? s.coef * pm : 0.f;
+#pragma unroll 1
+              for (int c = 0; c < 32; ++c) {
+                if (meta_y[h * 32 + c] != v) continue;
+                float z = 0.f;
+#pragma unroll
+                for (int q = 0; q < 32; ++q) z = q == c ? __uint_as_float(a[q]) : z;
+                z = s_coef * expm1f(fmaf(z, p.scale2, -meta_l[h * 32 + c]) * kLn2);
+#pragma unroll
+                for (int q = 0; q < 32; ++q) gv[q] = q == c ? z : gv[q];
+              }
             }
-            if (img) store_img32(img, row, h, gv);
+            if (h * 32 + 32 > kv) {
+              // rows beyond the last one may hold anything, NaN too
+#pragma unroll
+              for (int c = 0; c < 32; ++c) gv[c] = h * 32 + c < kv ? gv[c] : 0.f;
+            }
+            put(h, gv);
           }
-        } else if (p.mode == GM_KL) {
-          // G of the divergence for this 128 x 128 tile from both heads'
-          // fp32 logits (zn columns each) and the row's lse of each head and
-          // KL from the value sweep: reverse g inv_tau p_s (log p_s - log p_t
-          // - KL), forward g inv_tau (p_s - p_t)
+        } else if (kMode == GM_KL) {
+          // G of the divergence for this 128 x 256 tile from both heads' fp32
+          // logits and the row's lse of each head and KL from the value sweep:
+          // reverse g inv_tau p_s (log p_s - log p_t - KL), forward
+          // g inv_tau (p_s - p_t).  The student's logits arrive first and wait
+          // in registers for the teacher's.
+          float zs_all[4][32];
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            tmem_ld_32x32b_x32(zaddr + (hbeg + b) * 32, reinterpret_cast<uint32_t(&)[32]>(zs_all[b]));
+          tmem_ld_wait();
+          drained(hend - 1);
           const int rc = o * kBM + row;
           bool valid = false;
           float ls0 = 0.f, lt0 = 0.f, klv = 0.f, cf = 0.f;
@@ -761,26 +910,38 @@ __global__ void __launch_bounds__(kThreads, 1)
               cf = p.grad_kl[t] * p.inv_tau;
             }
           }
-#pragma unroll 1
-          for (int h = 0; h < hend; ++h) {
-            uint32_t a[32], b[32];
-            tmem_ld_32x32b_x32(zaddr + h * 32, a);
-            tmem_ld_32x32b_x32(zaddr + static_cast<uint32_t>(s.zn) + h * 32, b);
-            tmem_ld_wait();
-            float gv[32];
-            // log p_s - log p_t as (z_s - z_t) - (lse_s - lse_t): a teacher
-            // shifted by a constant per row cancels before the large terms meet
-            const float dl = ls0 - lt0;
+          if (!named_bar_and(1, kEpi, mbar_wait(zfull, zph, ctl))) { ok = false; break; }
+          zph ^= 1u;
+          tc_fence_after();
+          if (hbeg >= hend) drained(hend);
+          // log p_s - log p_t as (z_s - z_t) - (lse_s - lse_t): a teacher
+          // shifted by a constant per row cancels before the large terms meet
+          const float dl = ls0 - lt0;
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const float zs = __uint_as_float(a[c]) * p.inv_tau;
-              const float zt = __uint_as_float(b[c]) * p.inv_tau;
-              const float ps = fast_exp2((zs - ls0) * kLog2e);
-              const float gg = p.reverse ? cf * ps * (((zs - zt) - dl) - klv)
-                                         : cf * (ps - fast_exp2((zt - lt0) * kLog2e));
-              gv[c] = (valid && h * 32 + c < kv) ? gg : 0.f;
+          for (int b = 0; b < 4; ++b) {
+            const int h = hbeg + b;
+            if (h >= hend) break;
+            float(&gv)[32] = zs_all[b];
+#pragma unroll
+            for (int u = 0; u < 32; u += 16) {
+              uint32_t zt_b[16];
+              tmem_ld_32x32b_x16(zaddr + h * 32 + u, zt_b);
+              tmem_ld_wait();
+              if (u) drained(h);
+#pragma unroll
+              for (int c = 0; c < 16; ++c) {
+                const float zs = gv[u + c] * p.inv_tau;
+                const float zt = __uint_as_float(zt_b[c]) * p.inv_tau;
+                const float ps = fast_exp2((zs - ls0) * kLog2e);
+                gv[u + c] = cf * (p.reverse ? ps * (((zs - zt) - dl) - klv)
+                                            : ps - fast_exp2((zt - lt0) * kLog2e));
+              }
             }
-            if (img) store_img32(img, row, h, gv);
+            if (!valid || h * 32 + 32 > kv) {
+#pragma unroll
+              for (int c = 0; c < 32; ++c) gv[c] = valid && h * 32 + c < kv ? gv[c] : 0.f;
+            }
+            put(h, gv);
           }
         } else {
           if (o != cur_o) {
@@ -789,25 +950,42 @@ __global__ void __launch_bounds__(kThreads, 1)
             run_s = 0.f;
             run_m = -INFINITY;
           }
-          const int v0 = k * s.zn;
+          const int v0 = k * kZN;
 #pragma unroll 1
-          for (int h = 0; h < hend; ++h) {
+          for (int h = hbeg; h < hend; ++h) {
             uint32_t a[32];
             tmem_ld_32x32b_x32(zaddr + h * 32, a);
             tmem_ld_wait();
+            drained(h);
             float pv[32];
+            // two running sums and maxima of x - R: shorter chains
+            float s1 = 0.f, m1 = -INFINITY;
+            if (h * 32 + 32 <= kv) {
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int col = h * 32 + c;
-              const float x = __uint_as_float(a[c]) * p.scale2;
-              const bool in = col < kv;
-              run_m = in ? fmaxf(run_m, x) : run_m;
-              const float e = fast_exp2(x - ra.R);
-              pv[c] = in ? e : 0.f;
-              run_s += pv[c];
+              for (int c = 0; c < 32; c += 2) {
+                const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
+                const float x1 = fmaf(__uint_as_float(a[c + 1]), p.scale2, -ra.R);
+                run_m = fmaxf(run_m, x0);
+                m1 = fmaxf(m1, x1);
+                pv[c] = fast_exp2(x0);
+                pv[c + 1] = fast_exp2(x1);
+                run_s += pv[c];
+                s1 += pv[c + 1];
+              }
+            } else {
+#pragma unroll
+              for (int c = 0; c < 32; ++c) {
+                const bool in = h * 32 + c < kv;
+                const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
+                m1 = in ? fmaxf(m1, x0) : m1;
+                pv[c] = in ? fast_exp2(x0) : 0.f;
+                s1 += pv[c];
+              }
             }
+            run_s += s1;
+            run_m = fmaxf(run_m, m1);
             const int yo = ra.y - (v0 + h * 32);
-            if (p.mode == GM_A && yo >= 0 && yo < 32) {
+            if (kMode == GM_A && yo >= 0 && yo < 32) {
               // the target's exact logit and the bf16 value of P'_y the MMA
               // sees: the epilogue replaces that term by p_y - 1 from the
               // logit, so rows with p_y near 1 keep their accuracy
@@ -818,25 +996,30 @@ __global__ void __launch_bounds__(kThreads, 1)
                   p.pyb[o * kBM + row] = __bfloat162float(__float2bfloat16_rn(pv[c]));
                 }
             }
-            if (p.mode == GM_A && img) store_img32(img, row, h, pv);
+            if (kMode == GM_A) put(h, pv);
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(zempty_lead);
-        if (p.mode == GM_REF) {
-          if (o * kBM + row < s.n) p.rref[o * kBM + row] = run_m;
-        } else {
-          if (p.mode == GM_A && ra.valid &&
-              OLIVE_DCHECK(p.dev_status, s.m < p.part_groups && o * kBM + row < static_cast<int>(Tpad))) {
-            p.part_s[static_cast<size_t>(s.m) * Tpad + o * kBM + row] = run_s;
-            p.part_m[static_cast<size_t>(s.m) * Tpad + o * kBM + row] = run_m;
-          }
-          // publish the tile: every thread's stores, then one release
-          fence_proxy_async_global();
-          __threadfence();
+        if (kMode == GM_REF) {
+          // the row's two column halves meet in shared memory
+          if (half) meta_l[row] = run_m;
           named_bar_sync(1, kEpi);
-          if (threadIdx.x == 0) red_release_add(p.ready + ring0 + slot, 1u);
+          if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
+          named_bar_sync(1, kEpi);
+        } else {
+          if (kMode == GM_A && ra.valid &&
+              OLIVE_DCHECK(p.dev_status, 2 * s.m + half < p.part_groups && o * kBM + row < static_cast<int>(Tpad))) {
+            p.part_s[static_cast<size_t>(2 * s.m + half) * Tpad + o * kBM + row] = run_s;
+            p.part_m[static_cast<size_t>(2 * s.m + half) * Tpad + o * kBM + row] = run_m + ra.R;
+          }
+          // publish the warp's part of the tile once its copies are complete
+          if (lane == 0) {
+            bulk_wait();
+            fence_proxy_async_global();
+            red_release_add(p.ready + ring0 + slot, 1u);
+          }
+          __syncwarp();
+          // the row metadata of this tile is read: the next one's may be written
+          if (kMode == GM_B) named_bar_sync(1, kEpi);
         }
       }
       if (!consume || r == 0) continue;
@@ -846,50 +1029,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (e % s.ni != s.ni - 1) continue;
         const int i = e / s.ni;
         const int o = outer_of(p, s, i);
-        if (p.mode == GM_B) {
-          if (!named_bar_and(1, kEpi, mbar_wait(ofull, oph, ctl))) { ok = false; break; }
-          oph ^= 1u;
-          tc_fence_after();
+        float acc[4][32];
+        if (kMode == GM_B) {
+          if (!take_output(acc)) { ok = false; break; }
           const int v = o * kBM + row;
-#pragma unroll 1
-          for (int c = 0; c < s.cw; c += 32) {
-            uint32_t a[32];
-            tmem_ld_32x32b_x32(oaddr + c, a);
-            tmem_ld_wait();
-            float ov[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) ov[q] = __uint_as_float(a[q]);
-            if (v < p.V && OLIVE_DCHECK(p.dev_status, v >= 0 && s.c0 + c + min(32, s.cw - c) <= p.d))
-              store_out32(p.out, static_cast<size_t>(v) * p.d + s.c0 + c, p.out_dtype,
-                          min(32, s.cw - c), ov);
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(oempty_lead);
+          if (v < p.V && OLIVE_DCHECK(p.dev_status, v >= 0)) store_output(v, acc);
           continue;
         }
-        if (p.mode == GM_KL) {
+        if (kMode == GM_KL) {
           // the divergence gradient: G carried g inv_tau, so d_h_s is the sum
-          if (!named_bar_and(1, kEpi, mbar_wait(ofull, oph, ctl))) { ok = false; break; }
-          oph ^= 1u;
-          tc_fence_after();
+          if (!take_output(acc)) { ok = false; break; }
           const int rc = o * kBM + row;
           const int t = rc < s.n ? p.rows[rc] : -1;
-#pragma unroll 1
-          for (int c = 0; c < s.cw; c += 32) {
-            uint32_t a[32];
-            tmem_ld_32x32b_x32(oaddr + c, a);
-            tmem_ld_wait();
-            float ov[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) ov[q] = __uint_as_float(a[q]);
-            const int nv = min(32, s.cw - c);
-            if (t >= 0 && t < p.T && OLIVE_DCHECK(p.dev_status, s.c0 + c + nv <= p.d))
-              store_out32(p.out, static_cast<size_t>(t) * p.d + s.c0 + c, p.out_dtype, nv, ov);
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(oempty_lead);
+          if (t >= 0 && t < p.T) store_output(t, acc);
           continue;
         }
         // pass A: merge the members' partials, then dH
@@ -898,24 +1050,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         // every member's partials (and the target's z_y, P'_y from the
         // member that met it) are published before any member reads them
         if (rw.valid && !member_has_job(s, g, i)) {
-          p.part_s[static_cast<size_t>(s.m) * Tpad + rc] = 0.f;
-          p.part_m[static_cast<size_t>(s.m) * Tpad + rc] = -INFINITY;
+          p.part_s[static_cast<size_t>(2 * s.m + half) * Tpad + rc] = 0.f;
+          p.part_m[static_cast<size_t>(2 * s.m + half) * Tpad + rc] = -INFINITY;
         }
-        if (!phantom(p, s, i) && OLIVE_DCHECK(p.dev_status, o >= 0 && o * kBM < static_cast<int>(Tpad))) {
+        const bool whole = !phantom(p, s, i) && OLIVE_DCHECK(p.dev_status, o >= 0 && o * kBM < static_cast<int>(Tpad));
+        if (whole) {
           __threadfence();
           named_bar_sync(1, kEpi);
           if (threadIdx.x == 0) red_release_add(p.outer_ctr + o, 1u);
+        }
+        if (!take_output(acc)) { ok = false; break; }
+        if (whole) {
           const bool seen =
               threadIdx.x == 0 ? wait_counter(p.outer_ctr + o, static_cast<uint32_t>(g), ctl) : true;
           if (!named_bar_and(1, kEpi, seen)) { ok = false; break; }
         }
-        if (!named_bar_and(1, kEpi, mbar_wait(ofull, oph, ctl))) { ok = false; break; }
-        oph ^= 1u;
-        tc_fence_after();
         float lse2 = rw.R, mx = -INFINITY;
         if (!p.lse_known && rw.valid) {
           float sum = 0.f;
-          for (int mm = 0; mm < g; ++mm) {
+          for (int mm = 0; mm < 2 * g; ++mm) {
             sum += __ldcg(p.part_s + static_cast<size_t>(mm) * Tpad + rc);
             mx = fmaxf(mx, __ldcg(p.part_m + static_cast<size_t>(mm) * Tpad + rc));
           }
@@ -929,7 +1082,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           // the reference was too low for some row: the redo launch
           // recomputes this row tile with R = the rows' maxima
           if (s.m == 0) {
-            if (rw.valid) p.rmax[rc] = mx;
+            if (rw.valid && !half) p.rmax[rc] = mx;
             if (threadIdx.x == 0) {
               const uint32_t at = atomicAdd(p.redo_list, 1u);
               p.redo_list[1 + at] = static_cast<uint32_t>(o);
@@ -937,7 +1090,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         } else {
           const bool has_y = rw.valid && rw.y >= 0 && rw.y < p.V;
-          if (s.m == 0 && rw.valid) {
+          if (s.m == 0 && rw.valid && !half) {
             if (!has_y) atomicOr(p.dev_status, 1 << OLIVE_ERR_TOKEN_RANGE);
             if (p.write_fwd) {
               const float l = lse2 * kLn2;
@@ -958,13 +1111,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           const uint4* wy =
               has_y ? reinterpret_cast<const uint4*>(p.W + static_cast<size_t>(rw.y) * p.d + s.c0) : nullptr;
-#pragma unroll 1
-          for (int c = 0; c < s.cw; c += 32) {
-            uint32_t a[32];
-            tmem_ld_32x32b_x32(oaddr + c, a);
-            tmem_ld_wait();
-            float dv[32];
-            const int nv = min(32, s.cw - c);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const int c = ob + 32 * b;
+            if (c >= oe) continue;
+            const int nv = min(32, oe - c);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               uint4 w4 = make_uint4(0, 0, 0, 0);
@@ -973,18 +1124,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
               for (int u = 0; u < 4; ++u) {
                 const float2 wf = __bfloat1622float2(w2[u]);
-                dv[8 * q + 2 * u] = s.coef * fmaf(scale, __uint_as_float(a[8 * q + 2 * u]), corr * wf.x);
-                dv[8 * q + 2 * u + 1] =
-                    s.coef * fmaf(scale, __uint_as_float(a[8 * q + 2 * u + 1]), corr * wf.y);
+                float& a0 = acc[b][8 * q + 2 * u];
+                float& a1 = acc[b][8 * q + 2 * u + 1];
+                a0 = s.coef * fmaf(scale, a0, corr * wf.x);
+                a1 = s.coef * fmaf(scale, a1, corr * wf.y);
               }
             }
-            if (rw.valid && OLIVE_DCHECK(p.dev_status, rw.t >= 0 && rw.t < p.T && s.c0 + c + nv <= p.d))
-              store_out32(p.out, static_cast<size_t>(rw.t) * p.d + s.c0 + c, p.out_dtype, nv, dv);
           }
+          if (rw.valid && OLIVE_DCHECK(p.dev_status, rw.t >= 0 && rw.t < p.T)) store_output(rw.t, acc);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(oempty_lead);
       }
     }
   }
@@ -1000,7 +1148,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-constexpr int kGroupSmem = 1024 + kStages * kStageBytes + 8 * (2 * kStages + 5) + 128 + kMetaBytes;
+constexpr int kGroupSmem =
+    kStages * kStageBytes + kEpiWarps * kWarpSlice + 8 * (2 * kStages + 5) + 128 + kMetaBytes;
 static_assert(kGroupSmem <= 227 * 1024, "shared memory budget");
 
 int ring_slots_for(int g) { return 3 * g > 4 ? 3 * g : 4; }
@@ -1033,6 +1182,54 @@ GroupShape group_shape(int cols, int sms) {
   gs.ngroups = 2 * (sms / (2 * gs.g));
   gs.R = ring_slots_for(gs.g);
   return gs;
+}
+
+// Launches one mode of the kernel on `ctas` CTAs.
+template <int kMode>
+olive_status launch_mode(const Ctx& c, int sms, int ctas, const GroupMaps& maps, const GroupParams& p) {
+  static std::atomic<int> done[kMaxDevices];
+  if (!set_smem_once(reinterpret_cast<const void*>(lmhead_group_kernel<kMode>), kGroupSmem, c.device, done))
+    return OLIVE_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kGroupSmem;
+  cfg.stream = c.stream;
+  // clusters of two CTAs (the MMA pairs).  Members of a group wait on one
+  // another, so every CTA must be resident at once: the grid is at most one
+  // CTA per SM, and the first launch on each device checks that the GPU holds
+  // all of its clusters together (cudaOccupancyMaxActiveClusters), else the
+  // call is refused.  The launch is not marked cooperative: profilers (ncu)
+  // cannot launch cooperative grids of clusters, and a grid that fits starts
+  // whole on an idle GPU; if another stream's kernel holds SMs, the waits are
+  // bounded and report OLIVE_ERR_TIMEOUT.
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  static std::atomic<int> fits[kMaxDevices];  // clusters the device holds at once, + 1
+  const bool cached = c.device >= 0 && c.device < kMaxDevices;
+  int held = cached ? fits[c.device].load(std::memory_order_acquire) - 1 : -1;
+  if (held < 0) {
+    cudaLaunchConfig_t q = cfg;
+    q.gridDim = dim3(2 * (sms / 2));
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, lmhead_group_kernel<kMode>, &q) != cudaSuccess) {
+      cudaGetLastError();
+      return OLIVE_ERR_CUDA;
+    }
+    held = n;
+    if (cached) fits[c.device].store(n + 1, std::memory_order_release);
+  }
+  if (static_cast<int>(cfg.gridDim.x) > 2 * held) return OLIVE_ERR_UNSUPPORTED_DEVICE;
+  if (cudaLaunchKernelEx(&cfg, lmhead_group_kernel<kMode>, maps, p) != cudaSuccess) {
+    cudaGetLastError();
+    return OLIVE_ERR_CUDA;
+  }
+  return OLIVE_OK;
 }
 
 // output columns one sweep covers: the widest whose fewest members still
@@ -1097,18 +1294,16 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   const uint64_t zbRows = rowsA ? V : Tpad;
   // the ring viewed as rows of 64 bf16 (one 128-byte row of a slice image)
   const uint64_t ring_rows = group_ring_bytes(T, d, V) / 128;
-  // inner tiles of 256 vocabulary entries (rows in pass B), 128 for the
-  // divergence, whose Z jobs hold both heads' logits in the Z accumulator;
-  // each CTA of a pair loads half of them as its B rows
-  const int zn = mode == GM_KL ? 128 : kZN;
+  // inner tiles of 256 vocabulary entries (rows in pass B); each CTA of a pair
+  // loads half of them as its B rows
   if (!encode_bf16_2d(&maps.za, zaBase, d, zaRows, 2ull * d, 64, 128) ||
-      !encode_bf16_2d(&maps.zb, zbBase, d, zbRows, 2ull * d, 64, zn / 2) ||
+      !encode_bf16_2d(&maps.zb, zbBase, d, zbRows, 2ull * d, 64, kZN / 2) ||
       !encode_bf16_2d(&maps.xb, zbBase, d, zbRows, 2ull * d, 64, 64) ||
       !encode_bf16_2d_plain(&maps.xa, a.ring, 64, ring_rows, 128, 64, 128))
     return OLIVE_ERR_CUDA;
   if (mode == GM_KL) {
     if (!encode_bf16_2d(&maps.za2, a.hc2, a.d2, Tpad, 2ull * a.d2, 64, 128) ||
-        !encode_bf16_2d(&maps.zb2, a.W2, a.d2, V, 2ull * a.d2, 64, zn / 2))
+        !encode_bf16_2d(&maps.zb2, a.W2, a.d2, V, 2ull * a.d2, 64, kZN / 2))
       return OLIVE_ERR_CUDA;
   } else {
     maps.za2 = maps.za;
@@ -1158,8 +1353,7 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   p.out = mode == GM_B ? a.d_W : a.d_hidden;  // GM_KL: d_h_s
   p.out_dtype = a.out_dtype;
   p.ring_tiles = static_cast<int64_t>(group_ring_words(T, d, V));
-  p.part_groups = group_g_max(d);
-  p.zn = zn;
+  p.part_groups = 2 * group_g_max(d);
   p.d2 = a.d2;
   p.reverse = a.reverse;
   p.lse_sc = a.lse_sc;
@@ -1167,49 +1361,13 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   p.kl = a.kl;
   p.grad_kl = a.grad_kl;
 
-  static std::atomic<int> done[kMaxDevices];
-  if (!set_smem_once(reinterpret_cast<const void*>(lmhead_group_kernel), kGroupSmem, c.device, done))
-    return OLIVE_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(gs.ngroups * gs.g);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kGroupSmem;
-  cfg.stream = c.stream;
-  // clusters of two CTAs (the MMA pairs).  Members of a group wait on one
-  // another, so every CTA must be resident at once: the grid is at most one
-  // CTA per SM, and the first launch on each device checks that the GPU holds
-  // all of its clusters together (cudaOccupancyMaxActiveClusters), else the
-  // call is refused.  The launch is not marked cooperative: profilers (ncu)
-  // cannot launch cooperative grids of clusters, and a grid that fits starts
-  // whole on an idle GPU; if another stream's kernel holds SMs, the waits are
-  // bounded and report OLIVE_ERR_TIMEOUT.
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  static std::atomic<int> fits[kMaxDevices];  // clusters the device holds at once, + 1
-  const bool cached = c.device >= 0 && c.device < kMaxDevices;
-  int held = cached ? fits[c.device].load(std::memory_order_acquire) - 1 : -1;
-  if (held < 0) {
-    cudaLaunchConfig_t q = cfg;
-    q.gridDim = dim3(2 * (sms / 2));
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, lmhead_group_kernel, &q) != cudaSuccess) {
-      cudaGetLastError();
-      return OLIVE_ERR_CUDA;
-    }
-    held = n;
-    if (cached) fits[c.device].store(n + 1, std::memory_order_release);
+  const int ctas = gs.ngroups * gs.g;
+  switch (mode) {
+    case GM_REF: return launch_mode<GM_REF>(c, sms, ctas, maps, p);
+    case GM_A: return launch_mode<GM_A>(c, sms, ctas, maps, p);
+    case GM_B: return launch_mode<GM_B>(c, sms, ctas, maps, p);
+    default: return launch_mode<GM_KL>(c, sms, ctas, maps, p);
   }
-  if (static_cast<int>(cfg.gridDim.x) > 2 * held) return OLIVE_ERR_UNSUPPORTED_DEVICE;
-  if (cudaLaunchKernelEx(&cfg, lmhead_group_kernel, maps, p) != cudaSuccess) {
-    cudaGetLastError();
-    return OLIVE_ERR_CUDA;
-  }
-  return OLIVE_OK;
 }
 
 }  // namespace olive

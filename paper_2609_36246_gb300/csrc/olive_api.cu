@@ -271,8 +271,8 @@ static GroupWs carve_group_impl(void* ws, int64_t T, int64_t d, int64_t V, size_
   w.zy = static_cast<float*>(c.take(4ull * Tpad));
   w.pyb = static_cast<float*>(c.take(4ull * Tpad));
   w.nll = static_cast<float*>(c.take(4ull * Tpad));
-  w.part_s = static_cast<float*>(c.take(4ull * gmax * Tpad));
-  w.part_m = static_cast<float*>(c.take(4ull * gmax * Tpad));
+  w.part_s = static_cast<float*>(c.take(8ull * gmax * Tpad));
+  w.part_m = static_cast<float*>(c.take(8ull * gmax * Tpad));
   w.ring = c.take(group_ring_bytes(T, d, V));
   // counters in one region, zeroed by one memset per column sweep: group
   // barriers [2 rt] (first and redo launch), the redo list [1 + rt], then the

@@ -260,3 +260,16 @@ def test_wide_heads(direction):
                                         direction, grad_kl=gk.astype(np.float64))
     assert_close_logp(kl, rkl, "kl")
     assert_close_grad(dhs, rdhs, "dH_s")
+
+
+@pytest.mark.parametrize("T,ds,dt,V", [(2600, 4096, 72, 300), (5200, 2048, 200, 130), (6000, 520, 64, 700)])
+def test_outer_tiles_shorter_than_a_round(T, ds, dt, V):
+    """Row tiles of one to three inner tiles, several to a group's round: the
+    output accumulator changes hands between a round's two products."""
+    hs, Ws, ht, Wt, rows, gk = _case(T, T, ds, dt, V, std=0.02)
+    for direction in ("reverse", "forward"):
+        kl, dhs = _gpu(hs, Ws, ht, Wt, rows, gk, direction)
+        rkl, rdhs = oracle.token_divergence(to_f64(hs), to_f64(Ws), to_f64(ht), to_f64(Wt), rows, 1.0,
+                                            direction, grad_kl=gk.astype(np.float64))
+        assert_close_logp(kl, rkl, "kl")
+        assert_close_grad(dhs, rdhs, "dH_s")
