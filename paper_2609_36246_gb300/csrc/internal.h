@@ -122,6 +122,7 @@ struct KlWs {
   float* lse_p;   // [Tpad]
   float* lse_q;   // [Tpad]
   void* ring;     // group_ring_bytes(T, d_s, V)
+  float* tail_acc;  // group_tail_bytes(T, d_s, V)
   uint32_t* ctr;  // ctr_words words
   size_t ctr_words;
 };
@@ -141,6 +142,9 @@ struct GroupWs {
   float* part_s;     // [2 g_max, Tpad] partial sums per member and column half
   float* part_m;     // [2 g_max, Tpad] partial maxima
   void* ring;        // group_ring_bytes(T, d, V)
+  float* tail_acc;   // group_tail_bytes(T, d, V): partial accumulators of split row pairs
+  float* tail_s;     // group_tail_sums(T, d, V): their row sums
+  float* tail_m;     // and maxima
   uint32_t* outer;   // [2 rt] pass-A group barriers (first launch, redo launch)
   uint32_t* redo;    // [1 + rt] redo list
   uint32_t* ring_ctr;  // 3 launches x group_ctr_words(T, d, V)
@@ -153,6 +157,8 @@ int group_count_max(int64_t T, int64_t d, int64_t V);
 size_t group_ring_words(int64_t T, int64_t d, int64_t V);
 size_t group_ring_bytes(int64_t T, int64_t d, int64_t V);
 size_t group_ctr_words(int64_t T, int64_t d, int64_t V);
+size_t group_tail_bytes(int64_t T, int64_t d, int64_t V);
+size_t group_tail_sums(int64_t T, int64_t d, int64_t V);
 int group_sweep_cols(int sms);
 
 struct GroupArgs {
@@ -169,6 +175,7 @@ struct GroupArgs {
   uint32_t* redo_list;
   uint32_t* outer_ctr;
   void* ring;
+  float *tail_acc, *tail_s, *tail_m;
   void* d_hidden;
   void* d_W;
   int out_dtype;
@@ -190,8 +197,8 @@ olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct
                                   const int32_t* n_rows, int32_t T, int32_t V, float inv_tau,
                                   int reverse, const float* kl, const float* lse_s,
                                   const float* lse_t, const float* grad_kl, void* d_h_s,
-                                  int grad_dtype, void* ring, uint32_t* ctr, size_t ctr_words,
-                                  int32_t* dev_status);
+                                  int grad_dtype, void* ring, float* tail_acc, uint32_t* ctr,
+                                  size_t ctr_words, int32_t* dev_status);
 // The whole step: forward + backward when lse_given is null (logp, lse, loss
 // written), else the backward of that forward.
 olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,

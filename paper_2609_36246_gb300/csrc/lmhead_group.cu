@@ -120,6 +120,7 @@ constexpr int kSB = kBM * kBK * 2;   // B operand: this CTA's half of N (<= 128)
 constexpr int kStageBytes = kSA + kSB;
 constexpr int kXSlice = kSA;         // one 128 x 64 K-slice of an exchange tile
 constexpr int kXTile = 4 * kXSlice;  // 128 x 256 bf16 (64 KB)
+constexpr int kTailVecs = 32 * 256;  // float4 of a 128 x 256 fp32 accumulator
 constexpr int kWarpSlice = kXSlice / 4;  // an epilogue warp's 32 rows of a slice (4 KB, contiguous)
 constexpr int kEpiWarps = 8;         // two per TMEM lane quadrant, half of a tile's columns each
 constexpr int kEpi = 32 * kEpiWarps; // epilogue threads: two per accumulator row
@@ -192,6 +193,14 @@ struct GroupParams {
   uint32_t* ready;          // [ngroups][R]
   uint32_t* cons;           // [ngroups][R]
   uint32_t* pace;           // [ngroups] rounds each group has begun (a pacing hint)
+  // split row pairs (see GSched): partial accumulators [slot][2][g] of
+  // kTailVecs float4 (in the order of the epilogue's threads), GM_A's partial
+  // sums and maxima [slot][2 g][2 x 128], and how many runs have left their
+  // partial per row tile and member
+  float* tail_acc;
+  float *tail_s, *tail_m;
+  uint32_t* tail_ctr;
+  int32_t tail_parts, tail_slots;  // (debug checks)
   void* out;                // GM_A: d_hidden [T, d]; GM_B: d_W [V, d]
   int32_t out_dtype;
   int64_t ring_tiles;       // exchange tiles the ring holds (debug checks)
@@ -206,7 +215,27 @@ struct GroupParams {
   const float* grad_kl;     // [T]
 };
 
-// per-CTA schedule, the same in every CTA of a group
+// Per-CTA schedule, the same in every CTA of a group.
+//
+// Outer tiles go in pairs (a row pair: tile 2 rp for the even CTAs, 2 rp + 1
+// for the odd ones).  Pair-group pg takes the row pairs pg, pg + npg, ... as
+// far as every pair-group gets one; the last r = nrp mod npg pairs are the
+// tail.  Left whole, they keep r pair-groups busy for ni inner tiles while the
+// others idle, which is all of pass A at up to 256 rows.  So the tail's r * ni
+// inner tiles are laid end to end and cut into nt runs of equal length, one a
+// pair-group; a run covers the end of one row pair, the start of the next, or
+// a part of one.  Each run leaves its partial fp32 accumulator (and pass A's
+// row sums) in the workspace, in slot c + t for run c and row pair t of the
+// tail (c + t grows along the line, so slots are distinct and fewer than
+// 2 npg), and the last member to arrive for its columns adds the partials up
+// in run order, the same order every time.
+// A run costs its length and every partial of a row pair about 1.2 us to add,
+// a quarter of an inner tile's time at the least, so runs are at least
+// sqrt(ni / 4) long and the tail stays whole where that cost is not below ni.
+// Pass A, whole -> split: 365 rows, d = 2048, V = 151936 (2 row pairs for 8
+// pair-groups) 1580 -> 545 us; 1677 rows, d = 2560, V = 100003 (7 for 6)
+// 1910 -> 1275 us; 300 rows, d = 256, V = 4096 (2 row pairs of 16 tiles)
+// 126 -> 30 us.
 struct GSched {
   int n;      // masked rows
   int rank;   // 0: the pair's even CTA (issues the MMAs), 1: its peer
@@ -215,7 +244,12 @@ struct GSched {
   int ni;     // inner tiles per outer tile
   int nk;     // 64-wide K steps of a Z job
   int q, m;   // group, member
-  int myo;    // outer tiles of this group
+  int pg, npg;  // pair-group, pair-groups
+  int rp0;    // first row pair of the tail
+  int tail0;  // the group's first exchange tile in the tail
+  int x0;     // its place on the tail's line of inner tiles
+  int nt;     // runs the tail is cut into (0: left whole)
+  int xs;     // inner tiles in the tail
   int E;      // exchange tiles of this group
   int c0, cw; // output columns of this member
   int nbox;   // 64-column boxes of this CTA's half of the accumulation's B
@@ -225,6 +259,15 @@ struct GSched {
   int nk2;    // 64-wide K steps of a Z job's second product (GM_KL: the teacher)
   float coef;
 };
+
+// start of run c of the tail's line
+__device__ __forceinline__ int run_start(const GSched& s, int c) {
+  return static_cast<int>(static_cast<int64_t>(s.xs) * c / s.nt);
+}
+// the run that holds place x
+__device__ __forceinline__ int run_of(const GSched& s, int x) {
+  return static_cast<int>((static_cast<int64_t>(x + 1) * s.nt - 1) / s.xs);
+}
 
 // CTAs come in pairs (clusters of 2): pair-group pg of g pairs runs groups
 // 2 pg (even CTAs) and 2 pg + 1 (odd CTAs) in lockstep, pair m being member m
@@ -252,12 +295,33 @@ __device__ GSched make_gsched(const GroupParams& p) {
   s.m = pair % p.g;
   const int pg = pair / p.g;
   s.q = 2 * pg + s.rank;
-  // both groups of a pair-group run as many outer tiles as the even one
-  // (which has at least as many); the odd one's extra tile, if any, is a
-  // phantom whose rows are invalid
-  const int qe = 2 * pg;
-  s.myo = qe < s.no ? (s.no - qe + p.ngroups - 1) / p.ngroups : 0;
-  s.E = s.myo * s.ni;
+  // when the number of outer tiles is odd, the odd CTAs' half of the last row
+  // pair is a phantom whose rows are invalid
+  s.pg = pg;
+  s.npg = p.ngroups / 2;
+  const int nrp = (s.no + 1) / 2;
+  const int nfull = nrp / s.npg;
+  const int r = nrp - nfull * s.npg;
+  s.rp0 = nfull * s.npg;
+  s.tail0 = nfull * s.ni;
+  s.xs = r * s.ni;
+  s.nt = 0;
+  if (p.tail_acc && r > 0) {
+    int least = 2;
+    while (4 * least * least < s.ni) ++least;
+    const int nt = min(s.npg, s.xs / least);
+    if (nt > r) {
+      const int len = (s.xs + nt - 1) / nt;
+      if (len + (s.ni + len - 1) / len / 4 + 2 < s.ni) s.nt = nt;
+    }
+  }
+  if (s.nt > 0) {
+    s.x0 = pg < s.nt ? run_start(s, pg) : 0;
+    s.E = s.tail0 + (pg < s.nt ? run_start(s, pg + 1) - s.x0 : 0);
+  } else {
+    s.x0 = pg * s.ni;
+    s.E = s.tail0 + (pg < r ? s.ni : 0);
+  }
   s.c0 = p.c_base + s.m * p.chunk;
   s.cw = min(p.chunk, p.c_end - s.c0);
   if (s.cw < 0) s.cw = 0;
@@ -274,12 +338,25 @@ __device__ GSched make_gsched(const GroupParams& p) {
   return s;
 }
 
-// global index of the group's i-th outer tile (s.ph for a phantom)
-__device__ __forceinline__ bool phantom(const GroupParams& p, const GSched& s, int i) {
-  return s.q + i * p.ngroups >= s.no;
+// row pair and inner tile of the group's exchange tile e
+struct Pos {
+  int rp, k;
+};
+__device__ __forceinline__ Pos locate(const GSched& s, int e) {
+  const bool tail = e >= s.tail0;
+  const int x = tail ? s.x0 + e - s.tail0 : e;
+  const int i = x / s.ni;
+  return Pos{tail ? s.rp0 + i : s.pg + i * s.npg, x - i * s.ni};
 }
-__device__ __forceinline__ int outer_of(const GroupParams& p, const GSched& s, int i) {
-  const int k = s.q + i * p.ngroups;
+// does tile e open / close its outer tile's part in this group?
+__device__ __forceinline__ bool opens(const GSched& s, int e, int k) { return k == 0 || e == s.tail0; }
+__device__ __forceinline__ bool closes(const GSched& s, int e, int k) {
+  return k == s.ni - 1 || e == s.E - 1;
+}
+// index of this CTA's outer tile of a row pair (s.ph for a phantom)
+__device__ __forceinline__ bool phantom(const GSched& s, int rp) { return 2 * rp + s.rank >= s.no; }
+__device__ __forceinline__ int outer_of(const GroupParams& p, const GSched& s, int rp) {
+  const int k = 2 * rp + s.rank;
   if (k >= s.no) return s.ph;
   return (p.mode == GM_A && p.redo) ? static_cast<int>(p.redo_list[1 + k]) : k;
 }
@@ -290,11 +367,11 @@ __device__ __forceinline__ int kvalid_of(const GSched& s, int k) {
 __device__ __forceinline__ int slices_of(const GSched& s, int k) {
   return (kvalid_of(s, k) + kBK - 1) / kBK;
 }
-// does member m compute a Z job of the group's i-th outer tile?
-__device__ __forceinline__ bool member_has_job(const GSched& s, int g, int i) {
-  const int lo = i * s.ni;
-  const int first = lo + (((s.m - lo) % g) + g) % g;
-  return first < lo + s.ni;
+// does member m compute a Z job of the outer tile part that tile e (at inner
+// tile k) closes?
+__device__ __forceinline__ bool member_has_job(const GSched& s, int g, int e, int k) {
+  const int lo = e >= s.tail0 ? max(e - k, s.tail0) : e - k;
+  return lo + (((s.m - lo) % g) + g) % g <= e;
 }
 
 // Where a round's accumulation [e_lo, e_end) pauses for the second Z product.
@@ -307,8 +384,8 @@ __device__ __forceinline__ bool member_has_job(const GSched& s, int g, int i) {
 template <int kMode>
 __device__ __forceinline__ int split_point(const GSched& s, int e_lo, int e_end) {
   if (kMode != GM_KL || e_lo == e_end) return e_end;
-  const int opens = (e_lo / s.ni + 1) * s.ni;  // first tile after e_lo with k = 0
-  return min(e_lo + (e_end - e_lo + 1) / 2, opens);
+  const int next = e_lo + s.ni - locate(s, e_lo).k;  // first tile after e_lo that opens an outer tile
+  return min(e_lo + (e_end - e_lo + 1) / 2, next);
 }
 
 // byte offset of row r (a multiple of 8) of K-slice sl in an exchange tile.
@@ -318,35 +395,6 @@ __device__ __forceinline__ int split_point(const GSched& s, int e_lo, int e_end)
 // operand.
 __device__ __forceinline__ uint32_t img_off(int r, int sl) {
   return static_cast<uint32_t>(sl * kXSlice + r * 128);
-}
-
-__device__ __forceinline__ void store_out32(void* base, size_t off, int dtype, int n_valid,
-                                            const float (&v)[32]) {
-  if (dtype == OLIVE_DTYPE_BF16) {
-    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(base) + off;
-    if (n_valid >= 32) {
-      uint4* d4 = reinterpret_cast<uint4*>(o);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        d4[q] = make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
-                           pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
-    } else {
-#pragma unroll
-      for (int k = 0; k < 32; ++k)
-        if (k < n_valid) o[k] = __float2bfloat16_rn(v[k]);
-    }
-  } else {
-    float* o = static_cast<float*>(base) + off;
-    if (n_valid >= 32) {
-      float4* d4 = reinterpret_cast<float4*>(o);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 32; ++k)
-        if (k < n_valid) o[k] = v[k];
-    }
-  }
 }
 
 // 32 fp32 values (the slice's first or last 32 columns) -> four 16-byte
@@ -448,6 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t oempty = zfull + 24;
   const uint32_t drain = zfull + 32;
   uint8_t* misc = gbase + kStages * kStageBytes + kEpiWarps * kWarpSlice + 8 * (2 * kStages + 5);
+  static_assert(16 + sizeof(GSched) <= 128, "schedule area");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
   volatile uint32_t* copied = reinterpret_cast<volatile uint32_t*>(misc + 8);  // tiles copied
@@ -530,8 +579,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a Z product: za x zb, or GM_KL's teacher za2 x zb2; the B rows are this
         // CTA's half of the 256-wide vocabulary (or row) tile
         auto load_z = [&](bool second) {
-          const int o = outer_of(p, s, j / s.ni);
-          const int k = j % s.ni;
+            const Pos at = locate(s, j);
+          const int o = outer_of(p, s, at.rp);
+          const int k = at.k;
           const int steps = second ? s.nk2 : s.nk;
           for (int ks = 0; ok && ks < steps; ++ks) {
             if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
@@ -551,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         auto load_tiles = [&](int e_from, int e_to) {
           for (int e = e_from; ok && e < e_to; ++e) {
             const int slot = e % p.R;
-            const int k = e % s.ni;
+            const int k = locate(s, e).k;
             const int nsl = slices_of(s, k);
             for (int sl = 0; sl < nsl; ++sl) {
               if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
@@ -653,8 +703,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           };
           auto accumulate = [&](int e_from, int e_to) {
             for (int e = e_from; ok && e < e_to; ++e) {
-              const int k = e % s.ni;
-              if (k == 0) {
+              const int k = locate(s, e).k;
+              const bool first = opens(s, e, k);
+              if (first) {
                 if (!mbar_wait(oempty, oph ^ 1u, ctl)) { ok = false; break; }
                 tc_fence_after();
               }
@@ -668,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int kk = 0; kk < kBK / 16; ++kk)
                   umma_bf16_pair(oacc, sdesc_sw128(sA + kk * 32, 16, 1024),
                                  sdesc_sw128(sB + kk * 2048, 8192, 1024), idx,
-                                 (k > 0 || sl > 0 || kk > 0) ? 1u : 0u);
+                                 (!first || sl > 0 || kk > 0) ? 1u : 0u);
                 umma_commit_pair(empty_bar(stage));
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
               }
@@ -678,7 +729,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               // group's members have said so)
               *copied = static_cast<uint32_t>(e + 1);
               st_shared_cluster(copied_peer, static_cast<uint32_t>(e + 1));
-              if (k == s.ni - 1) {
+              if (closes(s, e, k)) {
                 umma_commit_pair(ofull);
                 oph ^= 1u;
               }
@@ -749,26 +800,78 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive_cluster(oempty_lead);
       return true;
     };
-    // acc -> output row t (a packed row or vocabulary row), stored as is
+    // acc -> output row t (a packed or vocabulary row; -1: none).  128 bytes
+    // of each of the warp's 32 rows at a time (64 bf16 or 32 fp32 columns) go
+    // through the staging area, so that a store instruction writes four whole
+    // lines; from the registers it would write half sectors of 32 lines, and
+    // a 128 x 224 tile took 5 us.
     auto store_output = [&](int t, const float(&acc)[4][32]) {
+      const bool wide = p.out_dtype == OLIVE_DTYPE_F32;
+      const int per = wide ? 32 : 64;  // columns of a step, 8 chunks of 16 bytes
+      const uint32_t mine = staging + lane * 128;
+      auto flush = [&](int c) {
+        __syncwarp();
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c = ob + 32 * b;
-        if (c < oe && OLIVE_DCHECK(p.dev_status, s.c0 + min(c + 32, oe) <= p.d))
-          store_out32(p.out, static_cast<size_t>(t) * p.d + s.c0 + c, p.out_dtype, min(32, oe - c), acc[b]);
+        for (int u = 0; u < 8; ++u) {
+          const int rr = u * 4 + (lane >> 3);
+          const int tr = __shfl_sync(0xffffffffu, t, rr);
+          const uint4 v = ld_shared_v4(staging + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
+          const int col = c + (lane & 7) * (per / 8);
+          if (tr >= 0 && col < oe && OLIVE_DCHECK(p.dev_status, s.c0 + col + per / 8 <= p.d)) {
+            const size_t at = static_cast<size_t>(tr) * p.d + s.c0 + col;
+            *reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) + (wide ? 4 : 2) * at) = v;
+          }
+        }
+        __syncwarp();
+      };
+      if (wide) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (ob + 32 * b >= oe) continue;
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            st_shared_v4(mine + ((q ^ (lane & 7)) << 4),
+                         make_uint4(__float_as_uint(acc[b][4 * q]), __float_as_uint(acc[b][4 * q + 1]),
+                                    __float_as_uint(acc[b][4 * q + 2]), __float_as_uint(acc[b][4 * q + 3])));
+          flush(ob + 32 * b);
+        }
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; b += 2) {
+          if (ob + 32 * b >= oe) continue;
+          stage32(staging, lane, 0, acc[b]);
+          stage32(staging, lane, 1, acc[b + 1]);
+          flush(ob + 32 * b);
+        }
       }
+    };
+
+    // pass A: this thread's sum and maximum of the row, for the part of the
+    // outer tile that exchange tile e belongs to
+    auto tail_row = [&](int slot, int mm) -> size_t {
+      return (static_cast<size_t>(slot) * 2 * g + mm) * 2 * kBM + s.rank * kBM + row;
+    };
+    auto put_sums = [&](int e, int rp, int o, float sum, float mx) {
+      const bool tail = s.nt > 0 && e >= s.tail0;
+      const size_t i = tail ? tail_row(s.pg + rp - s.rp0, 2 * s.m + half)
+                            : static_cast<size_t>(2 * s.m + half) * Tpad + o * kBM + row;
+      if (!OLIVE_DCHECK(p.dev_status, tail ? s.pg + rp - s.rp0 < p.tail_slots
+                                           : 2 * s.m + half < p.part_groups && o * kBM + row < static_cast<int>(Tpad)))
+        return;
+      (tail ? p.tail_s : p.part_s)[i] = sum;
+      (tail ? p.tail_m : p.part_m)[i] = mx;
     };
 
     if (kMode == GM_B && s.ni == 0) {
       // no masked rows: dW is zero on this member's columns of its outer tiles
       float acc[4][32] = {};
-      for (int i = 0; i < s.myo; ++i) {
-        const int v = outer_of(p, s, i) * kBM + row;
-        if (v < p.V) store_output(v, acc);
+      for (int rp = s.pg; 2 * rp < s.no; rp += s.npg) {
+        const int v = outer_of(p, s, rp) * kBM + row;
+        store_output(v < p.V ? v : -1, acc);
       }
     }
 
-    int cur_o = -1;             // pass A: the outer tile of the running partials
+    int cur_rp = -1;            // pass A: the row pair of the running partials
     RowA ra{false, -1, -1, 0.f};
     float run_s = 0.f, run_m = -INFINITY;  // of 2^(x - R) and of x - R
     const float s_coef = s.coef;
@@ -776,9 +879,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int j = r * g + s.m;
       if (r < nr && j < s.E) {
         // ---------------------------------------------------- Z epilogue
-        const int i = j / s.ni;
-        const int k = j % s.ni;
-        const int o = outer_of(p, s, i);
+        const Pos at = locate(s, j);
+        const int k = at.k;
+        const int o = outer_of(p, s, at.rp);
         const int slot = j % p.R;
         const int kv = kvalid_of(s, k);
         // 32-column blocks to read: every block of the slices the members
@@ -944,8 +1047,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             put(h, gv);
           }
         } else {
-          if (o != cur_o) {
-            cur_o = o;
+          if (at.rp != cur_rp) {
+            cur_rp = at.rp;
             ra = load_row_a(p, s, o * kBM + row);
             run_s = 0.f;
             run_m = -INFINITY;
@@ -1006,11 +1109,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
           named_bar_sync(1, kEpi);
         } else {
-          if (kMode == GM_A && ra.valid &&
-              OLIVE_DCHECK(p.dev_status, 2 * s.m + half < p.part_groups && o * kBM + row < static_cast<int>(Tpad))) {
-            p.part_s[static_cast<size_t>(2 * s.m + half) * Tpad + o * kBM + row] = run_s;
-            p.part_m[static_cast<size_t>(2 * s.m + half) * Tpad + o * kBM + row] = run_m + ra.R;
-          }
+          if (kMode == GM_A && ra.valid) put_sums(j, at.rp, o, run_s, run_m + ra.R);
           // publish the warp's part of the tile once its copies are complete
           if (lane == 0) {
             bulk_wait();
@@ -1026,51 +1125,107 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ------------------------------------------- outer tiles completed
       const int e_end = min(r * g, s.E);
       for (int e = (r - 1) * g; ok && e < e_end; ++e) {
-        if (e % s.ni != s.ni - 1) continue;
-        const int i = e / s.ni;
-        const int o = outer_of(p, s, i);
-        float acc[4][32];
-        if (kMode == GM_B) {
-          if (!take_output(acc)) { ok = false; break; }
-          const int v = o * kBM + row;
-          if (v < p.V && OLIVE_DCHECK(p.dev_status, v >= 0)) store_output(v, acc);
-          continue;
-        }
-        if (kMode == GM_KL) {
-          // the divergence gradient: G carried g inv_tau, so d_h_s is the sum
-          if (!take_output(acc)) { ok = false; break; }
-          const int rc = o * kBM + row;
-          const int t = rc < s.n ? p.rows[rc] : -1;
-          if (t >= 0 && t < p.T) store_output(t, acc);
-          continue;
-        }
-        // pass A: merge the members' partials, then dH
+        const Pos at = locate(s, e);
+        if (!closes(s, e, at.k)) continue;
+        const int o = outer_of(p, s, at.rp);
+        const bool split = s.nt > 0 && e >= s.tail0;
+        // the runs [run_lo, run_hi] of the tail that hold a part of this row pair
+        const int t = at.rp - s.rp0;
+        const int run_lo = split ? run_of(s, t * s.ni) : 0;
+        const int run_hi = split ? run_of(s, (t + 1) * s.ni - 1) : 0;
         const int rc = o * kBM + row;
-        const RowA rw = load_row_a(p, s, rc);
-        // every member's partials (and the target's z_y, P'_y from the
-        // member that met it) are published before any member reads them
-        if (rw.valid && !member_has_job(s, g, i)) {
-          p.part_s[static_cast<size_t>(2 * s.m + half) * Tpad + rc] = 0.f;
-          p.part_m[static_cast<size_t>(2 * s.m + half) * Tpad + rc] = -INFINITY;
-        }
-        const bool whole = !phantom(p, s, i) && OLIVE_DCHECK(p.dev_status, o >= 0 && o * kBM < static_cast<int>(Tpad));
-        if (whole) {
+        RowA rw{false, -1, -1, 0.f};
+        const bool whole = !phantom(s, at.rp) && OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph);
+        if (kMode == GM_A && whole) {
+          // every member's sums (and the target's z_y, P'_y from the member
+          // that met it) are published before any member reads them
+          rw = load_row_a(p, s, rc);
+          if (rw.valid && !member_has_job(s, g, e, at.k)) put_sums(e, at.rp, o, 0.f, -INFINITY);
           __threadfence();
           named_bar_sync(1, kEpi);
           if (threadIdx.x == 0) red_release_add(p.outer_ctr + o, 1u);
         }
+        float acc[4][32];
         if (!take_output(acc)) { ok = false; break; }
+        if (split) {
+          if (!whole) continue;  // a phantom: its rows are never stored
+          // the layout is the threads' own (16 bytes of every thread side by
+          // side), so stores and loads are whole lines
+          auto part = [&](int run) {
+            return reinterpret_cast<float4*>(p.tail_acc) +
+                   (static_cast<size_t>((run + t) * 2 + s.rank) * g + s.m) * kTailVecs + threadIdx.x;
+          };
+          if (!OLIVE_DCHECK(p.dev_status, ((run_hi + t) * 2 + s.rank) * g + s.m < p.tail_parts)) {
+            ok = false;
+            break;
+          }
+          float4* out = part(s.pg);
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            if (ob + 32 * b >= oe) continue;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              out[(8 * b + q) * kEpi] =
+                  make_float4(acc[b][4 * q], acc[b][4 * q + 1], acc[b][4 * q + 2], acc[b][4 * q + 3]);
+          }
+          __threadfence();
+          named_bar_sync(1, kEpi);
+          bool last = true;
+          if (threadIdx.x == 0) {
+            last = atomicAdd(p.tail_ctr + (2 * t + s.rank) * g + s.m, 1u) ==
+                   static_cast<uint32_t>(run_hi - run_lo);
+            __threadfence();
+          }
+          if (!named_bar_and(1, kEpi, last)) continue;
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[b][c] = 0.f;
+          }
+          for (int c = run_lo; c <= run_hi; ++c) {
+            const float4* in = part(c);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              if (ob + 32 * b >= oe) continue;
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const float4 v = __ldcg(in + (8 * b + q) * kEpi);
+                acc[b][4 * q] += v.x;
+                acc[b][4 * q + 1] += v.y;
+                acc[b][4 * q + 2] += v.z;
+                acc[b][4 * q + 3] += v.w;
+              }
+            }
+          }
+        }
+        if (kMode == GM_B) {
+          store_output(rc < p.V ? rc : -1, acc);
+          continue;
+        }
+        if (kMode == GM_KL) {
+          // the divergence gradient: G carried g inv_tau, so d_h_s is the sum
+          const int tr = rc < s.n ? p.rows[rc] : -1;
+          store_output(tr < p.T ? tr : -1, acc);
+          continue;
+        }
+        // pass A: merge the members' sums, then dH
         if (whole) {
-          const bool seen =
-              threadIdx.x == 0 ? wait_counter(p.outer_ctr + o, static_cast<uint32_t>(g), ctl) : true;
+          const uint32_t posts = static_cast<uint32_t>(g * (run_hi - run_lo + 1));
+          const bool seen = threadIdx.x == 0 ? wait_counter(p.outer_ctr + o, posts, ctl) : true;
           if (!named_bar_and(1, kEpi, seen)) { ok = false; break; }
         }
         float lse2 = rw.R, mx = -INFINITY;
         if (!p.lse_known && rw.valid) {
           float sum = 0.f;
-          for (int mm = 0; mm < 2 * g; ++mm) {
-            sum += __ldcg(p.part_s + static_cast<size_t>(mm) * Tpad + rc);
-            mx = fmaxf(mx, __ldcg(p.part_m + static_cast<size_t>(mm) * Tpad + rc));
+          for (int c = run_lo; c <= run_hi; ++c) {
+            const size_t from = split ? tail_row(c + t, 0) : rc;
+            const size_t stride = split ? 2 * kBM : Tpad;
+            const float* ps = split ? p.tail_s : p.part_s;
+            const float* pm = split ? p.tail_m : p.part_m;
+            for (int mm = 0; mm < 2 * g; ++mm) {
+              sum += __ldcg(ps + from + mm * stride);
+              mx = fmaxf(mx, __ldcg(pm + from + mm * stride));
+            }
           }
           lse2 = rw.R + log2f(sum);
         }
@@ -1131,7 +1286,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           }
-          if (rw.valid && OLIVE_DCHECK(p.dev_status, rw.t >= 0 && rw.t < p.T)) store_output(rw.t, acc);
+          store_output(rw.valid ? rw.t : -1, acc);
         }
       }
     }
@@ -1247,14 +1402,28 @@ int group_g_max(int64_t d) {
 
 int ring_slots(int g) { return ring_slots_for(g); }
 
-// groups a launch forms at most (an even number): as many as the SMs hold,
-// and no more than the outer tiles of either pass (row tiles of T rows,
-// vocabulary tiles) rounded up to a pair
+// groups a launch forms at most (an even number): as many pair-groups as the
+// SMs hold, and no more than a pass has (row pair, inner tile) places, the
+// same number in both passes
 int group_count_max(int64_t T, int64_t d, int64_t V) {
   const int64_t cap = static_cast<int64_t>(sweep_cols_for(kGroupMaxSms));
   const int gmin = g_min_for(static_cast<int>(d < cap ? d : cap));
-  const int64_t outer = std::max<int64_t>(std::max(ceil_div(T, kBM), ceil_div(V, kBM)), 2);
-  return static_cast<int>(std::min<int64_t>(2 * (kGroupMaxSms / (2 * gmin)), (outer + 1) / 2 * 2));
+  return static_cast<int>(2 * std::min<int64_t>(kGroupMaxSms / (2 * gmin),
+                                                ceil_div(T, 2 * kBM) * ceil_div(V, 2 * kBM)));
+}
+
+// partial accumulators of split row pairs: slots, and 128 x 256 tiles in all
+// (two a member of every slot; the grid's members are one a CTA)
+int group_tail_slots(int64_t T, int64_t d, int64_t V) { return group_count_max(T, d, V); }
+int64_t group_tail_parts(int64_t T, int64_t d, int64_t V) {
+  return std::min<int64_t>(2ll * group_tail_slots(T, d, V) * group_g_max(d), 2 * kGroupMaxSms);
+}
+size_t group_tail_bytes(int64_t T, int64_t d, int64_t V) {
+  return static_cast<size_t>(group_tail_parts(T, d, V)) * kTailVecs * sizeof(float4);
+}
+// GM_A's sums (and as many maxima) of those slots, in floats
+size_t group_tail_sums(int64_t T, int64_t d, int64_t V) {
+  return static_cast<size_t>(group_tail_slots(T, d, V)) * 2 * group_g_max(d) * 2 * kBM;
 }
 
 size_t group_ring_words(int64_t T, int64_t d, int64_t V) {
@@ -1263,9 +1432,10 @@ size_t group_ring_words(int64_t T, int64_t d, int64_t V) {
 
 size_t group_ring_bytes(int64_t T, int64_t d, int64_t V) { return group_ring_words(T, d, V) * kXTile; }
 
-// counter words of one launch: ready and cons per ring slot, pace per group
+// counter words of one launch: ready and cons per ring slot, pace per group,
+// arrivals per split row tile and member (at most one a CTA)
 size_t group_ctr_words(int64_t T, int64_t d, int64_t V) {
-  return 2 * group_ring_words(T, d, V) + static_cast<size_t>(group_count_max(T, d, V));
+  return 2 * group_ring_words(T, d, V) + static_cast<size_t>(group_count_max(T, d, V)) + kGroupMaxSms;
 }
 
 int group_sweep_cols(int sms) { return sweep_cols_for(sms < kGroupMaxSms ? sms : kGroupMaxSms); }
@@ -1350,6 +1520,12 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   p.ready = ring_ctr;
   p.cons = ring_ctr ? ring_ctr + static_cast<size_t>(gs.ngroups) * gs.R : nullptr;
   p.pace = ring_ctr ? ring_ctr + 2 * static_cast<size_t>(gs.ngroups) * gs.R : nullptr;
+  p.tail_ctr = ring_ctr ? p.pace + gs.ngroups : nullptr;
+  p.tail_acc = mode == GM_REF ? nullptr : a.tail_acc;
+  p.tail_s = a.tail_s;
+  p.tail_m = a.tail_m;
+  p.tail_parts = static_cast<int32_t>(group_tail_parts(T, d, V));
+  p.tail_slots = group_tail_slots(T, d, V);
   p.out = mode == GM_B ? a.d_W : a.d_hidden;  // GM_KL: d_h_s
   p.out_dtype = a.out_dtype;
   p.ring_tiles = static_cast<int64_t>(group_ring_words(T, d, V));
@@ -1413,6 +1589,9 @@ olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,
   a.redo_list = w.redo;
   a.outer_ctr = w.outer;
   a.ring = w.ring;
+  a.tail_acc = w.tail_acc;
+  a.tail_s = w.tail_s;
+  a.tail_m = w.tail_m;
   a.d_hidden = d_hidden;
   a.d_W = d_W;
   a.out_dtype = grad_dtype;
@@ -1452,8 +1631,8 @@ olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct
                                   const int32_t* n_rows, int32_t T, int32_t V, float inv_tau,
                                   int reverse, const float* kl, const float* lse_s,
                                   const float* lse_t, const float* grad_kl, void* d_h_s,
-                                  int grad_dtype, void* ring, uint32_t* ctr, size_t ctr_words,
-                                  int32_t* dev_status) {
+                                  int grad_dtype, void* ring, float* tail_acc, uint32_t* ctr,
+                                  size_t ctr_words, int32_t* dev_status) {
   const int64_t rt = align_up(static_cast<size_t>(T), kRowAlign) / kRowAlign;
   GroupArgs a = {};
   a.dev_status = dev_status;
@@ -1461,6 +1640,7 @@ olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct
   a.rows = rows;
   a.inv_tau = inv_tau;
   a.ring = ring;
+  a.tail_acc = tail_acc;
   a.d_hidden = d_h_s;
   a.out_dtype = grad_dtype;
   a.hc2 = hct;

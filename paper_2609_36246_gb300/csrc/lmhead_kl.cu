@@ -291,7 +291,8 @@ olive_status launch_divergence(const Ctx& c, const void* h_s, const void* W_s, i
     return OLIVE_ERR_CUDA;
   return launch_kl_group_grad(c, w.hcs, w.hct, W_s, d_s, W_t, d_t, rows, n_rows, T, V, inv_tau,
                               reverse, kl, reverse ? w.lse_p : w.lse_q, reverse ? w.lse_q : w.lse_p,
-                              grad_kl, d_h_s, grad_dtype, w.ring, w.ctr, w.ctr_words, dev_status);
+                              grad_kl, d_h_s, grad_dtype, w.ring, w.tail_acc, w.ctr, w.ctr_words,
+                              dev_status);
 }
 
 }  // namespace olive

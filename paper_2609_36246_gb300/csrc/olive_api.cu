@@ -274,6 +274,9 @@ static GroupWs carve_group_impl(void* ws, int64_t T, int64_t d, int64_t V, size_
   w.part_s = static_cast<float*>(c.take(8ull * gmax * Tpad));
   w.part_m = static_cast<float*>(c.take(8ull * gmax * Tpad));
   w.ring = c.take(group_ring_bytes(T, d, V));
+  w.tail_acc = static_cast<float*>(c.take(group_tail_bytes(T, d, V)));
+  w.tail_s = static_cast<float*>(c.take(4ull * group_tail_sums(T, d, V)));
+  w.tail_m = static_cast<float*>(c.take(4ull * group_tail_sums(T, d, V)));
   // counters in one region, zeroed by one memset per column sweep: group
   // barriers [2 rt] (first and redo launch), the redo list [1 + rt], then the
   // ring counters of the three launches of a sweep
@@ -308,6 +311,7 @@ static KlWs carve_kl_impl(void* ws, int64_t T, int64_t ds, int64_t dt, int64_t V
     w.lse_p = static_cast<float*>(c.take(4ull * Tpad));
     w.lse_q = static_cast<float*>(c.take(4ull * Tpad));
     w.ring = c.take(group_ring_bytes(T, ds, V));
+    w.tail_acc = static_cast<float*>(c.take(group_tail_bytes(T, ds, V)));
     // the same counter layout as the training step's (group barriers and
     // redo list unused here), so every sweep's launch has its ring counters
     w.ctr_words = static_cast<size_t>(3 * rt + 1) + 3 * group_ctr_words(T, ds, V);

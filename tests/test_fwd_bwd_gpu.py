@@ -321,3 +321,23 @@ def test_runs_are_bitwise_reproducible():
     torch.cuda.synchronize()
     for x, y in zip(*runs):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("n,V,d", [(1, 20000, 64), (128, 5000, 256), (130, 3000, 4096), (300, 9000, 1032),
+                                   (700, 2305, 2048), (1300, 6000, 2560), (4100, 1500, 136)])
+@pytest.mark.parametrize("redo", [False, True])
+def test_split_row_pairs(n, V, d, redo):
+    """Row pairs left over from the whole rounds of the pair-groups are split
+    between them (both passes), their sums and accumulators merged: one row to
+    several row pairs, runs that span two row pairs, odd row tiles, and rows
+    above their reference, whose redo launch is split the same way."""
+    rng = np.random.default_rng(n + V)
+    b = synth.batch_from_lengths(rng, [3, 2], [n - n // 3, n // 3], V)
+    h = synth.normal_bf16(rng, (b.T, d), 1.0)
+    W = synth.normal_bf16(rng, (V, d), 0.8 / d ** 0.5)
+    if redo:
+        # a direction that half of the rows share: their logit V // 2 is about
+        # 60 nats above every logit of the first vocabulary tile
+        h[::2, 0] = 8.0
+        W[V // 2, 0] = 8.0
+    _full_check(b, h, W, grad_loss=0.7, grad_dtype=torch.float32)
