@@ -22,8 +22,8 @@
 //
 // A Kern policy supplies:
 //   Params (with int32_t* dev_status and uint64_t wait_limit_ns), kBN, kAMn,
-//   kBMn, kDual, kStages, kEpiWarps, Sched, make_sched(p) (thread 0; may read
-//   device counters such as n_rows), num_units(p,s), unit_len(p,s,u),
+//   kBMn, kDual, kStages, kEpiWarps, Sched, make_sched(p) (one whole warp; may
+//   read device counters such as n_rows), num_units(p,s), unit_len(p,s,u),
 //   tile(p,s,u,t), kEpiSmem (bytes of shared-memory scratch for the epilogue)
 //   and Epi with init(smem, part), begin(p,s,u,row), tile(p,s,u,t,tc,taddr),
 //   end(p,s,u).  Every wait of the epilogue ends in one decision of all its
@@ -124,8 +124,12 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
-    *sched_smem = Kern::make_sched(p);
     fence_mbar_init();
+  }
+  if (warp == 0) {
+    __syncwarp();
+    const typename Kern::Sched sc = Kern::make_sched(p);
+    if (lane == 0) *sched_smem = sc;
   }
   if (warp == CT::kProducer && lane == 0) {
     tma_prefetch_desc(&mapA);

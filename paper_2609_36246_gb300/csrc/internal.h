@@ -12,11 +12,21 @@
 
 namespace olive {
 
-constexpr int kSvMax = 64;        // most vocabulary segments per row tile
+constexpr int kSvMax = 64;        // most vocabulary segments per row tile (more for one or two, kMinParts)
+// (row tile, segment) partials a sweep's workspace holds at least, so that one
+// or two row tiles can be cut finely enough to fill the SMs; the OPD sweep
+// writes two a segment
+constexpr int kMinParts = 160;
+constexpr int kMinPartsOpd = 320;
 constexpr int kRowAlign = 128;    // row tiles of the compacted hidden copy
 constexpr size_t kWsAlign = 256;  // alignment of every workspace region
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+// rows of one partial array of a sweep over Tpad rows
+inline size_t part_rows(int64_t Tpad, int min_parts) {
+  const size_t a = static_cast<size_t>(kSvMax) * Tpad, b = static_cast<size_t>(min_parts) * 128;
+  return a > b ? a : b;
+}
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Launch context gathered once per API call.
@@ -52,8 +62,8 @@ inline int64_t vpad(int64_t V) { return align_up(static_cast<size_t>(V), 8); }
 // ---- workspace carving (sizes in bytes; every region 256-byte aligned) ----
 struct FwdWs {
   void* hc;       // bf16 [Tpad, d] compacted hidden rows
-  float* part_m;  // [kSvMax, Tpad]
-  float* part_s;  // [kSvMax, Tpad]
+  float* part_m;  // [part_rows]: segment, row (row tiles x 128 to a segment)
+  float* part_s;  // [part_rows]
   float* zy;      // [Tpad]
   float* nll;     // [Tpad]
 };
@@ -62,11 +72,11 @@ FwdWs carve_fwd(void* ws, int64_t T, int64_t d);
 
 struct TopkWs {
   void* hc;          // bf16 [Tpad, d]
-  float* part_m;     // [kSvMax, Tpad]
-  float* part_s;     // [kSvMax, Tpad]
-  float* part_a;     // [kSvMax, Tpad] entropy numerators
-  float* part_tv;    // [kSvMax, Tpad, 16] per-segment top logits
-  int32_t* part_ti;  // [kSvMax, Tpad, 16] their vocabulary ids
+  float* part_m;     // [part_rows]
+  float* part_s;     // [part_rows]
+  float* part_a;     // [part_rows] entropy numerators
+  float* part_tv;    // [part_rows, 16] per-segment top logits
+  int32_t* part_ti;  // [part_rows, 16] their vocabulary ids
 };
 size_t topk_ws_bytes(int64_t T, int64_t d);
 TopkWs carve_topk(void* ws, int64_t T, int64_t d);
@@ -86,12 +96,12 @@ size_t topk_kl_bwd_ws_bytes(int64_t T, int64_t d, int64_t V, int grad_dtype);
 struct OpdWs {
   void* hcs;         // bf16 [Tpad, d_s]
   void* hct;         // bf16 [Tpad, d_t]
-  float* part;       // [6, kSvMax, Tpad]
-  float* part_sv;    // [kSvMax, Tpad, 16]
-  int32_t* part_si;  // [kSvMax, Tpad, 16]
-  float* part_sx;    // [kSvMax, Tpad, 16]
-  float* part_tv;    // [kSvMax, Tpad, 16]
-  int32_t* part_ti;  // [kSvMax, Tpad, 16]
+  float* part;       // [6, part_rows]
+  float* part_sv;    // [part_rows, 16]
+  int32_t* part_si;  // [part_rows, 16]
+  float* part_sx;    // [part_rows, 16]
+  float* part_tv;    // [part_rows, 16]
+  int32_t* part_ti;  // [part_rows, 16]
 };
 size_t opd_ws_bytes(int64_t T, int64_t ds, int64_t dt);
 OpdWs carve_opd(void* ws, int64_t T, int64_t ds, int64_t dt);
@@ -116,7 +126,7 @@ FbWs carve_fb(void* ws, int64_t T, int64_t d, int64_t V, int grad_dtype);
 struct KlWs {
   void* hcs;      // bf16 [Tpad, d_s]
   void* hct;      // bf16 [Tpad, d_t]
-  float* part;    // [5, kSvMax, Tpad] value-sweep partials
+  float* part;    // [5, part_rows] value-sweep partials
   // gradient only: both heads' lse per compact row (p the primary head), the
   // exchange ring of the on-chip gradient pass and its counters
   float* lse_p;   // [Tpad]

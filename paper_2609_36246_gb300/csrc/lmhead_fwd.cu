@@ -17,6 +17,7 @@
 //   finalize    merges the per-segment partials, writes lse and
 //               logp = z_y - lse (or entropy and top-K) on the packed rows
 //   loss        one block sums -logp in a fixed order (deterministic)
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -51,15 +52,14 @@ struct FwdKernT {
     int32_t T, d, V;
     int32_t ctas;        // CTAs the decomposition is computed for (= grid)
     int32_t group_rows;  // row tiles per raster group
-    int32_t ld;          // row stride of the partial arrays
     float scale2;        // inv_tau * log2(e): logits in base-2 units
     float inv_tau;
     float* part_m;
     float* part_s;
     float* zy;           // loss variant
-    float* part_a;       // stats: [kSvMax][ld]
-    float* part_tv;      // stats: [kSvMax][ld][16] raw logits
-    int32_t* part_ti;    // stats: [kSvMax][ld][16] vocabulary ids
+    float* part_a;       // stats: as part_m, [segment][rt 128]
+    float* part_tv;      // stats: [segment][rt 128][16] raw logits
+    int32_t* part_ti;    // stats: [segment][rt 128][16] vocabulary ids
   };
   struct Sched {
     Split sp;
@@ -68,7 +68,7 @@ struct FwdKernT {
   static __device__ Sched make_sched(const Params& p) {
     Sched s;
     const int n = read_n_rows(p.n_rows, p.T, p.dev_status);
-    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas);
+    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas, split_cap((n + 127) / 128, kMinParts));
     return s;
   }
   static __device__ int num_units(const Params&, const Sched& s) { return s.sp.units; }
@@ -216,7 +216,7 @@ struct FwdKernT {
 
     __device__ void end(const Params& p, const Sched& sc, int) {
       if (r >= sc.sp.n) return;
-      const size_t o = static_cast<size_t>(sg) * p.ld + r;
+      const size_t o = static_cast<size_t>(sg) * sc.sp.rt * kBM + r;
       p.part_m[o] = m;
       p.part_s[o] = s;
       if constexpr (kStats) {
@@ -264,23 +264,25 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, const int32
   }
 }
 
-__global__ void fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
-                                    const int32_t* __restrict__ targets, int T, int V, int vt,
-                                    int ctas, int ld, const float* __restrict__ part_m,
-                                    const float* __restrict__ part_s, const float* __restrict__ zy,
-                                    float* __restrict__ logp, float* __restrict__ lse,
-                                    float* __restrict__ nll, int32_t* dev_status) {
-  __shared__ int sh_sv;
+// One warp a row, its lanes over the row's segments.  (One thread a row walked
+// up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
+__global__ void __launch_bounds__(128)
+    fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
+                        const int32_t* __restrict__ targets, int T, int V, int vt, int ctas,
+                        const float* __restrict__ part_m, const float* __restrict__ part_s,
+                        const float* __restrict__ zy, float* __restrict__ logp,
+                        float* __restrict__ lse, float* __restrict__ nll, int32_t* dev_status) {
   const int n = read_n_rows(n_rows, T, nullptr);
-  if (threadIdx.x == 0) sh_sv = choose_split(n, vt, ctas).sv;
-  __syncthreads();
-  const int sv = sh_sv;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    float M = -INFINITY;
-    for (int s = 0; s < sv; ++s) M = fmaxf(M, part_m[static_cast<size_t>(s) * ld + r]);
-    float S = 0.f;
-    for (int s = 0; s < sv; ++s)
-      S += part_s[static_cast<size_t>(s) * ld + r] * exp2f(part_m[static_cast<size_t>(s) * ld + r] - M);
+  const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
+  const int lane = threadIdx.x & 31;
+  const size_t ld = static_cast<size_t>(sp.rt) * 128;
+  const int warps = gridDim.x * 4;
+  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
+    float M = -INFINITY, S = 0.f;
+    for (int s = lane; s < sp.sv; s += 32) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
+    for (int o = 16; o > 0; o >>= 1)
+      merge_ms(M, S, __shfl_xor_sync(0xffffffffu, M, o), __shfl_xor_sync(0xffffffffu, S, o));
+    if (lane) continue;
     const float l = (M + log2f(S)) * kLn2;
     const int t = rows[r];
     if (t < 0 || t >= T) {
@@ -301,55 +303,50 @@ __global__ void fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const in
   }
 }
 
-__global__ void stats_finalize_kernel(const int32_t* __restrict__ n_rows,
-                                      const int32_t* __restrict__ rows, int T, int vt, int ctas,
-                                      int ld, int K, float inv_tau, const float* __restrict__ part_m,
-                                      const float* __restrict__ part_s,
-                                      const float* __restrict__ part_a,
-                                      const float* __restrict__ part_tv,
-                                      const int32_t* __restrict__ part_ti,
-                                      float* __restrict__ lse, float* __restrict__ entropy,
-                                      float* __restrict__ topk_logp, int32_t* __restrict__ topk_ids) {
-  __shared__ int sh_sv;
+// One warp a row: lanes share the segments' sums and merge their top lists
+// (topk.cuh).
+__global__ void __launch_bounds__(128)
+    stats_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
+                          int vt, int ctas, int K, float inv_tau, const float* __restrict__ part_m,
+                          const float* __restrict__ part_s, const float* __restrict__ part_a,
+                          const float* __restrict__ part_tv, const int32_t* __restrict__ part_ti,
+                          float* __restrict__ lse, float* __restrict__ entropy,
+                          float* __restrict__ topk_logp, int32_t* __restrict__ topk_ids) {
   const int n = read_n_rows(n_rows, T, nullptr);
-  if (threadIdx.x == 0) sh_sv = choose_split(n, vt, ctas).sv;
-  __syncthreads();
-  const int sv = sh_sv;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+  const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
+  const int lane = threadIdx.x & 31;
+  const size_t ld = static_cast<size_t>(sp.rt) * 128;
+  const int warps = gridDim.x * 4;
+  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
     const int t = rows[r];
     if (t < 0 || t >= T) continue;  // reported by the gather kernel
-    float M = -INFINITY;
-    for (int s = 0; s < sv; ++s) M = fmaxf(M, part_m[static_cast<size_t>(s) * ld + r]);
-    float S = 0.f, A = 0.f;
-    float tv[kTopMax];
-    int ti[kTopMax];
-#pragma unroll
-    for (int j = 0; j < kTopMax; ++j) {
-      tv[j] = -INFINITY;
-      ti[j] = INT_MAX;
+    float M = -INFINITY, S = 0.f, A = 0.f;
+    for (int s = lane; s < sp.sv; s += 32) {
+      float f[2];
+      merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r], f);
+      A = A * f[0] + part_a[s * ld + r] * f[1];
     }
-    for (int s = 0; s < sv; ++s) {
-      const size_t o = static_cast<size_t>(s) * ld + r;
-      const float w = exp2f(part_m[o] - M);
-      S += part_s[o] * w;
-      A += part_a[o] * w;
-      for (int j = 0; j < kTopMax; ++j) {
-        const float cv = part_tv[o * kTopMax + j];
-        const int ci = part_ti[o * kTopMax + j];
-        if (cv > tv[kTopMax - 1] || (cv == tv[kTopMax - 1] && ci < ti[kTopMax - 1]))
-          topk_insert(tv, ti, cv, ci);
-      }
+    for (int o = 16; o > 0; o >>= 1) {
+      float f[2];
+      const float m2 = __shfl_xor_sync(0xffffffffu, M, o);
+      const float s2 = __shfl_xor_sync(0xffffffffu, S, o);
+      const float a2 = __shfl_xor_sync(0xffffffffu, A, o);
+      merge_ms(M, S, m2, s2, f);
+      A = A * f[0] + a2 * f[1];
     }
     const float l2 = M + log2f(S);
     const float l = l2 * kLn2;
-    lse[t] = l;
-    entropy[t] = kLn2 * (l2 - A / S);  // lse - E_p[z] in natural units
-#pragma unroll
-    for (int j = 0; j < kTopMax; ++j) {
-      if (j < K) {
-        topk_logp[static_cast<size_t>(t) * K + j] = tv[j] * inv_tau - l;
-        topk_ids[static_cast<size_t>(t) * K + j] = ti[j];
-      }
+    if (lane == 0) {
+      lse[t] = l;
+      entropy[t] = kLn2 * (l2 - A / S);  // lse - E_p[z] in natural units
+    }
+    float tv;
+    int ti;
+    size_t at;
+    warp_top_merge(part_tv, part_ti, sp.sv, ld, r, K, lane, tv, ti, at);
+    if (lane < K) {
+      topk_logp[static_cast<size_t>(t) * K + lane] = tv * inv_tau - l;
+      topk_ids[static_cast<size_t>(t) * K + lane] = ti;
     }
   }
 }
@@ -429,7 +426,6 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
   p.V = V;
   p.ctas = c.num_sms;
   p.group_rows = 16;
-  p.ld = static_cast<int32_t>(Tpad);
   p.scale2 = inv_tau * kLog2e;
   p.inv_tau = inv_tau;
   p.part_m = w.part_m;
@@ -438,9 +434,10 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
   if ((st = launch_fwd_core<FwdKern>(c, mA, mB, p)) != OLIVE_OK) return st;
 
   const int vt = (V + FwdKern::kBN - 1) / FwdKern::kBN;
-  fwd_finalize_kernel<<<c.num_sms * 4, 256, 0, c.stream>>>(n_rows, rows, targets, T, V, vt,
-                                                            c.num_sms, p.ld, w.part_m, w.part_s,
-                                                            w.zy, logp, lse, w.nll, dev_status);
+  const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
+  fwd_finalize_kernel<<<blocks, 128, 0, c.stream>>>(n_rows, rows, targets, T, V, vt, c.num_sms,
+                                                     w.part_m, w.part_s, w.zy, logp, lse, w.nll,
+                                                     dev_status);
   if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
   loss_reduce_kernel<<<1, 1024, 0, c.stream>>>(n_rows, T, w.nll, reduction, loss);
   if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
@@ -477,7 +474,6 @@ olive_status launch_topk_fwd(const Ctx& c, const void* hidden, const void* W, co
   p.V = V;
   p.ctas = c.num_sms;
   p.group_rows = 16;
-  p.ld = static_cast<int32_t>(Tpad);
   p.scale2 = inv_tau * kLog2e;
   p.inv_tau = inv_tau;
   p.part_m = w.part_m;
@@ -488,8 +484,9 @@ olive_status launch_topk_fwd(const Ctx& c, const void* hidden, const void* W, co
   if ((st = launch_fwd_core<StatsKern>(c, mA, mB, p)) != OLIVE_OK) return st;
 
   const int vt = (V + StatsKern::kBN - 1) / StatsKern::kBN;
-  stats_finalize_kernel<<<c.num_sms * 4, 128, 0, c.stream>>>(
-      n_rows, rows, T, vt, c.num_sms, p.ld, K, inv_tau, w.part_m, w.part_s, w.part_a, w.part_tv,
+  const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
+  stats_finalize_kernel<<<blocks, 128, 0, c.stream>>>(
+      n_rows, rows, T, vt, c.num_sms, K, inv_tau, w.part_m, w.part_s, w.part_a, w.part_tv,
       w.part_ti, lse, entropy, topk_logp, topk_ids);
   return cudaGetLastError() == cudaSuccess ? OLIVE_OK : OLIVE_ERR_CUDA;
 }

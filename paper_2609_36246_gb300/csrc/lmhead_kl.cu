@@ -19,6 +19,7 @@
 //   forward: G = g_t inv_tau (p_s - p_t),   d_h_s = G . W_s
 // comes from one pass of the group kernel (lmhead_group.cu), which recomputes
 // both heads' logits tile by tile and contracts G with W_s on chip.
+#include <algorithm>
 #include <cmath>
 
 #include "gemm_core.cuh"
@@ -53,16 +54,18 @@ struct KlFwdKern {
     uint64_t wait_limit_ns;
     const int32_t* n_rows;
     int32_t T, V, d_s, d_t;
-    int32_t ctas, group_rows, ld, reverse;
+    int32_t ctas, group_rows, reverse;
     float scale2;
-    float* part;  // [5][kSvMax][ld]: m_p, s_p, m_q, s_q, A
+    size_t plane;  // floats of one of the partial arrays
+    float* part;   // [5][plane], [segment][rt 128] each: m_p, s_p, m_q, s_q, A
   };
   struct Sched {
     Split sp;
   };
   static __device__ Sched make_sched(const Params& p) {
     Sched s;
-    s.sp = choose_split(read_n_rows(p.n_rows, p.T, p.dev_status), (p.V + kBN - 1) / kBN, p.ctas);
+    const int n = read_n_rows(p.n_rows, p.T, p.dev_status);
+    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas, split_cap((n + 127) / 128, kMinParts));
     return s;
   }
   static __device__ int num_units(const Params&, const Sched& s) { return s.sp.units; }
@@ -179,8 +182,8 @@ struct KlFwdKern {
       float unused = 0.f;
       merge3(mq, sq, unused, merge[3 * 128 + row], merge[4 * 128 + row], 0.f);
       if (r >= s.sp.n) return;
-      const size_t plane = static_cast<size_t>(kSvMax) * p.ld;
-      const size_t o = static_cast<size_t>(sg) * p.ld + r;
+      const size_t plane = p.plane;
+      const size_t o = static_cast<size_t>(sg) * s.sp.rt * kBM + r;
       p.part[0 * plane + o] = mp;
       p.part[1 * plane + o] = sp;
       p.part[2 * plane + o] = mq;
@@ -192,35 +195,39 @@ struct KlFwdKern {
 
 // kl[t] per masked row; with lse_p / lse_q non-null also both heads' lse per
 // compact row (p the primary head: the student for the reverse KL)
-__global__ void kl_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
-                                   int T, int vt, int ctas, int ld,
-                                   const float* __restrict__ part, float* __restrict__ kl,
-                                   float* __restrict__ lse_p_out, float* __restrict__ lse_q_out) {
-  __shared__ int sh_sv;
+// (one warp a row, its lanes over the row's segments)
+__global__ void __launch_bounds__(128)
+    kl_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
+                       int vt, int ctas, size_t plane, const float* __restrict__ part,
+                       float* __restrict__ kl, float* __restrict__ lse_p_out,
+                       float* __restrict__ lse_q_out) {
   const int n = read_n_rows(n_rows, T, nullptr);
-  if (threadIdx.x == 0) sh_sv = choose_split(n, vt, ctas).sv;
-  __syncthreads();
-  const int sv = sh_sv;
-  const size_t plane = static_cast<size_t>(kSvMax) * ld;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    float Mp = -INFINITY, Mq = -INFINITY;
-    for (int s = 0; s < sv; ++s) {
-      Mp = fmaxf(Mp, part[0 * plane + static_cast<size_t>(s) * ld + r]);
-      Mq = fmaxf(Mq, part[2 * plane + static_cast<size_t>(s) * ld + r]);
+  const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
+  const int lane = threadIdx.x & 31;
+  const size_t ld = static_cast<size_t>(sp.rt) * 128;
+  const int warps = gridDim.x * 4;
+  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
+    float Mp = -INFINITY, Mq = -INFINITY, Sp = 0.f, Sq = 0.f, A = 0.f;
+    float f[2];
+    for (int s = lane; s < sp.sv; s += 32) {
+      const size_t o = s * ld + r;
+      merge_ms(Mp, Sp, part[0 * plane + o], part[1 * plane + o], f);
+      A = A * f[0] + part[4 * plane + o] * f[1];
+      merge_ms(Mq, Sq, part[2 * plane + o], part[3 * plane + o]);
     }
-    float Sp = 0.f, Sq = 0.f, A = 0.f;
-    for (int s = 0; s < sv; ++s) {
-      const size_t o = static_cast<size_t>(s) * ld + r;
-      const float wp = exp2f(part[0 * plane + o] - Mp);
-      Sp += part[1 * plane + o] * wp;
-      A += part[4 * plane + o] * wp;
-      Sq += part[3 * plane + o] * exp2f(part[2 * plane + o] - Mq);
+    for (int o = 16; o > 0; o >>= 1) {
+      const float mp2 = __shfl_xor_sync(0xffffffffu, Mp, o), sp2 = __shfl_xor_sync(0xffffffffu, Sp, o);
+      const float mq2 = __shfl_xor_sync(0xffffffffu, Mq, o), sq2 = __shfl_xor_sync(0xffffffffu, Sq, o);
+      const float a2 = __shfl_xor_sync(0xffffffffu, A, o);
+      merge_ms(Mp, Sp, mp2, sp2, f);
+      A = A * f[0] + a2 * f[1];
+      merge_ms(Mq, Sq, mq2, sq2);
     }
+    if (lane) continue;
     const float lse_p = (Mp + log2f(Sp)) * kLn2;
     const float lse_q = (Mq + log2f(Sq)) * kLn2;
-    const float k = kLn2 * (A / Sp) - lse_p + lse_q;
     const int t = rows[r];
-    if (t >= 0 && t < T) kl[t] = k;
+    if (t >= 0 && t < T) kl[t] = kLn2 * (A / Sp) - lse_p + lse_q;
     if (lse_p_out) {
       lse_p_out[r] = lse_p;
       lse_q_out[r] = lse_q;
@@ -271,16 +278,17 @@ olive_status launch_divergence(const Ctx& c, const void* h_s, const void* W_s, i
   p.d_t = d_t;
   p.ctas = c.num_sms;
   p.group_rows = 16;
-  p.ld = static_cast<int32_t>(Tpad);
+  p.plane = part_rows(Tpad, kMinParts);
   p.reverse = reverse;
   p.scale2 = inv_tau * kLog2e;
   p.part = w.part;
   if ((st = launch_dual<KlFwdKern>(c, mHs, mWs, mHt, mWt, p)) != OLIVE_OK) return st;
 
   const int vt = (V + KlFwdKern::kBN - 1) / KlFwdKern::kBN;
-  kl_finalize_kernel<<<c.num_sms * 4, 256, 0, c.stream>>>(n_rows, rows, T, vt, c.num_sms, p.ld,
-                                                           w.part, kl, grad ? w.lse_p : nullptr,
-                                                           grad ? w.lse_q : nullptr);
+  const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
+  kl_finalize_kernel<<<blocks, 128, 0, c.stream>>>(n_rows, rows, T, vt, c.num_sms, p.plane, w.part, kl,
+                                                    grad ? w.lse_p : nullptr,
+                                                    grad ? w.lse_q : nullptr);
   if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
   if (!grad) return OLIVE_OK;
   // the gradient: G formed from both heads' logits, recomputed tile by tile

@@ -135,8 +135,8 @@ static FwdWs carve_fwd_impl(void* ws, int64_t T, int64_t d, size_t* total) {
   Carver c{static_cast<char*>(ws)};
   FwdWs w;
   w.hc = c.take(2ull * Tpad * d);
-  w.part_m = static_cast<float*>(c.take(4ull * kSvMax * Tpad));
-  w.part_s = static_cast<float*>(c.take(4ull * kSvMax * Tpad));
+  w.part_m = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
+  w.part_s = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
   w.zy = static_cast<float*>(c.take(4ull * Tpad));
   w.nll = static_cast<float*>(c.take(4ull * Tpad));
   if (total) *total = c.off;
@@ -154,11 +154,11 @@ static TopkWs carve_topk_impl(void* ws, int64_t T, int64_t d, size_t* total) {
   Carver c{static_cast<char*>(ws)};
   TopkWs w;
   w.hc = c.take(2ull * Tpad * d);
-  w.part_m = static_cast<float*>(c.take(4ull * kSvMax * Tpad));
-  w.part_s = static_cast<float*>(c.take(4ull * kSvMax * Tpad));
-  w.part_a = static_cast<float*>(c.take(4ull * kSvMax * Tpad));
-  w.part_tv = static_cast<float*>(c.take(4ull * 16 * kSvMax * Tpad));
-  w.part_ti = static_cast<int32_t*>(c.take(4ull * 16 * kSvMax * Tpad));
+  w.part_m = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
+  w.part_s = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
+  w.part_a = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
+  w.part_tv = static_cast<float*>(c.take(4ull * 16 * part_rows(Tpad, kMinParts)));
+  w.part_ti = static_cast<int32_t*>(c.take(4ull * 16 * part_rows(Tpad, kMinParts)));
   if (total) *total = c.off;
   return w;
 }
@@ -193,12 +193,12 @@ BwdWs carve_bwd(void* ws, int64_t T, int64_t d, int64_t V, int grad_dtype) {
 
 static OpdWs carve_opd_impl(void* ws, int64_t T, int64_t ds, int64_t dt, size_t* total) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
-  const size_t lst = 4ull * 16 * kSvMax * Tpad;
+  const size_t lst = 4ull * 16 * part_rows(Tpad, kMinPartsOpd);
   Carver c{static_cast<char*>(ws)};
   OpdWs w;
   w.hcs = c.take(2ull * Tpad * ds);
   w.hct = c.take(2ull * Tpad * dt);
-  w.part = static_cast<float*>(c.take(4ull * 6 * kSvMax * Tpad));
+  w.part = static_cast<float*>(c.take(4ull * 6 * part_rows(Tpad, kMinPartsOpd)));
   w.part_sv = static_cast<float*>(c.take(lst));
   w.part_si = static_cast<int32_t*>(c.take(lst));
   w.part_sx = static_cast<float*>(c.take(lst));
@@ -306,7 +306,7 @@ static KlWs carve_kl_impl(void* ws, int64_t T, int64_t ds, int64_t dt, int64_t V
   KlWs w = {};
   w.hcs = c.take(2ull * Tpad * ds);
   w.hct = c.take(2ull * Tpad * dt);
-  w.part = static_cast<float*>(c.take(4ull * 5 * kSvMax * Tpad));
+  w.part = static_cast<float*>(c.take(4ull * 5 * part_rows(Tpad, kMinParts)));
   if (grad) {
     w.lse_p = static_cast<float*>(c.take(4ull * Tpad));
     w.lse_q = static_cast<float*>(c.take(4ull * Tpad));

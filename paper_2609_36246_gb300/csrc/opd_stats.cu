@@ -25,8 +25,9 @@
 // chunk's registers by a 5-level select tree and the insertion network runs
 // once per candidate, so the network exists in one copy (a copy per column
 // overflows the instruction cache).  Each half writes its own partial, as
-// segment 2 sg + half of the row's vocabulary segment sg (so a row tile has at
-// most kSvMax / 2 segments); opd_finalize_kernel merges them.
+// segment 2 sg + half of the row's vocabulary segment sg; opd_finalize_kernel
+// merges them, one warp a row.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -63,20 +64,22 @@ struct OpdKern {
   static constexpr int kAccBufs = 1;
   static constexpr int kEpiWarps = 8;
   static constexpr int kEpiSmem = 0;
-  static constexpr int kSvCap = kSvMax / 2;  // segments per row tile (x 2 halves)
+  // segments per row tile (each writes two halves)
+  static __device__ int seg_cap(int n) { return split_cap((n + 127) / 128, kMinPartsOpd) / 2; }
 
   struct Params {
     int32_t* dev_status;
     uint64_t wait_limit_ns;
     const int32_t* n_rows;
     int32_t T, V, d_s, d_t;
-    int32_t ctas, group_rows, ld, reverse;
+    int32_t ctas, group_rows, reverse;
     float scale2;
-    float* part;       // [6][kSvMax][ld]: m_s, s_s, E_s, m_t, s_t, A
-    float* part_sv;    // [kSvMax][ld][16] student top raw logits
+    size_t plane;      // floats of one of the partial arrays
+    float* part;       // [6][plane], [2 segment + half][rt 128] each: m_s, s_s, E_s, m_t, s_t, A
+    float* part_sv;    // [2 segment + half][rt 128][16] student top raw logits
     int32_t* part_si;  // their ids
     float* part_sx;    // the teacher's raw logits at those ids
-    float* part_tv;    // [kSvMax][ld][16] teacher top raw logits
+    float* part_tv;    // teacher top raw logits
     int32_t* part_ti;  // their ids
   };
   struct Sched {
@@ -84,8 +87,8 @@ struct OpdKern {
   };
   static __device__ Sched make_sched(const Params& p) {
     Sched s;
-    s.sp = choose_split(read_n_rows(p.n_rows, p.T, p.dev_status), (p.V + kBN - 1) / kBN, p.ctas,
-                        kSvCap);
+    const int n = read_n_rows(p.n_rows, p.T, p.dev_status);
+    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas, seg_cap(n));
     return s;
   }
   static __device__ int num_units(const Params&, const Sched& s) { return s.sp.units; }
@@ -206,8 +209,8 @@ struct OpdKern {
 
     __device__ void end(const Params& p, const Sched& s, int) {
       if (r >= s.sp.n) return;
-      const size_t plane = static_cast<size_t>(kSvMax) * p.ld;
-      const size_t o = static_cast<size_t>(2 * sg + half) * p.ld + r;
+      const size_t plane = p.plane;
+      const size_t o = static_cast<size_t>(2 * sg + half) * s.sp.rt * kBM + r;
       p.part[0 * plane + o] = ms;
       p.part[1 * plane + o] = ss;
       p.part[2 * plane + o] = es;
@@ -236,83 +239,73 @@ struct OpdOut {
   int32_t* s_topk_ids;
 };
 
-__global__ void opd_finalize_kernel(const int32_t* __restrict__ n_rows,
-                                    const int32_t* __restrict__ rows, int T, int vt, int ctas,
-                                    int ld, int reverse, int K, float inv_tau,
-                                    const float* __restrict__ part,
-                                    const float* __restrict__ part_sv,
-                                    const int32_t* __restrict__ part_si,
-                                    const float* __restrict__ part_sx,
-                                    const float* __restrict__ part_tv,
-                                    const int32_t* __restrict__ part_ti, OpdOut out) {
-  __shared__ int sh_sv;
+__global__ void __launch_bounds__(128)
+    opd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
+                        int vt, int ctas, size_t plane, int reverse, int K, float inv_tau,
+                        const float* __restrict__ part, const float* __restrict__ part_sv,
+                        const int32_t* __restrict__ part_si, const float* __restrict__ part_sx,
+                        const float* __restrict__ part_tv, const int32_t* __restrict__ part_ti,
+                        OpdOut out) {
   const int n = read_n_rows(n_rows, T, nullptr);
-  if (threadIdx.x == 0) sh_sv = 2 * choose_split(n, vt, ctas, OpdKern::kSvCap).sv;
-  __syncthreads();
-  const int nsv = sh_sv;  // two halves per vocabulary segment
-  const size_t plane = static_cast<size_t>(kSvMax) * ld;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+  const Split sp = choose_split(n, vt, ctas, OpdKern::seg_cap(n));
+  const int nsv = 2 * sp.sv;  // two halves per vocabulary segment
+  const size_t ld = static_cast<size_t>(sp.rt) * 128;
+  const int lane = threadIdx.x & 31;
+  const int warps = gridDim.x * 4;
+  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
     const int t = rows[r];
     if (t < 0 || t >= T) continue;  // reported by the gather kernel
-    float Ms = -INFINITY, Mt = -INFINITY;
-    for (int s = 0; s < nsv; ++s) {
-      Ms = fmaxf(Ms, part[0 * plane + static_cast<size_t>(s) * ld + r]);
-      Mt = fmaxf(Mt, part[3 * plane + static_cast<size_t>(s) * ld + r]);
+    float Ms = -INFINITY, Mt = -INFINITY, Ss = 0.f, Es = 0.f, St = 0.f, A = 0.f;
+    float fs[2], ft[2];
+    for (int s = lane; s < nsv; s += 32) {
+      const size_t o = s * ld + r;
+      merge_ms(Ms, Ss, part[0 * plane + o], part[1 * plane + o], fs);
+      merge_ms(Mt, St, part[3 * plane + o], part[4 * plane + o], ft);
+      Es = Es * fs[0] + part[2 * plane + o] * fs[1];
+      A = reverse ? A * fs[0] + part[5 * plane + o] * fs[1] : A * ft[0] + part[5 * plane + o] * ft[1];
     }
-    float Ss = 0.f, Es = 0.f, St = 0.f, A = 0.f;
-    float sv[kTopMax], sx[kTopMax], tv[kTopMax];
-    int si[kTopMax], ti[kTopMax];
-#pragma unroll
-    for (int j = 0; j < kTopMax; ++j) {
-      sv[j] = tv[j] = sx[j] = -INFINITY;
-      si[j] = ti[j] = INT_MAX;
-    }
-    for (int s = 0; s < nsv; ++s) {
-      const size_t o = static_cast<size_t>(s) * ld + r;
-      const float ws = exp2f(part[0 * plane + o] - Ms);
-      const float wt = exp2f(part[3 * plane + o] - Mt);
-      Ss += part[1 * plane + o] * ws;
-      Es += part[2 * plane + o] * ws;
-      St += part[4 * plane + o] * wt;
-      A += part[5 * plane + o] * (reverse ? ws : wt);
-      for (int j = 0; j < kTopMax; ++j) {
-        const float cv = part_sv[o * kTopMax + j];
-        const int ci = part_si[o * kTopMax + j];
-        if (topk_beats_last(sv, si, cv, ci)) topk_insert3(sv, si, sx, cv, ci, part_sx[o * kTopMax + j]);
-        const float cw = part_tv[o * kTopMax + j];
-        const int cj = part_ti[o * kTopMax + j];
-        if (topk_beats_last(tv, ti, cw, cj)) topk_insert(tv, ti, cw, cj);
-      }
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ms2 = __shfl_xor_sync(0xffffffffu, Ms, o), ss2 = __shfl_xor_sync(0xffffffffu, Ss, o);
+      const float mt2 = __shfl_xor_sync(0xffffffffu, Mt, o), st2 = __shfl_xor_sync(0xffffffffu, St, o);
+      const float es2 = __shfl_xor_sync(0xffffffffu, Es, o), a2 = __shfl_xor_sync(0xffffffffu, A, o);
+      merge_ms(Ms, Ss, ms2, ss2, fs);
+      merge_ms(Mt, St, mt2, st2, ft);
+      Es = Es * fs[0] + es2 * fs[1];
+      A = reverse ? A * fs[0] + a2 * fs[1] : A * ft[0] + a2 * ft[1];
     }
     const float l2s = Ms + log2f(Ss);
     const float l2t = Mt + log2f(St);
     const float ls = l2s * kLn2, lt = l2t * kLn2;
-    // KL = ln2 A / S_p - lse_p + lse_q
-    const float k = reverse ? kLn2 * (A / Ss) - ls + lt : kLn2 * (A / St) - lt + ls;
-    if (out.kl) out.kl[t] = k;
-    if (out.s_lse) out.s_lse[t] = ls;
-    if (out.t_lse) out.t_lse[t] = lt;
-    if (out.s_entropy) out.s_entropy[t] = kLn2 * (l2s - Es / Ss);
-    int common = 0;
-    float kl_k = 0.f;
-#pragma unroll
-    for (int j = 0; j < kTopMax; ++j) {
-      if (j < K) {
-        const float lps = sv[j] * inv_tau - ls;
-        const float lpt = sx[j] * inv_tau - lt;
-        kl_k += expf(lps) * (lps - lpt);
-        bool hit = false;
-#pragma unroll
-        for (int q = 0; q < kTopMax; ++q) hit |= q < K && ti[q] == si[j];
-        common += hit ? 1 : 0;
-        const size_t oj = static_cast<size_t>(t) * K + j;
-        if (out.s_topk_logp) out.s_topk_logp[oj] = lps;
-        if (out.s_topk_ids) out.s_topk_ids[oj] = si[j];
-        if (out.t_logp_s) out.t_logp_s[oj] = lpt;
-      }
+    if (lane == 0) {
+      // KL = ln2 A / S_p - lse_p + lse_q
+      if (out.kl) out.kl[t] = reverse ? kLn2 * (A / Ss) - ls + lt : kLn2 * (A / St) - lt + ls;
+      if (out.s_lse) out.s_lse[t] = ls;
+      if (out.t_lse) out.t_lse[t] = lt;
+      if (out.s_entropy) out.s_entropy[t] = kLn2 * (l2s - Es / Ss);
     }
-    if (out.overlap) out.overlap[t] = static_cast<float>(common) / static_cast<float>(K);
-    if (out.kl_topk) out.kl_topk[t] = kl_k;
+    float sv, tv;
+    int si, ti;
+    size_t at;
+    warp_top_merge(part_tv, part_ti, nsv, ld, r, K, lane, tv, ti, at);
+    warp_top_merge(part_sv, part_si, nsv, ld, r, K, lane, sv, si, at);
+    bool hit = false;
+    for (int q = 0; q < K; ++q) hit |= __shfl_sync(0xffffffffu, ti, q) == si;
+    const int common = __popc(__ballot_sync(0xffffffffu, lane < K && hit));
+    float term = 0.f;
+    if (lane < K) {
+      const float lps = sv * inv_tau - ls;
+      const float lpt = (si == INT_MAX ? -INFINITY : part_sx[at]) * inv_tau - lt;
+      term = expf(lps) * (lps - lpt);
+      const size_t oj = static_cast<size_t>(t) * K + lane;
+      if (out.s_topk_logp) out.s_topk_logp[oj] = lps;
+      if (out.s_topk_ids) out.s_topk_ids[oj] = si;
+      if (out.t_logp_s) out.t_logp_s[oj] = lpt;
+    }
+    for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xffffffffu, term, o);
+    if (lane == 0) {
+      if (out.overlap) out.overlap[t] = static_cast<float>(common) / static_cast<float>(K);
+      if (out.kl_topk) out.kl_topk[t] = term;
+    }
   }
 }
 
@@ -356,7 +349,7 @@ olive_status launch_opd_stats(const Ctx& c, const void* h_s, const void* W_s, in
   p.d_t = d_t;
   p.ctas = c.num_sms;
   p.group_rows = 16;
-  p.ld = static_cast<int32_t>(Tpad);
+  p.plane = part_rows(Tpad, kMinPartsOpd);
   p.reverse = direction == OLIVE_KL_REVERSE;
   p.scale2 = inv_tau * kLog2e;
   p.part = w.part;
@@ -374,8 +367,9 @@ olive_status launch_opd_stats(const Ctx& c, const void* h_s, const void* W_s, in
 
   const int vt = (V + OpdKern::kBN - 1) / OpdKern::kBN;
   const OpdOut out{kl, s_lse, t_lse, s_entropy, s_topk_logp, t_logp_s, overlap, kl_topk, s_topk_ids};
-  opd_finalize_kernel<<<c.num_sms * 4, 128, 0, c.stream>>>(
-      n_rows, rows, T, vt, c.num_sms, p.ld, p.reverse, K, inv_tau, w.part, w.part_sv, w.part_si,
+  const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
+  opd_finalize_kernel<<<blocks, 128, 0, c.stream>>>(
+      n_rows, rows, T, vt, c.num_sms, p.plane, p.reverse, K, inv_tau, w.part, w.part_sv, w.part_si,
       w.part_sx, w.part_tv, w.part_ti, out);
   return cudaGetLastError() == cudaSuccess ? OLIVE_OK : OLIVE_ERR_CUDA;
 }

@@ -7,9 +7,12 @@
 // unit is one (row tile, segment); its partial (max, sum) per row is merged by
 // the finalize kernel.  sv is chosen to minimise the critical path
 // ceil(units / ctas) * seg, which removes most of the wave-quantisation loss
-// when rt is small compared with the SM count.
+// when rt is small compared with the SM count.  One or two row tiles may be cut
+// into more than kSvMax segments, as many as fill the SMs: with 64, 96 rows of
+// d = 4096 ran on 60 SMs (276 us over V = 151936).
 #pragma once
 
+#include <climits>
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -25,25 +28,42 @@ struct Split {
   int units; // rt * sv
 };
 
-__host__ __device__ inline Split choose_split(int n, int vt, int ctas, int sv_cap = kSvMax) {
+// Segments a row tile may be cut into when there are rt of them; `parts` is
+// the least number of (row tile, segment) partials the workspace holds.
+__device__ inline int split_cap(int rt, int parts) {
+  return rt > 0 ? max(kSvMax, parts / rt) : kSvMax;
+}
+
+// Every lane of a warp: the decomposition of n rows over vt vocabulary tiles
+// for `ctas` CTAs, at most sv_cap segments (a lane tries every 32nd count; on
+// one thread the search took several microseconds of each kernel that needs
+// it).
+__device__ inline Split choose_split(int n, int vt, int ctas, int sv_cap) {
   Split s;
   s.n = n;
   s.rt = (n + 127) / 128;
   s.vt = vt;
   int best_sv = 1;
-  long long best_cost = -1;
-  const int max_sv = vt < sv_cap ? vt : sv_cap;
-  for (int sv = 1; sv <= max_sv; ++sv) {
+  long long best_cost = LLONG_MAX;
+  const int max_sv = min(vt, sv_cap);
+  for (int sv = static_cast<int>(threadIdx.x & 31) + 1; sv <= max_sv; sv += 32) {
     const int seg = (vt + sv - 1) / sv;
-    const int sv_eff = (vt + seg - 1) / seg;
-    if (sv_eff != sv) continue;
-    const long long units = static_cast<long long>(s.rt) * sv;
-    const long long waves = (units + ctas - 1) / ctas;
+    if ((vt + seg - 1) / seg != sv) continue;
+    const uint32_t units = static_cast<uint32_t>(s.rt) * static_cast<uint32_t>(sv);
+    const uint32_t waves = (units + static_cast<uint32_t>(ctas) - 1) / static_cast<uint32_t>(ctas);
     // a unit also pays a pipeline fill and a partial write: ~1/8 tile
-    const long long cost = waves * (8LL * seg + 1);
-    if (best_cost < 0 || cost < best_cost) {
+    const long long cost = static_cast<long long>(waves) * (8LL * seg + 1);
+    if (cost < best_cost) {
       best_cost = cost;
       best_sv = sv;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long c = __shfl_xor_sync(0xffffffffu, best_cost, o);
+    const int v = __shfl_xor_sync(0xffffffffu, best_sv, o);
+    if (c < best_cost || (c == best_cost && v < best_sv)) {
+      best_cost = c;
+      best_sv = v;
     }
   }
   s.sv = best_sv;
@@ -75,6 +95,20 @@ __device__ inline int read_n_rows(const int32_t* n_rows, int T, int32_t* dev_sta
     n = n < 0 ? 0 : T;
   }
   return n;
+}
+
+// (m, s) + (m2, s2): a base-2 maximum and the sum of 2^(x - m); an empty side
+// (m = -inf) adds nothing.  w receives the factors applied to each side.
+__device__ __forceinline__ void merge_ms(float& m, float& s, float m2, float s2, float* w = nullptr) {
+  const float mn = fmaxf(m, m2);
+  const float f1 = m == -INFINITY ? 0.f : exp2f(m - mn);
+  const float f2 = m2 == -INFINITY ? 0.f : exp2f(m2 - mn);
+  s = s * f1 + s2 * f2;
+  m = mn;
+  if (w) {
+    w[0] = f1;
+    w[1] = f2;
+  }
 }
 
 }  // namespace olive

@@ -208,3 +208,50 @@ def test_constant_column_shift_invariance():
     assert np.abs((s1[r] - s0[r]) - 24.0).max() <= 1e-4
     assert np.linalg.norm(dh1[:, :63] - dh0[:, :63]) <= 2e-2 * np.linalg.norm(dh0[:, :63])
     assert np.linalg.norm(dw1[:, :63] - dw0[:, :63]) <= 2e-2 * np.linalg.norm(dw0[:, :63])
+
+
+@pytest.mark.parametrize("n", [1, 100, 129, 256, 257, 400])
+def test_few_rows_many_segments(n):
+    """One to four row tiles over a vocabulary of 240 tiles, which are cut into
+    more than 64 segments at one or two: log-probs, top lists, entropy and the
+    dual sweeps' values against fp64."""
+    rng = np.random.default_rng(n)
+    V, d, K = 61300, 64, 16
+    b = synth.batch_from_lengths(rng, [2], [n], V)
+    h = synth.normal_bf16(rng, (b.T, d), 1.0)
+    W = synth.normal_bf16(rng, (V, d), 0.3)
+    ht = synth.normal_bf16(rng, (b.T, d), 1.0)
+    Wt = synth.normal_bf16(rng, (V, d), 0.3)
+    g = gpu_pack(b)
+    hc, Wc, htc, Wtc = h.cuda(), W.cuda(), ht.cuda(), Wt.cuda()
+    rows, nr, st = g["rows"], g["n_rows"], g["dev_status"]
+    logp, lse, _ = B.olive_token_logprob_fwd(hc, Wc, g["targets"], rows, nr, dev_status=st)
+    lse2, ent, tv, ti = B.olive_token_topk_fwd(hc, Wc, rows, nr, K, dev_status=st)
+    opd = B.olive_opd_token_stats(hc, Wc, htc, Wtc, rows, nr, K, dev_status=st)
+    kl, _ = B.olive_token_divergence(hc, Wc, htc, Wtc, rows, nr, dev_status=st)
+    torch.cuda.synchronize()
+    assert B.status_bits(st) == []
+    r = rows[:n].long()
+    l = torch.log_softmax(hc[r].double() @ Wc.double().t(), 1)
+    lt = torch.log_softmax(htc[r].double() @ Wtc.double().t(), 1)
+    y = g["targets"][r].long()[:, None]
+    want_v, want_i = l.topk(K, 1)
+    want_kl = (l.exp() * (l - lt)).sum(1)
+    # fp32 sums of 64 products and of 61300 exponentials: 2e-5 of a value near 10
+    close = lambda a, b: torch.testing.assert_close(a.double(), b, rtol=2e-5, atol=2e-4)
+    close(logp[r], l.gather(1, y)[:, 0])
+    close(lse2[r], lse[r].double())
+    close(ent[r], -(l.exp() * l).sum(1))
+    close(tv[r], want_v)
+    close(opd["s_topk_logp"][r], want_v)
+    close(opd["kl"][r], want_kl)
+    close(kl[r], want_kl)
+    # ids where neighbours are further apart than the fp32 error
+    gap = (want_v[:, :-1] - want_v[:, 1:]) > 1e-3
+    sure = torch.ones_like(want_i, dtype=torch.bool)
+    sure[:, :-1] &= gap
+    sure[:, 1:] &= gap
+    sure[:, -1] = False
+    for ids in (ti[r], opd["s_topk_ids"][r]):
+        assert torch.equal(ids.long()[sure], want_i[sure])
+    close(opd["t_logp_s"][r][sure], lt.gather(1, want_i)[sure])
