@@ -67,8 +67,8 @@ struct FwdWs {
   float* zy;      // [Tpad]
   float* nll;     // [Tpad]
 };
-size_t fwd_ws_bytes(int64_t T, int64_t d);
-FwdWs carve_fwd(void* ws, int64_t T, int64_t d);
+size_t fwd_ws_bytes(int64_t T, int64_t d, int min_parts = kMinParts);
+FwdWs carve_fwd(void* ws, int64_t T, int64_t d, int min_parts = kMinParts);
 
 struct TopkWs {
   void* hc;          // bf16 [Tpad, d]
@@ -201,7 +201,7 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
                           int32_t d, int32_t V, const GroupArgs& a, int c_base, int c_end,
                           uint32_t* ring_ctr);
 // The divergence gradient on chip: d_h_s = G . W_s with G from both heads'
-// logits (recomputed tile by tile by groups of CTA pairs) and the value sweep's kl, lse_s, lse_t; ctr (ctr_words) is zeroed here.
+// logits (recomputed tile by tile by groups of CTA pairs) and the value sweep's kl, lse_s, lse_t.
 olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct, const void* W_s,
                                   int32_t d_s, const void* W_t, int32_t d_t, const int32_t* rows,
                                   const int32_t* n_rows, int32_t T, int32_t V, float inv_tau,
@@ -236,17 +236,41 @@ olive_status launch_splice_pack_masked(const Ctx& c, const int32_t* prefix_ids,
                                        int32_t* cut_offsets, int32_t* rows, int32_t* n_rows,
                                        void* ws, int32_t* dev_status);
 
-// Copies hidden[rows[r]] to hc[r] for r < n_rows and zero-fills the rest of
-// the last 128-row tile.
-olive_status launch_gather_rows(const Ctx& c, const void* hidden, const int32_t* rows,
-                                const int32_t* n_rows, int32_t T, int32_t d, void* hc,
-                                int32_t* dev_status);
+// What a call does before its sweeps, as one launch: copies of masked rows
+// (hidden[rows[r]] to hc[r] for r < n_rows, the rest of the last 128-row tile
+// zero) and buffers filled with one byte value (sizes multiples of 4, bases
+// 4-byte aligned).
+struct Prepare {
+  static constexpr int kMaxFills = 12;
+  const void* src[2];
+  void* hc[2];
+  int32_t d[2];
+  int n_src = 0;
+  void* ptr[kMaxFills];
+  size_t bytes[kMaxFills];
+  int value[kMaxFills];
+  int n_fill = 0;
+  void gather(const void* hidden, int32_t width, void* to) {
+    src[n_src] = hidden;
+    d[n_src] = width;
+    hc[n_src++] = to;
+  }
+  // (null: nothing to fill)
+  void fill(void* p, size_t n, int v = 0) {
+    if (!p || n == 0) return;
+    ptr[n_fill] = p;
+    bytes[n_fill] = n;
+    value[n_fill++] = v;
+  }
+};
+olive_status launch_prepare(const Ctx& c, const Prepare& q, const int32_t* rows,
+                            const int32_t* n_rows, int32_t T, int32_t* dev_status);
 
 olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
                                 const int32_t* targets, const int32_t* rows, const int32_t* n_rows,
                                 int32_t T, int32_t d, int32_t V, float inv_tau, int reduction,
                                 float* logp, float* lse, float* loss, void* ws,
-                                int32_t* dev_status);
+                                int32_t* dev_status, int min_parts = kMinParts);
 
 // y = x * (*scale) on n bf16 or fp32 elements (x == y allowed).
 olive_status launch_scale(const Ctx& c, const void* x, void* y, size_t n, int dtype,

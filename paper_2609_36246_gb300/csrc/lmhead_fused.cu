@@ -1297,12 +1297,12 @@ olive_status launch_loss_bwd(const Ctx& c, const void* hidden, const void* W,
   const int64_t ldg = vpad(V);
   const size_t elt = grad_dtype == OLIVE_DTYPE_BF16 ? 2 : 4;
 
-  olive_status st = launch_gather_rows(c, hidden, rows, n_rows, T, d, w.hc, dev_status);
+  Prepare q;
+  q.gather(hidden, d, w.hc);
+  q.fill(d_hidden, elt * T * static_cast<size_t>(d));
+  q.fill(w.counters, 4 * bwd_counter_words(Tpad, w.tc));
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(d_hidden, 0, elt * T * static_cast<size_t>(d), c.stream) != cudaSuccess)
-    return OLIVE_ERR_CUDA;
-  const size_t nctr = bwd_counter_words(Tpad, w.tc);
-  if (cudaMemsetAsync(w.counters, 0, 4 * nctr, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
 
   FusedMaps maps;
   if (!encode_bf16_2d(&maps.m[0], w.hc, d, Tpad, 2ull * d, 64, 128) ||
@@ -1350,12 +1350,13 @@ olive_status launch_loss_fwd_bwd(const Ctx& c, const void* hidden, const void* W
   const size_t elt = grad_dtype == OLIVE_DTYPE_BF16 ? 2 : 4;
   const int vh = static_cast<int>(ceil_div(V, kHalf));
 
-  olive_status st = launch_gather_rows(c, hidden, rows, n_rows, T, d, w.hc, dev_status);
+  Prepare q;
+  q.gather(hidden, d, w.hc);
+  q.fill(d_hidden, elt * T * static_cast<size_t>(d));
+  q.fill(logp, sizeof(float) * T);
+  q.fill(lse, sizeof(float) * T);
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(d_hidden, 0, elt * T * static_cast<size_t>(d), c.stream) != cudaSuccess ||
-      cudaMemsetAsync(logp, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(lse, 0, sizeof(float) * T, c.stream) != cudaSuccess)
-    return OLIVE_ERR_CUDA;
 
   FusedMaps maps;
   if (!encode_bf16_2d(&maps.m[0], w.hc, d, Tpad, 2ull * d, 64, 128) ||
@@ -1425,16 +1426,17 @@ olive_status launch_topk_kl_fwd_bwd(const Ctx& c, const void* h_s, const void* W
   const int vh = static_cast<int>(ceil_div(V, kHalf));
   const size_t tk = static_cast<size_t>(T) * K;
 
-  olive_status st = launch_gather_rows(c, h_s, rows, n_rows, T, d_s, w.hc, dev_status);
+  Prepare q;
+  q.gather(h_s, d_s, w.hc);
+  q.fill(d_h_s, elt * T * static_cast<size_t>(d_s));
+  q.fill(s_lse, sizeof(float) * T);
+  q.fill(kl_topk, sizeof(float) * T);
+  q.fill(overlap, sizeof(float) * T);
+  q.fill(s_logp, sizeof(float) * tk);
+  q.fill(t_logp_s, sizeof(float) * tk);
+  q.fill(s_ids, sizeof(int32_t) * tk, 0xff);
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(d_h_s, 0, elt * T * static_cast<size_t>(d_s), c.stream) != cudaSuccess ||
-      cudaMemsetAsync(s_lse, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(kl_topk, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      (overlap && cudaMemsetAsync(overlap, 0, sizeof(float) * T, c.stream) != cudaSuccess) ||
-      cudaMemsetAsync(s_logp, 0, sizeof(float) * tk, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(t_logp_s, 0, sizeof(float) * tk, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(s_ids, 0xff, sizeof(int32_t) * tk, c.stream) != cudaSuccess)
-    return OLIVE_ERR_CUDA;
 
   FusedMaps maps;
   if (!encode_bf16_2d(&maps.m[0], w.hc, d_s, Tpad, 2ull * d_s, 64, 128) ||

@@ -52,6 +52,7 @@ struct FwdKernT {
     int32_t T, d, V;
     int32_t ctas;        // CTAs the decomposition is computed for (= grid)
     int32_t group_rows;  // row tiles per raster group
+    int32_t min_parts;   // partials the workspace holds at least
     float scale2;        // inv_tau * log2(e): logits in base-2 units
     float inv_tau;
     float* part_m;
@@ -68,7 +69,8 @@ struct FwdKernT {
   static __device__ Sched make_sched(const Params& p) {
     Sched s;
     const int n = read_n_rows(p.n_rows, p.T, p.dev_status);
-    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas, split_cap((n + 127) / 128, kMinParts));
+    s.sp = choose_split(n, (p.V + kBN - 1) / kBN, p.ctas,
+                        split_cap((n + 127) / 128, p.min_parts));
     return s;
   }
   static __device__ int num_units(const Params&, const Sched& s) { return s.sp.units; }
@@ -238,14 +240,34 @@ struct FwdKernT {
 using FwdKern = FwdKernT<false>;
 using StatsKern = FwdKernT<true>;
 
-__global__ void gather_rows_kernel(const uint4* __restrict__ hidden, const int32_t* __restrict__ rows,
-                                   const int32_t* __restrict__ n_rows, int T, int d8,
-                                   uint4* __restrict__ hc, int32_t* dev_status) {
+// The copies and fills of a call's start (Prepare) in one launch: up to 11
+// launches and memsets of the larger calls, each 2 to 5 us where little else
+// runs (the 300-row step of d = 256 began with 5).  Fills take 16 bytes a
+// thread from the first 16-byte boundary on, 4 at the ragged ends.
+__global__ void __launch_bounds__(256)
+    prepare_kernel(const Prepare q, const int32_t* __restrict__ rows,
+                   const int32_t* __restrict__ n_rows, int T, int32_t* dev_status) {
+  const size_t tid = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const size_t all = static_cast<size_t>(gridDim.x) * blockDim.x;
+  for (int f = 0; f < q.n_fill; ++f) {
+    const uint32_t w = (q.value[f] & 0xff) * 0x01010101u;
+    uint8_t* base = static_cast<uint8_t*>(q.ptr[f]);
+    const size_t bytes = q.bytes[f];
+    size_t head = (16 - (reinterpret_cast<uintptr_t>(base) & 15)) & 15;
+    if (head > bytes) head = bytes;
+    const size_t vecs = (bytes - head) / 16;
+    uint4* v = reinterpret_cast<uint4*>(base + head);
+    for (size_t i = tid; i < vecs; i += all) v[i] = make_uint4(w, w, w, w);
+    const size_t tail = head + vecs * 16;
+    if (tid < head / 4) reinterpret_cast<uint32_t*>(base)[tid] = w;
+    if (tid < (bytes - tail) / 4) reinterpret_cast<uint32_t*>(base + tail)[tid] = w;
+  }
+  if (q.n_src == 0) return;
   const int n = read_n_rows(n_rows, T, dev_status);
   const int npad = (n + 127) / 128 * 128;
   const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < npad; r += warps) {
+  const int warps = static_cast<int>(all >> 5);
+  for (int r = static_cast<int>(tid >> 5); r < npad; r += warps) {
     int t = -1;
     if (r < n) {
       t = rows[r];
@@ -254,12 +276,12 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, const int32
         t = -1;
       }
     }
-    uint4* dst = hc + static_cast<size_t>(r) * d8;
-    if (t >= 0) {
-      const uint4* src = hidden + static_cast<size_t>(t) * d8;
-      for (int c = lane; c < d8; c += 32) dst[c] = __ldg(src + c);
-    } else {
-      for (int c = lane; c < d8; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
+    for (int s = 0; s < q.n_src; ++s) {
+      const int d8 = q.d[s] / 8;
+      uint4* dst = static_cast<uint4*>(q.hc[s]) + static_cast<size_t>(r) * d8;
+      const uint4* src = static_cast<const uint4*>(q.src[s]) + static_cast<size_t>(t < 0 ? 0 : t) * d8;
+#pragma unroll 4
+      for (int c = lane; c < d8; c += 32) dst[c] = t >= 0 ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
     }
   }
 }
@@ -268,12 +290,12 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ hidden, const int32
 // up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
 __global__ void __launch_bounds__(128)
     fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
-                        const int32_t* __restrict__ targets, int T, int V, int vt, int ctas,
+                        const int32_t* __restrict__ targets, int T, int V, int vt, int ctas, int min_parts,
                         const float* __restrict__ part_m, const float* __restrict__ part_s,
                         const float* __restrict__ zy, float* __restrict__ logp,
                         float* __restrict__ lse, float* __restrict__ nll, int32_t* dev_status) {
   const int n = read_n_rows(n_rows, T, nullptr);
-  const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
+  const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, min_parts));
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
   const int warps = gridDim.x * 4;
@@ -384,13 +406,35 @@ olive_status launch_fwd_core(const Ctx& c, const CUtensorMap& a, const CUtensorM
 
 }  // namespace
 
-olive_status launch_gather_rows(const Ctx& c, const void* hidden, const int32_t* rows,
-                                const int32_t* n_rows, int32_t T, int32_t d, void* hc,
-                                int32_t* dev_status) {
-  const int blocks = c.num_sms * 8;
-  gather_rows_kernel<<<blocks, 256, 0, c.stream>>>(static_cast<const uint4*>(hidden), rows, n_rows,
-                                                    T, d / 8, static_cast<uint4*>(hc), dev_status);
-  return cudaGetLastError() == cudaSuccess ? OLIVE_OK : OLIVE_ERR_CUDA;
+olive_status launch_prepare(const Ctx& c, const Prepare& q, const int32_t* rows,
+                            const int32_t* n_rows, int32_t T, int32_t* dev_status) {
+  // a fill that overlaps a copy's source (a gradient written over its input)
+  // has to come after the copy
+  Prepare now = q, later;
+  now.n_fill = 0;
+  size_t work = 0;
+  for (int f = 0; f < q.n_fill; ++f) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(q.ptr[f]), e = a + q.bytes[f];
+    bool over = false;
+    for (int s = 0; s < q.n_src; ++s) {
+      const uintptr_t b = reinterpret_cast<uintptr_t>(q.src[s]);
+      over = over || (a < b + 2ull * T * q.d[s] && b < e);
+    }
+    const uintptr_t b = reinterpret_cast<uintptr_t>(rows);
+    over = over || (a < b + 4ull * T && b < e);
+    (over ? later : now).fill(q.ptr[f], q.bytes[f], q.value[f]);
+    work += q.bytes[f];
+  }
+  for (int s = 0; s < q.n_src; ++s) work += 4ull * T * q.d[s];
+  // about 16 KB a block of 256 threads, at most 8 blocks an SM
+  const int blocks = static_cast<int>(
+      std::max<int64_t>(1, std::min<int64_t>(ceil_div(static_cast<int64_t>(work), 16384), c.num_sms * 8)));
+  prepare_kernel<<<blocks, 256, 0, c.stream>>>(now, rows, n_rows, T, dev_status);
+  if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
+  for (int f = 0; f < later.n_fill; ++f)
+    if (cudaMemsetAsync(later.ptr[f], later.value[f], later.bytes[f], c.stream) != cudaSuccess)
+      return OLIVE_ERR_CUDA;
+  return OLIVE_OK;
 }
 
 olive_status launch_loss_reduce(const Ctx& c, const int32_t* n_rows, int32_t T, const float* nll,
@@ -403,13 +447,15 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
                                 const int32_t* targets, const int32_t* rows, const int32_t* n_rows,
                                 int32_t T, int32_t d, int32_t V, float inv_tau, int reduction,
                                 float* logp, float* lse, float* loss, void* ws,
-                                int32_t* dev_status) {
+                                int32_t* dev_status, int min_parts) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
-  const FwdWs w = carve_fwd(ws, T, d);
-  olive_status st = launch_gather_rows(c, hidden, rows, n_rows, T, d, w.hc, dev_status);
+  const FwdWs w = carve_fwd(ws, T, d, min_parts);
+  Prepare q;
+  q.gather(hidden, d, w.hc);
+  q.fill(logp, sizeof(float) * T);
+  q.fill(lse, sizeof(float) * T);
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(logp, 0, sizeof(float) * T, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
-  if (cudaMemsetAsync(lse, 0, sizeof(float) * T, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
 
   CUtensorMap mA, mB;
   if (!encode_bf16_2d(&mA, w.hc, d, Tpad, 2ull * d, 64, 128)) return OLIVE_ERR_CUDA;
@@ -431,11 +477,12 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
   p.part_m = w.part_m;
   p.part_s = w.part_s;
   p.zy = w.zy;
+  p.min_parts = min_parts;
   if ((st = launch_fwd_core<FwdKern>(c, mA, mB, p)) != OLIVE_OK) return st;
 
   const int vt = (V + FwdKern::kBN - 1) / FwdKern::kBN;
   const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
-  fwd_finalize_kernel<<<blocks, 128, 0, c.stream>>>(n_rows, rows, targets, T, V, vt, c.num_sms,
+  fwd_finalize_kernel<<<blocks, 128, 0, c.stream>>>(n_rows, rows, targets, T, V, vt, c.num_sms, min_parts,
                                                      w.part_m, w.part_s, w.zy, logp, lse, w.nll,
                                                      dev_status);
   if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
@@ -450,15 +497,15 @@ olive_status launch_topk_fwd(const Ctx& c, const void* hidden, const void* W, co
                              int32_t* topk_ids, void* ws, int32_t* dev_status) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
   const TopkWs w = carve_topk(ws, T, d);
-  olive_status st = launch_gather_rows(c, hidden, rows, n_rows, T, d, w.hc, dev_status);
+  const size_t tk = sizeof(float) * T * static_cast<size_t>(K);
+  Prepare q;
+  q.gather(hidden, d, w.hc);
+  q.fill(lse, sizeof(float) * T);
+  q.fill(entropy, sizeof(float) * T);
+  q.fill(topk_logp, tk);
+  q.fill(topk_ids, tk, 0xff);
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(lse, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(entropy, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(topk_logp, 0, sizeof(float) * T * static_cast<size_t>(K), c.stream) !=
-          cudaSuccess ||
-      cudaMemsetAsync(topk_ids, 0xff, sizeof(int32_t) * T * static_cast<size_t>(K), c.stream) !=
-          cudaSuccess)
-    return OLIVE_ERR_CUDA;
 
   CUtensorMap mA, mB;
   if (!encode_bf16_2d(&mA, w.hc, d, Tpad, 2ull * d, 64, 128)) return OLIVE_ERR_CUDA;
@@ -481,6 +528,7 @@ olive_status launch_topk_fwd(const Ctx& c, const void* hidden, const void* W, co
   p.part_a = w.part_a;
   p.part_tv = w.part_tv;
   p.part_ti = w.part_ti;
+  p.min_parts = kMinParts;
   if ((st = launch_fwd_core<StatsKern>(c, mA, mB, p)) != OLIVE_OK) return st;
 
   const int vt = (V + StatsKern::kBN - 1) / StatsKern::kBN;

@@ -480,6 +480,10 @@ __device__ void pace_wait(const uint32_t* pace, int ngroups, int need, int lane)
 template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1)
     lmhead_group_kernel(const __grid_constant__ GroupMaps maps, const GroupParams p) {
+  // the redo launch mostly has nothing to do: it leaves before any barrier or
+  // TMEM is set up (the same decision in every CTA)
+  if (kMode == GM_A && p.redo && p.redo_list[0] == 0) return;
+
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   uint8_t* gbase = smem_raw;
@@ -1559,14 +1563,16 @@ olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,
   const bool fwd = lse_given == nullptr;
   const GroupWs w = carve_group(ws, T, d, V);
   const size_t elt = grad_dtype == OLIVE_DTYPE_BF16 ? 2 : 4;
-  olive_status st = launch_gather_rows(c, hidden, rows, n_rows, T, d, w.hc, dev_status);
+  Prepare q;
+  q.gather(hidden, d, w.hc);
+  q.fill(d_hidden, elt * T * static_cast<size_t>(d));
+  q.fill(w.outer, 4 * w.ctr_words);
+  if (fwd) {
+    q.fill(logp, sizeof(float) * T);
+    q.fill(lse, sizeof(float) * T);
+  }
+  olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
-  if (cudaMemsetAsync(d_hidden, 0, elt * T * static_cast<size_t>(d), c.stream) != cudaSuccess ||
-      cudaMemsetAsync(w.outer, 0, 4 * w.ctr_words, c.stream) != cudaSuccess)
-    return OLIVE_ERR_CUDA;
-  if (fwd && (cudaMemsetAsync(logp, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-              cudaMemsetAsync(lse, 0, sizeof(float) * T, c.stream) != cudaSuccess))
-    return OLIVE_ERR_CUDA;
 
   GroupArgs a = {};
   a.dev_status = dev_status;
@@ -1655,7 +1661,7 @@ olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct
   const int cols = group_sweep_cols(c.num_sms);
   for (int cb = 0; cb < d_s; cb += cols) {
     const int ce = d_s - cb < cols ? d_s : cb + cols;
-    if (cudaMemsetAsync(ctr, 0, 4 * ctr_words, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
+    if (cb > 0 && cudaMemsetAsync(ctr, 0, 4 * ctr_words, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
     const olive_status st = launch_group(c, GM_KL, hcs, W_s, T, d_s, V, a, cb, ce, ring_ctr);
     if (st != OLIVE_OK) return st;
   }

@@ -257,10 +257,16 @@ olive_status launch_divergence(const Ctx& c, const void* h_s, const void* W_s, i
   const int grad = d_h_s != nullptr;
   const KlWs w = carve_kl(ws, T, d_s, d_t, V, grad);
   const int reverse = direction == OLIVE_KL_REVERSE;
+  Prepare q;
+  q.gather(h_s, d_s, w.hcs);
+  q.gather(h_t, d_t, w.hct);
+  q.fill(kl, sizeof(float) * T);
+  if (grad) {
+    q.fill(d_h_s, (grad_dtype == OLIVE_DTYPE_BF16 ? 2ull : 4ull) * T * d_s);
+    q.fill(w.ctr, 4 * w.ctr_words);
+  }
   olive_status st;
-  if ((st = launch_gather_rows(c, h_s, rows, n_rows, T, d_s, w.hcs, dev_status)) != OLIVE_OK) return st;
-  if ((st = launch_gather_rows(c, h_t, rows, n_rows, T, d_t, w.hct, dev_status)) != OLIVE_OK) return st;
-  if (cudaMemsetAsync(kl, 0, sizeof(float) * T, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
+  if ((st = launch_prepare(c, q, rows, n_rows, T, dev_status)) != OLIVE_OK) return st;
 
   CUtensorMap mHs, mWs, mHt, mWt;
   if (!encode_bf16_2d(&mHs, w.hcs, d_s, Tpad, 2ull * d_s, 64, 128)) return OLIVE_ERR_CUDA;
@@ -294,9 +300,6 @@ olive_status launch_divergence(const Ctx& c, const void* h_s, const void* W_s, i
   // the gradient: G formed from both heads' logits, recomputed tile by tile
   // and exchanged on chip (lmhead_group.cu); the student's lse is the
   // primary head's for the reverse KL, the other one's for the forward KL
-  const size_t elt = grad_dtype == OLIVE_DTYPE_BF16 ? 2 : 4;
-  if (cudaMemsetAsync(d_h_s, 0, elt * T * static_cast<size_t>(d_s), c.stream) != cudaSuccess)
-    return OLIVE_ERR_CUDA;
   return launch_kl_group_grad(c, w.hcs, w.hct, W_s, d_s, W_t, d_t, rows, n_rows, T, V, inv_tau,
                               reverse, kl, reverse ? w.lse_p : w.lse_q, reverse ? w.lse_q : w.lse_p,
                               grad_kl, d_h_s, grad_dtype, w.ring, w.tail_acc, w.ctr, w.ctr_words,

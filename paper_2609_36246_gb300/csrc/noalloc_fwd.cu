@@ -70,8 +70,10 @@ extern "C" OLIVE_API olive_status olive_token_logprob_fwd_noalloc(
   if (!(inv_tau > 0.f) || !std::isfinite(inv_tau)) return OLIVE_ERR_INVALID_ARG;
   if (T < 1 || V < 1 || d < 1 || d > (1 << 20)) return OLIVE_ERR_SHAPE;
   if (d % 8 != 0 || !is_aligned16(hidden) || !is_aligned16(W)) return OLIVE_ERR_ALIGNMENT;
-  // the whole scratch of this call must fit the fixed array
-  if (fwd_ws_bytes(T, d) > kNoallocScratchBytes) return OLIVE_ERR_SHAPE;
+  // the whole scratch of this call must fit the fixed array, if need be with
+  // no more segments for one or two row tiles than for many
+  const int parts = fwd_ws_bytes(T, d) <= kNoallocScratchBytes ? kMinParts : 0;
+  if (fwd_ws_bytes(T, d, parts) > kNoallocScratchBytes) return OLIVE_ERR_SHAPE;
   Ctx c;
   olive_status st = make_ctx(stream, &c);
   if (st != OLIVE_OK) return st;
@@ -79,5 +81,5 @@ extern "C" OLIVE_API olive_status olive_token_logprob_fwd_noalloc(
   st = scratch_address(c.device, &ws);
   if (st != OLIVE_OK) return st;
   return launch_logprob_fwd(c, hidden, W, targets, rows, n_rows, T, d, V, inv_tau, reduction,
-                            logp, lse, loss, ws, dev_status);
+                            logp, lse, loss, ws, dev_status, parts);
 }

@@ -49,14 +49,22 @@ olive_status make_ctx(void* stream, Ctx* ctx) {
     cudaGetLastError();
     return OLIVE_ERR_CUDA;
   }
-  int major = 0, minor = 0, sms = 0;
-  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return OLIVE_ERR_CUDA;
+  // SMs of a device of the right capability, + 1 (a device's attributes do not
+  // change; 0: not asked yet)
+  static std::atomic<int> known[kMaxDevices];
+  const bool cached = dev >= 0 && dev < kMaxDevices;
+  int sms = cached ? known[dev].load(std::memory_order_acquire) - 1 : -1;
+  if (sms < 0) {
+    int major = 0, minor = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return OLIVE_ERR_CUDA;
+    }
+    if (major != 10 || minor != 3) return OLIVE_ERR_UNSUPPORTED_DEVICE;
+    if (cached) known[dev].store(sms + 1, std::memory_order_release);
   }
-  if (major != 10 || minor != 3) return OLIVE_ERR_UNSUPPORTED_DEVICE;
   if (!encode_fn()) return OLIVE_ERR_CUDA;
   ctx->stream = static_cast<cudaStream_t>(stream);
   ctx->device = dev;
@@ -130,24 +138,26 @@ struct Carver {
 };
 }  // namespace
 
-static FwdWs carve_fwd_impl(void* ws, int64_t T, int64_t d, size_t* total) {
+static FwdWs carve_fwd_impl(void* ws, int64_t T, int64_t d, int min_parts, size_t* total) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
   Carver c{static_cast<char*>(ws)};
   FwdWs w;
   w.hc = c.take(2ull * Tpad * d);
-  w.part_m = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
-  w.part_s = static_cast<float*>(c.take(4ull * part_rows(Tpad, kMinParts)));
+  w.part_m = static_cast<float*>(c.take(4ull * part_rows(Tpad, min_parts)));
+  w.part_s = static_cast<float*>(c.take(4ull * part_rows(Tpad, min_parts)));
   w.zy = static_cast<float*>(c.take(4ull * Tpad));
   w.nll = static_cast<float*>(c.take(4ull * Tpad));
   if (total) *total = c.off;
   return w;
 }
-size_t fwd_ws_bytes(int64_t T, int64_t d) {
+size_t fwd_ws_bytes(int64_t T, int64_t d, int min_parts) {
   size_t n = 0;
-  carve_fwd_impl(nullptr, T, d, &n);
+  carve_fwd_impl(nullptr, T, d, min_parts, &n);
   return n;
 }
-FwdWs carve_fwd(void* ws, int64_t T, int64_t d) { return carve_fwd_impl(ws, T, d, nullptr); }
+FwdWs carve_fwd(void* ws, int64_t T, int64_t d, int min_parts) {
+  return carve_fwd_impl(ws, T, d, min_parts, nullptr);
+}
 
 static TopkWs carve_topk_impl(void* ws, int64_t T, int64_t d, size_t* total) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);

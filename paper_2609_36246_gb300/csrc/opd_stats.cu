@@ -320,17 +320,16 @@ olive_status launch_opd_stats(const Ctx& c, const void* h_s, const void* W_s, in
                               int32_t* dev_status) {
   const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
   const OpdWs w = carve_opd(ws, T, d_s, d_t);
-  olive_status st;
-  if ((st = launch_gather_rows(c, h_s, rows, n_rows, T, d_s, w.hcs, dev_status)) != OLIVE_OK) return st;
-  if ((st = launch_gather_rows(c, h_t, rows, n_rows, T, d_t, w.hct, dev_status)) != OLIVE_OK) return st;
   const size_t tb = sizeof(float) * T, tkb = sizeof(float) * T * static_cast<size_t>(K);
-  float* zero_t[] = {kl, s_lse, t_lse, s_entropy, overlap, kl_topk};
-  for (float* z : zero_t)
-    if (z && cudaMemsetAsync(z, 0, tb, c.stream) != cudaSuccess) return OLIVE_ERR_CUDA;
-  if ((s_topk_logp && cudaMemsetAsync(s_topk_logp, 0, tkb, c.stream) != cudaSuccess) ||
-      (t_logp_s && cudaMemsetAsync(t_logp_s, 0, tkb, c.stream) != cudaSuccess) ||
-      (s_topk_ids && cudaMemsetAsync(s_topk_ids, 0xff, tkb, c.stream) != cudaSuccess))
-    return OLIVE_ERR_CUDA;
+  Prepare q;
+  q.gather(h_s, d_s, w.hcs);
+  q.gather(h_t, d_t, w.hct);
+  for (float* z : {kl, s_lse, t_lse, s_entropy, overlap, kl_topk}) q.fill(z, tb);
+  q.fill(s_topk_logp, tkb);
+  q.fill(t_logp_s, tkb);
+  q.fill(s_topk_ids, tkb, 0xff);
+  olive_status st;
+  if ((st = launch_prepare(c, q, rows, n_rows, T, dev_status)) != OLIVE_OK) return st;
 
   CUtensorMap mHs, mWs, mHt, mWt;
   if (!encode_bf16_2d(&mHs, w.hcs, d_s, Tpad, 2ull * d_s, 64, 128) ||

@@ -155,12 +155,12 @@ olive_status launch_topk_compare(const Ctx& c, const void* h_t, const void* W_t,
                                  const float* s_logp, const int32_t* t_ids, const float* t_lse,
                                  float* overlap, float* kl_topk, float* t_logp_s,
                                  int32_t* dev_status) {
-  if (cudaMemsetAsync(overlap, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      cudaMemsetAsync(kl_topk, 0, sizeof(float) * T, c.stream) != cudaSuccess ||
-      (t_logp_s &&
-       cudaMemsetAsync(t_logp_s, 0, sizeof(float) * T * static_cast<size_t>(K), c.stream) !=
-           cudaSuccess))
-    return OLIVE_ERR_CUDA;
+  Prepare q;
+  q.fill(overlap, sizeof(float) * T);
+  q.fill(kl_topk, sizeof(float) * T);
+  q.fill(t_logp_s, sizeof(float) * T * static_cast<size_t>(K));
+  const olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
+  if (st != OLIVE_OK) return st;
   topk_compare_kernel<<<c.num_sms * 8, 256, 0, c.stream>>>(
       static_cast<const uint4*>(h_t), static_cast<const uint4*>(W_t), d_t / 8, rows, n_rows, T, V,
       inv_tau, K, s_ids, s_logp, t_ids, t_lse, overlap, kl_topk, t_logp_s, dev_status);
