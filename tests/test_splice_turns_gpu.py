@@ -126,3 +126,34 @@ def test_multi_turn_forward_and_backward():
     rdh, rdw = oracle.token_loss_bwd(to_f64(h), to_f64(W), o["targets"], o["rows"], reduction="mean")
     assert_close_grad(dh.cpu().numpy(), rdh, "dH")
     assert_close_grad(dw.cpu().numpy(), rdw, "dW")
+
+
+@pytest.mark.parametrize("S,T_cap", [(1, None), (255, None), (257, None), (2048, None), (2049, None),
+                                     (300, 4096 * 2048), (300, 4096 * 2048 + 1), (2100, 4096 * 2048 + 1)])
+def test_both_sides_of_the_block_scans(S, T_cap):
+    """Sequences and 2048-position chunks on both sides of what a block scans
+    for itself, with and without turn flags, then malformed offsets."""
+    rng = np.random.default_rng(S)
+    b = synth.batch_from_lengths(rng, rng.integers(1, 30, size=S), rng.integers(0, 40, size=S), 5000)
+    flags = (rng.random(len(b.cont_ids)) < 0.5).astype(np.uint8)
+    _compare(b, flags, T_cap)
+    pi, po, ci, co = batch_to_cuda(b)
+    cap = T_cap or b.T
+    g = B.olive_splice_pack(pi, po, ci, co, b.V, cap)
+    o = oracle.splice_pack(b.prefix_ids, b.prefix_off, b.cont_ids, b.cont_off, b.V)
+    n = o["n_rows"]
+    assert int(g["n_rows"].item()) == n and (g["rows"][n:] == -1).all()
+    assert np.array_equal(g["rows"][:n].cpu().numpy(), o["rows"])
+    for k in ("ids", "targets", "loss_mask"):
+        assert np.array_equal(g[k][:b.T].cpu().numpy().astype(np.int64), o[k]), k
+        assert (g[k][b.T:] == (-1 if k == "targets" else 0)).all(), k
+    for k in ("cu_seqlens", "cut_offsets"):
+        assert np.array_equal(g[k].cpu().numpy().astype(np.int64), o[k]), k
+    # an empty prefix (a repeated offset) clears every output
+    po[S // 2 + 1:] -= po[S // 2 + 1] - po[S // 2]
+    fl = torch.from_numpy(flags).cuda()
+    for g in (B.olive_splice_pack(pi, po, ci, co, b.V, cap),
+              B.olive_splice_pack_masked(pi, po, ci, co, fl, b.V, cap)):
+        assert B.status_bits(g["dev_status"]) == ["OLIVE_ERR_OFFSETS"]
+        assert int(g["n_rows"].item()) == 0 and (g["rows"] == -1).all()
+        assert not any(g[k].any() for k in ("ids", "loss_mask", "cu_seqlens", "cut_offsets"))
