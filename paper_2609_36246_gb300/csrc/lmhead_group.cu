@@ -544,7 +544,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
 
   const uint32_t tmem_base = *tmem_slot;
-  // (read from shared memory where it is used: the epilogue needs its registers)
+  // (each role copies it to registers: shared memory is busy with the MMAs'
+  // operands, and the epilogue's reads of it cost pass B 3 %)
   const GSched& s = *sched_smem;
   const WaitCtl ctl{abort_flag, p.wait_limit_ns};
   const int g = p.g;
@@ -764,6 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // accumulator rows (thread = row), `half` choosing the columns: the first
     // or last 128 of a Z tile, the first or last 32-column blocks of the
     // member's output chunk
+    const GSched s = *sched_smem;
     const int half = warp >> 2;
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_addr = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
