@@ -123,6 +123,9 @@ OLIVE_API int olive_abi_version(void);
 /* Static text for a status code. Never NULL. */
 OLIVE_API const char* olive_status_string(olive_status s);
 
+/* Zeroes a device status word on `stream` (asynchronous). */
+OLIVE_API olive_status olive_status_clear(int32_t* dev_status, void* stream);
+
 /*
  * Workspace bytes a compute call needs for host-side upper bound T rows.
  *   op  OLIVE_OP_LOGPROB_FWD / OLIVE_OP_LOSS_BWD: d = hidden width, d_t ignored.

@@ -195,11 +195,6 @@ struct GroupArgs {
   int d2, reverse;
   const float *lse_sc, *lse_tc, *kl, *grad_kl;
 };
-// mode 0: reference maxima, 1: pass A (lse, logp, dH), 2: pass B (dW),
-// 3: divergence gradient (d_hidden = G . W with G from both heads)
-olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W, int32_t T,
-                          int32_t d, int32_t V, const GroupArgs& a, int c_base, int c_end,
-                          uint32_t* ring_ctr);
 // The divergence gradient on chip: d_h_s = G . W_s with G from both heads'
 // logits (recomputed tile by tile by groups of CTA pairs) and the value sweep's kl, lse_s, lse_t.
 olive_status launch_kl_group_grad(const Ctx& c, const void* hcs, const void* hct, const void* W_s,

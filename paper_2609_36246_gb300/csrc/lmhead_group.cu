@@ -1446,11 +1446,45 @@ size_t group_ctr_words(int64_t T, int64_t d, int64_t V) {
 
 int group_sweep_cols(int sms) { return sweep_cols_for(sms < kGroupMaxSms ? sms : kGroupMaxSms); }
 
+namespace {
+
+// The tensor maps of a mode's operands (GM_REF and GM_A share theirs, so a call
+// encodes them once: half a microsecond of host time a map).
+bool make_maps(GroupMaps* maps, int mode, const void* hc, const void* W, int32_t T, int32_t d, int32_t V,
+               const GroupArgs& a) {
+  const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
+  const bool rowsA = mode != GM_B;
+  const void* zaBase = rowsA ? hc : W;
+  const void* zbBase = rowsA ? W : hc;
+  const uint64_t zaRows = rowsA ? Tpad : V;
+  const uint64_t zbRows = rowsA ? V : Tpad;
+  // the ring viewed as rows of 64 bf16 (one 128-byte row of a slice image)
+  const uint64_t ring_rows = group_ring_bytes(T, d, V) / 128;
+  // inner tiles of 256 vocabulary entries (rows in pass B); each CTA of a pair
+  // loads half of them as its B rows
+  if (!encode_bf16_2d(&maps->za, zaBase, d, zaRows, 2ull * d, 64, 128) ||
+      !encode_bf16_2d(&maps->zb, zbBase, d, zbRows, 2ull * d, 64, kZN / 2) ||
+      !encode_bf16_2d(&maps->xb, zbBase, d, zbRows, 2ull * d, 64, 64) ||
+      !encode_bf16_2d_plain(&maps->xa, a.ring, 64, ring_rows, 128, 64, 128))
+    return false;
+  if (mode == GM_KL) {
+    if (!encode_bf16_2d(&maps->za2, a.hc2, a.d2, Tpad, 2ull * a.d2, 64, 128) ||
+        !encode_bf16_2d(&maps->zb2, a.W2, a.d2, V, 2ull * a.d2, 64, kZN / 2))
+      return false;
+  } else {
+    maps->za2 = maps->za;
+    maps->zb2 = maps->zb;
+  }
+  return true;
+}
+
+// mode 0: reference maxima, 1: pass A (lse, logp, dH), 2: pass B (dW), 3:
+// divergence gradient (d_hidden = G . W with G from both heads); maps_in: the
+// mode's tensor maps, null to make them here
 olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W, int32_t T,
                           int32_t d, int32_t V, const GroupArgs& a, int c_base, int c_end,
-                          uint32_t* ring_ctr) {
+                          uint32_t* ring_ctr, const GroupMaps* maps_in = nullptr) {
   const int sms = c.num_sms < kGroupMaxSms ? c.num_sms : kGroupMaxSms;
-  const int64_t Tpad = align_up(static_cast<size_t>(T), kRowAlign);
   GroupShape gs;
   if (mode == GM_REF) {
     gs.g = 1;
@@ -1462,29 +1496,12 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
     gs.ngroups = std::min(gs.ngroups, group_count_max(T, d, V));
     if (gs.ngroups < 2 || gs.g * gs.ngroups > sms) return OLIVE_ERR_SHAPE;
   }
-  GroupMaps maps;
-  const bool rowsA = mode != GM_B;
-  const void* zaBase = rowsA ? hc : W;
-  const void* zbBase = rowsA ? W : hc;
-  const uint64_t zaRows = rowsA ? Tpad : V;
-  const uint64_t zbRows = rowsA ? V : Tpad;
-  // the ring viewed as rows of 64 bf16 (one 128-byte row of a slice image)
-  const uint64_t ring_rows = group_ring_bytes(T, d, V) / 128;
-  // inner tiles of 256 vocabulary entries (rows in pass B); each CTA of a pair
-  // loads half of them as its B rows
-  if (!encode_bf16_2d(&maps.za, zaBase, d, zaRows, 2ull * d, 64, 128) ||
-      !encode_bf16_2d(&maps.zb, zbBase, d, zbRows, 2ull * d, 64, kZN / 2) ||
-      !encode_bf16_2d(&maps.xb, zbBase, d, zbRows, 2ull * d, 64, 64) ||
-      !encode_bf16_2d_plain(&maps.xa, a.ring, 64, ring_rows, 128, 64, 128))
-    return OLIVE_ERR_CUDA;
-  if (mode == GM_KL) {
-    if (!encode_bf16_2d(&maps.za2, a.hc2, a.d2, Tpad, 2ull * a.d2, 64, 128) ||
-        !encode_bf16_2d(&maps.zb2, a.W2, a.d2, V, 2ull * a.d2, 64, kZN / 2))
-      return OLIVE_ERR_CUDA;
-  } else {
-    maps.za2 = maps.za;
-    maps.zb2 = maps.zb;
+  GroupMaps own;
+  if (!maps_in) {
+    if (!make_maps(&own, mode, hc, W, T, d, V, a)) return OLIVE_ERR_CUDA;
+    maps_in = &own;
   }
+  const GroupMaps& maps = *maps_in;
 
   GroupParams p = {};
   p.dev_status = a.dev_status;
@@ -1552,6 +1569,7 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   }
 }
 
+}  // namespace
 }  // namespace olive
 
 namespace olive {
@@ -1604,7 +1622,10 @@ olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,
   a.d_W = d_W;
   a.out_dtype = grad_dtype;
 
-  if (fwd && (st = launch_group(c, GM_REF, w.hc, W, T, d, V, a, 0, d, nullptr)) != OLIVE_OK)
+  GroupMaps ma, mb;
+  if (!make_maps(&ma, GM_A, w.hc, W, T, d, V, a) || !make_maps(&mb, GM_B, w.hc, W, T, d, V, a))
+    return OLIVE_ERR_CUDA;
+  if (fwd && (st = launch_group(c, GM_REF, w.hc, W, T, d, V, a, 0, d, nullptr, &ma)) != OLIVE_OK)
     return st;
   // one sweep of both passes per range of output columns the SMs can hold
   // (every d up to 19456 at 152 SMs takes one)
@@ -1617,14 +1638,15 @@ olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,
     a.lse_known = (!fwd || cb > 0) ? 1 : 0;
     a.write_fwd = (fwd && cb == 0) ? 1 : 0;
     a.redo = 0;
-    if ((st = launch_group(c, GM_A, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr)) != OLIVE_OK) return st;
+    if ((st = launch_group(c, GM_A, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr, &ma)) != OLIVE_OK)
+      return st;
     if (fwd && cb == 0) {
       a.redo = 1;
-      if ((st = launch_group(c, GM_A, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr + rw)) != OLIVE_OK)
+      if ((st = launch_group(c, GM_A, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr + rw, &ma)) != OLIVE_OK)
         return st;
       a.redo = 0;
     }
-    if ((st = launch_group(c, GM_B, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr + 2 * rw)) != OLIVE_OK)
+    if ((st = launch_group(c, GM_B, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr + 2 * rw, &mb)) != OLIVE_OK)
       return st;
   }
   return fwd ? launch_loss_reduce(c, n_rows, T, w.nll, reduction, loss) : OLIVE_OK;

@@ -384,6 +384,13 @@ const char* olive_status_string(olive_status s) {
   return "unknown status";
 }
 
+olive_status olive_status_clear(int32_t* dev_status, void* stream) {
+  if (!dev_status) return OLIVE_ERR_INVALID_ARG;
+  return cudaMemsetAsync(dev_status, 0, sizeof(int32_t), static_cast<cudaStream_t>(stream)) == cudaSuccess
+             ? OLIVE_OK
+             : OLIVE_ERR_CUDA;
+}
+
 size_t olive_workspace_size(int op, int32_t T, int32_t d, int32_t d_t, int32_t V, int grad,
                             int grad_dtype) {
   if (op == OLIVE_OP_SPLICE_MASKED) return T < 1 ? 0 : splice_masked_ws_bytes(T);
