@@ -348,6 +348,32 @@ __device__ __forceinline__ Pos locate(const GSched& s, int e) {
   const int i = x / s.ni;
   return Pos{tail ? s.rp0 + i : s.pg + i * s.npg, x - i * s.ni};
 }
+// Walks a group's exchange tiles in order without a division a tile.  What the
+// producer and MMA warps do between two instructions of theirs shows in the
+// tensor pipe, which has little of a queue: pass A at 1024 rows, d = 4096,
+// V = 151936 took 657 cycles a K step (480 at the tensor pipe's peak) with
+// locate(), a remainder and whole descriptors built at every tile and MMA, 633
+// with this and additions, and 511 with the roles' loops run by whole warps
+// (mbar_wait_warp).
+struct TileWalk {
+  int e, k, slot;
+  int ni, tail0, ktail, R;
+  __device__ __forceinline__ TileWalk(const GSched& s, int ring_slots) {
+    e = 0;
+    slot = 0;
+    ni = s.ni;
+    R = ring_slots;
+    tail0 = s.tail0;
+    ktail = s.nt > 0 ? s.x0 % s.ni : 0;
+    k = tail0 == 0 ? ktail : 0;
+  }
+  __device__ __forceinline__ void next() {
+    ++e;
+    k = k + 1 == ni ? 0 : k + 1;
+    if (e == tail0) k = ktail;
+    slot = slot + 1 == R ? 0 : slot + 1;
+  }
+};
 // does tile e open / close its outer tile's part in this group?
 __device__ __forceinline__ bool opens(const GSched& s, int e, int k) { return k == 0 || e == s.tail0; }
 __device__ __forceinline__ bool closes(const GSched& s, int e, int k) {
@@ -508,9 +534,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* meta_l = reinterpret_cast<float*>(misc + 128);                 // [256] lse2 (GM_B)
   int* meta_y = reinterpret_cast<int*>(misc + 128 + kMetaBytes / 2);    // [256] targets (GM_B)
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank();
+  const uint32_t rank = warp_uniform(cluster_rank());
 
   if (threadIdx.x == 0) {
     for (int st = 0; st < kStages; ++st) {
@@ -556,17 +582,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp >= kEpiWarps) {
     regs_dec<kOtherRegs>();
     if (warp == kProducerWarp) {
-      // lane 0 issues every copy (this CTA's 128 rows of A and its half of B;
+      // one lane issues every copy (this CTA's 128 rows of A and its half of B;
       // completion counted on the even CTA's full barrier, whose producer
       // announces both CTAs' bytes: the odd CTA's copies may land first, the
       // transaction count then dips below zero within the phase, which mbarriers
       // allow; no phase can mix with the next, since a CTA refills a stage only
-      // after the MMAs that read it have committed); the whole warp checks the
-      // `ready` flags of a round's g exchange tiles at once
-      const GSched s = *sched_smem;
+      // after the MMAs that read it have committed); the lanes share the check
+      // of the `ready` flags of a round's g exchange tiles
+      const GSched s = warp_uniform_copy(sched_smem);
+      const bool leader = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
+      TileWalk at(s, p.R);
+      const int xrow = s.q * p.R * 4;  // the group's first slice in the ring
       const bool paced = consume && p.ngroups > 2;
       // the streamed operand of a Z job (W rows in pass A, hc rows in pass B)
       // is read again by the accumulation a round later: keep it in the L2
@@ -584,48 +613,54 @@ __global__ void __launch_bounds__(kThreads, 1)
         // a Z product: za x zb, or GM_KL's teacher za2 x zb2; the B rows are this
         // CTA's half of the 256-wide vocabulary (or row) tile
         auto load_z = [&](bool second) {
-            const Pos at = locate(s, j);
-          const int o = outer_of(p, s, at.rp);
-          const int k = at.k;
+          const Pos z = locate(s, j);
+          const int o = warp_uniform(outer_of(p, s, z.rp));
+          const int k = z.k;
           const int steps = second ? s.nk2 : s.nk;
           for (int ks = 0; ok && ks < steps; ++ks) {
-            if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
+            if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
             const uint32_t sA = stages + stage * kStageBytes;
             const uint32_t fb = map_shared(full_bar(stage), 0);
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kStageBytes);
             // (a skipped copy leaves its stage short: the MMA's wait then runs
             // out and the call reports OLIVE_ERR_TIMEOUT as well)
-            if (OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph && k >= 0 && k < s.ni)) {
-              tma_load_2d_pair(sA, second ? &maps.za2 : &maps.za, fb, ks * kBK, o * kBM);
-              tma_load_2d_pair_hint(sA + kSA, second ? &maps.zb2 : &maps.zb, fb, ks * kBK,
-                                    k * kZN + static_cast<int>(rank) * (kZN / 2), keep);
+            const bool in = OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph && k >= 0 && k < s.ni);
+            if (leader) {
+              if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * kStageBytes);
+              if (in) {
+                tma_load_2d_pair(sA, second ? &maps.za2 : &maps.za, fb, ks * kBK, o * kBM);
+                tma_load_2d_pair_hint(sA + kSA, second ? &maps.zb2 : &maps.zb, fb, ks * kBK,
+                                      k * kZN + static_cast<int>(rank) * (kZN / 2), keep);
+              }
             }
             if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
         };
-        auto load_tiles = [&](int e_from, int e_to) {
-          for (int e = e_from; ok && e < e_to; ++e) {
-            const int slot = e % p.R;
-            const int k = locate(s, e).k;
+        auto load_tiles = [&](int e_to) {
+          for (; ok && at.e < e_to; at.next()) {
+            const int slot = at.slot;
+            const int k = at.k;
             const int nsl = slices_of(s, k);
             for (int sl = 0; sl < nsl; ++sl) {
-              if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
+              if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
               const uint32_t sA = stages + stage * kStageBytes;
               const uint32_t fb = map_shared(full_bar(stage), 0);
-              if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * (kXSlice + s.nbox * 8192));
               // TMA x coordinates must be 16-byte aligned (8 bf16)
-              if (OLIVE_DCHECK(p.dev_status, static_cast<int64_t>(ring0 + slot) < p.ring_tiles &&
-                                                 s.b0 % 8 == 0 && s.b0 >= 0 && s.b0 < p.d + 64)) {
-                tma_load_2d_pair(sA, &maps.xa, fb, 0, static_cast<int>(((ring0 + slot) * 4 + sl) * kBM));
-                for (int b = 0; b < s.nbox; ++b)
-                  tma_load_2d_pair(sA + kSA + b * 8192, &maps.xb, fb, s.b0 + 64 * b, k * kZN + sl * kBK);
+              const bool in = OLIVE_DCHECK(p.dev_status, static_cast<int64_t>(ring0 + slot) < p.ring_tiles &&
+                                                             s.b0 % 8 == 0 && s.b0 >= 0 && s.b0 < p.d + 64);
+              if (leader) {
+                if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * (kXSlice + s.nbox * 8192));
+                if (in) {
+                  tma_load_2d_pair(sA, &maps.xa, fb, 0, (xrow + slot * 4 + sl) * kBM);
+                  tma_load_2d_pair(sA + kSA, &maps.xb, fb, s.b0, k * kZN + sl * kBK);
+                  if (s.nbox > 1)
+                    tma_load_2d_pair(sA + kSA + 8192, &maps.xb, fb, s.b0 + 64, k * kZN + sl * kBK);
+                }
               }
               if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
           }
         };
-        if (job && lane == 0) load_z(false);
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (job) load_z(false);
         if (!ok || !consume) continue;
         const int e_lo = r > 0 ? (r - 1) * g : 0;
         const int e_end = r > 0 ? min(r * g, s.E) : 0;
@@ -633,14 +668,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
           if (!ok) break;
         }
-        if (lane == 0) {
-          fence_proxy_async_global();
-          const int e_mid = split_point<kMode>(s, e_lo, e_end);
-          load_tiles(e_lo, e_mid);
-          if (kMode == GM_KL && job) load_z(true);
-          load_tiles(e_mid, e_end);
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+        fence_proxy_async_global();
+        const int e_mid = split_point<kMode>(s, e_lo, e_end);
+        load_tiles(e_mid);
+        if (kMode == GM_KL && job) load_z(true);
+        load_tiles(e_end);
       }
       if (paced && s.m == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = kPaceDone;
       if (!ok && lane == 0) {
@@ -673,69 +705,79 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       __syncwarp();
     } else if (warp == kMmaWarp) {
-      // the even CTA's lane 0 issues the pair's MMAs (M = 256: 128 rows in each
-      // CTA's TMEM); the odd CTA's MMA warp only holds its TMEM allocation
-      if (lane == 0 && rank == 0) {
-        const GSched s = *sched_smem;
-        const uint32_t zacc = tmem_base;
-        const uint32_t oacc = tmem_base + 256;
+      // a lane of the even CTA's MMA warp issues the pair's MMAs (M = 256: 128
+      // rows in each CTA's TMEM); the odd CTA's only holds its TMEM allocation
+      if (rank == 0) {
+        const GSched s = warp_uniform_copy(sched_smem);
+        const bool leader = elect_one();
+        const uint32_t zacc = warp_uniform(tmem_base);
+        const uint32_t oacc = zacc + 256;
         const uint32_t idz = idesc_bf16(2 * kBM, kZN, false, false);
         const uint32_t idx = idesc_bf16(2 * kBM, s.nacc, false, true);
         const uint32_t copied_peer = map_shared(smem_u32(const_cast<uint32_t*>(copied)), 1);
+        // a stage's operand descriptors are these plus its offset in 16-byte
+        // units: the issuing thread then adds twice an MMA
+        const uint64_t dA = sdesc_sw128(stages, 16, 1024);
+        const uint64_t dBk = sdesc_sw128(stages + kSA, 16, 1024);     // B K-major (Z)
+        const uint64_t dBm = sdesc_sw128(stages + kSA, 8192, 1024);   // B MN-major (accumulation)
         int stage = 0;
         uint32_t phase = 0, zph = 0, oph = 0;
         bool ok = true;
+        TileWalk at(s, p.R);
         for (int r = 0; ok && r <= nr; ++r) {
           const int j = r * g + s.m;
           const bool job = r < nr && j < s.E;
           auto z_product = [&](int steps) {
-            if (!mbar_wait(zempty, zph ^ 1u, ctl)) { ok = false; return; }
+            if (!mbar_wait_warp(zempty, zph ^ 1u, ctl)) { ok = false; return; }
             tc_fence_after();
             for (int ks = 0; ks < steps; ++ks) {
-              if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; return; }
+              if (!mbar_wait_warp(full_bar(stage), phase, ctl)) { ok = false; return; }
               tc_fence_after();
-              const uint32_t sA = stages + stage * kStageBytes;
-              const uint32_t sB = sA + kSA;
+              const uint32_t so = static_cast<uint32_t>(stage) * (kStageBytes >> 4);
+              const uint32_t acc0 = ks > 0 ? 1u : 0u;
+              if (leader) {
 #pragma unroll
-              for (int kk = 0; kk < kBK / 16; ++kk)
-                umma_bf16_pair(zacc, sdesc_sw128(sA + kk * 32, 16, 1024), sdesc_sw128(sB + kk * 32, 16, 1024),
-                               idz, (ks > 0 || kk > 0) ? 1u : 0u);
-              umma_commit_pair(empty_bar(stage));
+                for (int kk = 0; kk < kBK / 16; ++kk)
+                  umma_bf16_pair(zacc, dA + (so + kk * 2), dBk + (so + kk * 2), idz, kk > 0 ? 1u : acc0);
+                umma_commit_pair(empty_bar(stage));
+              }
               if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            umma_commit_pair(zfull);
+            if (leader) umma_commit_pair(zfull);
             zph ^= 1u;
           };
-          auto accumulate = [&](int e_from, int e_to) {
-            for (int e = e_from; ok && e < e_to; ++e) {
-              const int k = locate(s, e).k;
+          auto accumulate = [&](int e_to) {
+            for (; ok && at.e < e_to; at.next()) {
+              const int e = at.e, k = at.k;
               const bool first = opens(s, e, k);
               if (first) {
-                if (!mbar_wait(oempty, oph ^ 1u, ctl)) { ok = false; break; }
+                if (!mbar_wait_warp(oempty, oph ^ 1u, ctl)) { ok = false; break; }
                 tc_fence_after();
               }
               const int nsl = slices_of(s, k);
               for (int sl = 0; sl < nsl; ++sl) {
-                if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
+                if (!mbar_wait_warp(full_bar(stage), phase, ctl)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t sA = stages + stage * kStageBytes;
-                const uint32_t sB = sA + kSA;
+                const uint32_t so = static_cast<uint32_t>(stage) * (kStageBytes >> 4);
+                const uint32_t acc0 = !first || sl > 0 ? 1u : 0u;
+                if (leader) {
 #pragma unroll
-                for (int kk = 0; kk < kBK / 16; ++kk)
-                  umma_bf16_pair(oacc, sdesc_sw128(sA + kk * 32, 16, 1024),
-                                 sdesc_sw128(sB + kk * 2048, 8192, 1024), idx,
-                                 (!first || sl > 0 || kk > 0) ? 1u : 0u);
-                umma_commit_pair(empty_bar(stage));
+                  for (int kk = 0; kk < kBK / 16; ++kk)
+                    umma_bf16_pair(oacc, dA + (so + kk * 2), dBm + (so + kk * 128), idx, kk > 0 ? 1u : acc0);
+                  umma_commit_pair(empty_bar(stage));
+                }
                 if (++stage == kStages) { stage = 0; phase ^= 1u; }
               }
               if (!ok) break;
               // every slice of tile e has landed in both CTAs: their signal warps
               // tell the two groups (a slot may be rewritten once all of its
               // group's members have said so)
-              *copied = static_cast<uint32_t>(e + 1);
-              st_shared_cluster(copied_peer, static_cast<uint32_t>(e + 1));
+              if (leader) {
+                *copied = static_cast<uint32_t>(e + 1);
+                st_shared_cluster(copied_peer, static_cast<uint32_t>(e + 1));
+              }
               if (closes(s, e, k)) {
-                umma_commit_pair(ofull);
+                if (leader) umma_commit_pair(ofull);
                 oph ^= 1u;
               }
             }
@@ -745,17 +787,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int e_lo = r > 0 ? (r - 1) * g : 0;
           const int e_end = r > 0 ? min(r * g, s.E) : 0;
           const int e_mid = split_point<kMode>(s, e_lo, e_end);
-          accumulate(e_lo, e_mid);
+          accumulate(e_mid);
           if (kMode == GM_KL && ok && job) z_product(s.nk2);
-          if (ok) accumulate(e_mid, e_end);
+          if (ok) accumulate(e_end);
         }
         // arrives once every MMA issued above has completed (bounded wait that
         // ignores the abort flag: it only waits for work already in flight)
-        umma_commit_pair(drain);
+        if (leader) umma_commit_pair(drain);
         volatile int keep_waiting = 0;
         const uint64_t floor_ns = 200ull * 1000 * 1000;
         const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
-        mbar_wait(drain, 0, own);
+        mbar_wait_warp(drain, 0, own);
       }
       __syncwarp();
     }
