@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
   typename Kern::Sched* sched_smem = reinterpret_cast<typename Kern::Sched*>(misc + 16);
   static_assert(sizeof(typename Kern::Sched) <= L::MISC_BYTES - 16, "Sched too large");
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -152,27 +152,32 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
   const WaitCtl ctl{abort_flag, p.wait_limit_ns};
   const int n_units = Kern::num_units(p, sched);
 
+  // (the producer and MMA warps run their loops converged and elect the lane
+  // that issues: mbar_wait_warp)
   if (warp == CT::kProducer) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-        const int nt = Kern::unit_len(p, sched, u);
-        for (int t = 0; ok && t < nt; ++t) {
-          const TileC tc = Kern::tile(p, sched, u, t);
-          const int nk_all = tc.nk + (Kern::kDual ? tc.nk2 : 0);
-          for (int k = 0; k < nk_all; ++k) {
-            if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
-            const uint32_t sA = ring + stage * L::STAGE_BYTES;
-            const uint32_t sB = sA + L::A_BYTES;
-            const uint32_t fb = full_bar(stage);
-            const bool second = Kern::kDual && k >= tc.nk;
-            const CUtensorMap* mA = second ? &mapA2 : &mapA;
-            const CUtensorMap* mB = second ? &mapB2 : &mapB;
-            const int kl = second ? k - tc.nk : k;
-            const int ka = (second ? 0 : tc.ka0) + kl * kBK;
-            const int kb = (second ? 0 : tc.kb0) + kl * kBK;
+    const typename Kern::Sched sw = warp_uniform_copy(sched_smem);
+    const int nu = warp_uniform(n_units);
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < nu; u += gridDim.x) {
+      const int nt = Kern::unit_len(p, sw, u);
+      for (int t = 0; ok && t < nt; ++t) {
+        const TileC tc = Kern::tile(p, sw, u, t);
+        const int nk_all = tc.nk + (Kern::kDual ? tc.nk2 : 0);
+        for (int k = 0; k < nk_all; ++k) {
+          if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
+          const uint32_t sA = ring + stage * L::STAGE_BYTES;
+          const uint32_t sB = sA + L::A_BYTES;
+          const uint32_t fb = full_bar(stage);
+          const bool second = Kern::kDual && k >= tc.nk;
+          const CUtensorMap* mA = second ? &mapA2 : &mapA;
+          const CUtensorMap* mB = second ? &mapB2 : &mapB;
+          const int kl = second ? k - tc.nk : k;
+          const int ka = (second ? 0 : tc.ka0) + kl * kBK;
+          const int kb = (second ? 0 : tc.kb0) + kl * kBK;
+          if (leader) {
             mbar_arrive_expect_tx(fb, L::STAGE_BYTES);
             if constexpr (Kern::kAMn) {
 #pragma unroll
@@ -187,65 +192,69 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
             } else {
               tma_load_2d(sB, mB, fb, kb, tc.n0);
             }
-            if (++stage == Kern::kStages) { stage = 0; phase ^= 1u; }
           }
+          if (++stage == Kern::kStages) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) {
-        // give copies that were already issued time to land before retiring
-        const uint64_t t0 = global_timer_ns();
-        while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
-      }
+    }
+    if (!ok) {
+      // give copies that were already issued time to land before retiring
+      const uint64_t t0 = global_timer_ns();
+      while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
     }
     __syncwarp();
   } else if (warp == CT::kMma) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = idesc_bf16(kBM, Kern::kBN, Kern::kAMn, Kern::kBMn);
-      int stage = 0;
-      uint32_t phase = 0;
-      int buf = 0;
-      uint32_t aphase = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < n_units; u += gridDim.x) {
-        const int nt = Kern::unit_len(p, sched, u);
-        for (int t = 0; ok && t < nt; ++t) {
-          const TileC tc = Kern::tile(p, sched, u, t);
-          const int nk_all = tc.nk + (Kern::kDual ? tc.nk2 : 0);
-          if (!mbar_wait(tempty_bar(buf), aphase ^ 1u, ctl)) { ok = false; break; }
+    constexpr uint32_t idesc = idesc_bf16(kBM, Kern::kBN, Kern::kAMn, Kern::kBMn);
+    const typename Kern::Sched sw = warp_uniform_copy(sched_smem);
+    const int nu = warp_uniform(n_units);
+    const uint32_t tb = warp_uniform(tmem_base);
+    const bool leader = elect_one();
+    // a stage's operand descriptors are these plus its offset in 16-byte units
+    const uint64_t dA = Kern::kAMn ? sdesc_sw128(ring, 8192, 1024) : sdesc_sw128(ring, 16, 1024);
+    const uint64_t dB = Kern::kBMn ? sdesc_sw128(ring + L::A_BYTES, 8192, 1024)
+                                   : sdesc_sw128(ring + L::A_BYTES, 16, 1024);
+    constexpr uint32_t kStepA = Kern::kAMn ? 2048 >> 4 : 32 >> 4;  // 16 K-elements on
+    constexpr uint32_t kStepB = Kern::kBMn ? 2048 >> 4 : 32 >> 4;
+    int stage = 0;
+    uint32_t phase = 0;
+    int buf = 0;
+    uint32_t aphase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < nu; u += gridDim.x) {
+      const int nt = Kern::unit_len(p, sw, u);
+      const TileC tc = Kern::tile(p, sw, u, 0);  // (every tile of a unit has the same K steps)
+      const int nk_all = tc.nk + (Kern::kDual ? tc.nk2 : 0);
+      for (int t = 0; ok && t < nt; ++t) {
+        if (!mbar_wait_warp(tempty_bar(buf), aphase ^ 1u, ctl)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t acc = tb + static_cast<uint32_t>(buf * L::ACC_COLS);
+        for (int k = 0; k < nk_all; ++k) {
+          if (!mbar_wait_warp(full_bar(stage), phase, ctl)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t acc = tmem_base + static_cast<uint32_t>(buf * L::ACC_COLS);
-          for (int k = 0; k < nk_all; ++k) {
-            if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
-            tc_fence_after();
-            const bool second = Kern::kDual && k >= tc.nk;
-            const uint32_t dt = second ? acc + Kern::kBN : acc;
-            const int kl = second ? k - tc.nk : k;
-            const uint32_t sA = ring + stage * L::STAGE_BYTES;
-            const uint32_t sB = sA + L::A_BYTES;
+          const bool second = Kern::kDual && k >= tc.nk;
+          const uint32_t dt = second ? acc + Kern::kBN : acc;
+          const uint32_t acc0 = (second ? k - tc.nk : k) > 0 ? 1u : 0u;
+          const uint32_t so = static_cast<uint32_t>(stage) * (L::STAGE_BYTES >> 4);
+          if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const uint64_t ad = Kern::kAMn ? sdesc_sw128(sA + kk * 2048, 8192, 1024)
-                                             : sdesc_sw128(sA + kk * 32, 16, 1024);
-              const uint64_t bd = Kern::kBMn ? sdesc_sw128(sB + kk * 2048, 8192, 1024)
-                                             : sdesc_sw128(sB + kk * 32, 16, 1024);
-              umma_bf16(dt, ad, bd, idesc, (kl > 0 || kk > 0) ? 1u : 0u);
-            }
+            for (int kk = 0; kk < kBK / 16; ++kk)
+              umma_bf16(dt, dA + (so + kk * kStepA), dB + (so + kk * kStepB), idesc, kk > 0 ? 1u : acc0);
             umma_commit(empty_bar(stage));
-            if (++stage == Kern::kStages) { stage = 0; phase ^= 1u; }
           }
-          if (!ok) break;
-          umma_commit(tfull_bar(buf));
-          if (++buf == L::ACC_BUFS) { buf = 0; aphase ^= 1u; }
+          if (++stage == Kern::kStages) { stage = 0; phase ^= 1u; }
         }
+        if (!ok) break;
+        if (leader) umma_commit(tfull_bar(buf));
+        if (++buf == L::ACC_BUFS) { buf = 0; aphase ^= 1u; }
       }
-      // arrives once every MMA issued above has completed (bounded wait that
-      // ignores the abort flag: it only waits for work already in flight)
-      umma_commit(drain_bar);
-      volatile int keep_waiting = 0;
-      const uint64_t floor_ns = 200ull * 1000 * 1000;  // in-flight MMAs finish in microseconds
-      const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
-      mbar_wait(drain_bar, 0, own);
     }
+    // arrives once every MMA issued above has completed (bounded wait that
+    // ignores the abort flag: it only waits for work already in flight)
+    if (leader) umma_commit(drain_bar);
+    volatile int keep_waiting = 0;
+    const uint64_t floor_ns = 200ull * 1000 * 1000;  // in-flight MMAs finish in microseconds
+    const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
+    mbar_wait_warp(drain_bar, 0, own);
     __syncwarp();
   } else {
     // epilogue warps: thread = accumulator row = TMEM lane (quadrant warp % 4)

@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
   Plan* plan_smem = reinterpret_cast<Plan*>(misc + 64);
   static_assert(sizeof(Plan) <= 64, "Plan too large");
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_uniform(static_cast<int>(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
@@ -588,35 +588,43 @@ __global__ void __launch_bounds__(kFThreads, 1)
 
   const int total = total_units(p, pl);
 
+  // (the producer and MMA warps run their loops converged and elect the lane
+  // that issues: mbar_wait_warp)
   if (warp == kFProducer) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < total; u += gridDim.x) {
-        const Unit x = decode(p, pl, u);
-        // wait until the tiles this one reads are published
-        bool dep = true;
-        if (p.phase != PH_ALL) {
-          // phases are separate launches in stream order: nothing to wait for
-        } else if (x.kind == K_GRAD && x.s > 0) {
-          const int pin = slab_in(pl, x.s - 1);
+    const Plan plw = warp_uniform_copy(plan_smem);
+    const int units = warp_uniform(total);
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+      const Unit x = decode(p, plw, u);
+      // wait until the tiles this one reads are published (lane 0 looks)
+      bool dep = true;
+      if (p.phase != PH_ALL) {
+        // phases are separate launches in stream order: nothing to wait for
+      } else if (lane == 0) {
+        if (x.kind == K_GRAD && x.s > 0) {
+          const int pin = slab_in(plw, x.s - 1);
           const int pmt = (pin + 127) / 128;
           dep = wait_counter(ctr_dhdw(p, x.s - 1),
-                             units_dh(pl, pmt) + units_dw(pl, x.s - 1, pin), ctl);
+                             units_dh(plw, pmt) + units_dw(plw, x.s - 1, pin), ctl);
         } else if (x.kind == K_DH) {
-          dep = wait_counter(ctr_row(p, x.s, x.i), pl.vt, ctl);
+          dep = wait_counter(ctr_row(p, x.s, x.i), plw.vt, ctl);
         } else if (x.kind == K_DW) {
-          dep = wait_counter(ctr_grad(p, x.s), units_grad(pl, x.mt), ctl);
+          dep = wait_counter(ctr_grad(p, x.s), units_grad(plw, x.mt), ctl);
         }
-        if (!dep) { ok = false; break; }
-        fence_proxy_async_global();
-        const int nk = unit_ksteps(p, x);
-        for (int k = 0; k < nk; ++k) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
-          const uint32_t sA = ring + stage * L::STAGE_BYTES;
-          const uint32_t sB = sA + L::A_BYTES;
-          const uint32_t fb = full_bar(stage);
+      }
+      if (!__all_sync(0xffffffffu, dep)) { ok = false; break; }
+      __syncwarp();
+      fence_proxy_async_global();
+      const int nk = unit_ksteps(p, x);
+      for (int k = 0; k < nk; ++k) {
+        if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
+        const uint32_t sA = ring + stage * L::STAGE_BYTES;
+        const uint32_t sB = sA + L::A_BYTES;
+        const uint32_t fb = full_bar(stage);
+        if (leader) {
           mbar_arrive_expect_tx(fb, L::STAGE_BYTES);
           switch (x.kind) {
             case K_GRAD:
@@ -639,59 +647,62 @@ __global__ void __launch_bounds__(kFThreads, 1)
               break;
             default: break;
           }
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        const uint64_t t0 = global_timer_ns();
-        while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
-      }
+    }
+    if (!ok) {
+      const uint64_t t0 = global_timer_ns();
+      while (global_timer_ns() - t0 < 50000) nanosleep_ns(1000);
     }
     __syncwarp();
   } else if (warp == kFMma) {
-    if (lane == 0) {
-      int stage = 0, buf = 0;
-      uint32_t phase = 0, aphase = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; ok && u < total; u += gridDim.x) {
-        const Unit x = decode(p, pl, u);
-        const int nk = unit_ksteps(p, x);
-        uint32_t idesc;
-        bool a_mn = false, b_mn = false;
-        switch (x.kind) {
-          case K_DH: idesc = idesc_bf16(kBM, kBN, false, true); b_mn = true; break;
-          case K_DW: idesc = idesc_bf16(kBM, kBN, true, true); a_mn = b_mn = true; break;
-          default: idesc = idesc_bf16(kBM, kBN, false, false); break;
-        }
-        if (!mbar_wait(tempty_bar(buf), aphase ^ 1u, ctl)) { ok = false; break; }
+    const Plan plw = warp_uniform_copy(plan_smem);
+    const int units = warp_uniform(total);
+    const uint32_t tb = warp_uniform(tmem_base);
+    const bool leader = elect_one();
+    // a stage's operand descriptors are these plus its offset in 16-byte units
+    // (K-major operands step 32 bytes on every 16 K-elements, MN-major 2048)
+    const uint64_t dAk = sdesc_sw128(ring, 16, 1024), dAm = sdesc_sw128(ring, 8192, 1024);
+    const uint64_t dBk = sdesc_sw128(ring + L::A_BYTES, 16, 1024);
+    const uint64_t dBm = sdesc_sw128(ring + L::A_BYTES, 8192, 1024);
+    int stage = 0, buf = 0;
+    uint32_t phase = 0, aphase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+      const Unit x = decode(p, plw, u);
+      const int nk = unit_ksteps(p, x);
+      const bool a_mn = x.kind == K_DW, b_mn = x.kind == K_DW || x.kind == K_DH;
+      const uint32_t idesc = a_mn ? idesc_bf16(kBM, kBN, true, true)
+                             : b_mn ? idesc_bf16(kBM, kBN, false, true)
+                                    : idesc_bf16(kBM, kBN, false, false);
+      const uint64_t dA = a_mn ? dAm : dAk, dB = b_mn ? dBm : dBk;
+      const uint32_t stepA = a_mn ? 2048 >> 4 : 32 >> 4, stepB = b_mn ? 2048 >> 4 : 32 >> 4;
+      if (!mbar_wait_warp(tempty_bar(buf), aphase ^ 1u, ctl)) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t acc = tb + static_cast<uint32_t>(buf * kBN);
+      for (int k = 0; k < nk; ++k) {
+        if (!mbar_wait_warp(full_bar(stage), phase, ctl)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t acc = tmem_base + static_cast<uint32_t>(buf * kBN);
-        for (int k = 0; k < nk; ++k) {
-          if (!mbar_wait(full_bar(stage), phase, ctl)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sA = ring + stage * L::STAGE_BYTES;
-          const uint32_t sB = sA + L::A_BYTES;
+        const uint32_t so = static_cast<uint32_t>(stage) * (L::STAGE_BYTES >> 4);
+        const uint32_t acc0 = k > 0 ? 1u : 0u;
+        if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk) {
-            const uint64_t ad = a_mn ? sdesc_sw128(sA + kk * 2048, 8192, 1024)
-                                     : sdesc_sw128(sA + kk * 32, 16, 1024);
-            const uint64_t bd = b_mn ? sdesc_sw128(sB + kk * 2048, 8192, 1024)
-                                     : sdesc_sw128(sB + kk * 32, 16, 1024);
-            umma_bf16(acc, ad, bd, idesc, (k > 0 || kk > 0) ? 1u : 0u);
-          }
+          for (int kk = 0; kk < kBK / 16; ++kk)
+            umma_bf16(acc, dA + (so + kk * stepA), dB + (so + kk * stepB), idesc, kk > 0 ? 1u : acc0);
           umma_commit(empty_bar(stage));
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        umma_commit(tfull_bar(buf));
-        if (++buf == nbufs) { buf = 0; aphase ^= 1u; }
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      umma_commit(drain_bar);
-      volatile int keep_waiting = 0;
-      const uint64_t floor_ns = 200ull * 1000 * 1000;  // in-flight MMAs finish in microseconds
-      const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
-      mbar_wait(drain_bar, 0, own);
+      if (!ok) break;
+      if (leader) umma_commit(tfull_bar(buf));
+      if (++buf == nbufs) { buf = 0; aphase ^= 1u; }
     }
+    if (leader) umma_commit(drain_bar);
+    volatile int keep_waiting = 0;
+    const uint64_t floor_ns = 200ull * 1000 * 1000;  // in-flight MMAs finish in microseconds
+    const WaitCtl own{&keep_waiting, p.wait_limit_ns > floor_ns ? p.wait_limit_ns : floor_ns};
+    mbar_wait_warp(drain_bar, 0, own);
     __syncwarp();
   } else {
     const int quad = warp & 3;

@@ -668,6 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
           if (!ok) break;
         }
+        __syncwarp();
         fence_proxy_async_global();
         const int e_mid = split_point<kMode>(s, e_lo, e_end);
         load_tiles(e_mid);
