@@ -133,6 +133,7 @@ constexpr int kThreads = 32 * (kEpiWarps + 4);  // three whole warpgroups (warp 
 // the epilogue, whose 128 held accumulator values otherwise spill (the L1 left
 // beside 227 KB of shared memory is too small for 384 stacks: spilled, a
 // 32-column block took ~5500 cycles).  2 x 216 + 72 = 3 x 168.
+constexpr int kPieceMax = 4;  // K steps (~2000 cycles) of a Z product at an outer tile's boundary
 constexpr int kEpiRegs = 216;
 constexpr int kOtherRegs = 72;
 constexpr int kStatusTimeoutBit = 1 << OLIVE_ERR_TIMEOUT;
@@ -400,18 +401,68 @@ __device__ __forceinline__ bool member_has_job(const GSched& s, int g, int e, in
   return lo + (((s.m - lo) % g) + g) % g <= e;
 }
 
-// Where a round's accumulation [e_lo, e_end) pauses for the second Z product.
-// The divergence's two products share the 256-column Z accumulator one after
-// the other: half of the previous round's tiles are accumulated between them,
-// which is when the epilogue takes the student's logits into registers.  It
-// pauses no later than before a tile that opens an outer tile: that tile
-// needs the accumulator which the epilogue hands back only after it has had
-// the teacher's logits.
+// Order of a round's work, the same for the producer, MMA and epilogue warps of
+// a pair.  The round accumulates tiles [e_lo, e_end); where one of them opens
+// an outer tile, its MMAs must wait until the epilogue has taken the previous
+// outer tile's accumulator.  So the Z product is cut: its first `head` K steps
+// start the round, `piece` more run at every such boundary while the
+// accumulator changes hands, the rest at the last one, and the Z epilogue comes
+// after the outer tiles that close before it (first in the round, it held all
+// of them up).  The tail of the round covers the Z epilogue, the head (at least
+// half of the product) the latency of the exchange.  Only pass B is cut so: the
+// outer tiles of the others are as long as the vocabulary.
+//
+// A round is `count` + 1 steps of the same two parts, so that each part's code
+// stands once in each role (a call of a few microseconds waits for much of its
+// code to come from memory): K steps [z0, z1) of a Z product, then tiles up to
+// `until`.  The divergence's two products are its two steps: half of the
+// previous round's tiles are accumulated between them, which is when the
+// epilogue takes the student's logits into registers, and no later than before
+// a tile that opens an outer tile (that needs the accumulator which the
+// epilogue hands back only after it has had the teacher's logits).
+struct Round {
+  int count;        // steps after the first
+  int first, last;  // tiles that the second and the last step open with
+  int head, piece;  // K steps of the Z product in the first step, and in the others
+};
+struct Step {
+  int z0, z1, steps;  // K steps of the product of `steps`
+  bool second;        // GM_KL: the teacher's product
+  int until;          // then the tiles before this one
+};
 template <int kMode>
-__device__ __forceinline__ int split_point(const GSched& s, int e_lo, int e_end) {
-  if (kMode != GM_KL || e_lo == e_end) return e_end;
-  const int next = e_lo + s.ni - locate(s, e_lo).k;  // first tile after e_lo that opens an outer tile
-  return min(e_lo + (e_end - e_lo + 1) / 2, next);
+__device__ __forceinline__ Round plan_round(const GSched& s, int e_lo, int e_end) {
+  Round rd{0, e_lo, e_lo, s.nk, 0};
+  if (kMode == GM_KL) {
+    rd.count = 1;
+    rd.first = e_lo == e_end ? e_end : min(e_lo + (e_end - e_lo + 1) / 2, e_lo + s.ni - locate(s, e_lo).k);
+    return rd;
+  }
+  if (kMode != GM_B || e_end - e_lo < 2) return rd;
+  rd.first = e_lo + s.ni - locate(s, e_lo).k;
+  // (tiles past the start of a split tail open at other distances)
+  const int end = e_lo < s.tail0 ? min(e_end, s.tail0 + 1) : e_end;
+  if (rd.first >= end) return rd;
+  rd.count = (end - 1 - rd.first) / s.ni + 1;
+  rd.last = rd.first + (rd.count - 1) * s.ni;
+  rd.piece = max(1, min(kPieceMax, s.nk / 2 / rd.count));
+  rd.head = max(1, s.nk - rd.count * rd.piece);
+  return rd;
+}
+template <int kMode>
+__device__ __forceinline__ Step round_step(const GSched& s, const Round& rd, int b, int e_end) {
+  Step st;
+  st.until = b == rd.count ? e_end : rd.first + b * s.ni;
+  st.second = kMode == GM_KL && b == 1;
+  if (kMode == GM_KL) {
+    st.z0 = 0;
+    st.z1 = st.steps = b == 0 ? s.nk : s.nk2;
+  } else {
+    st.steps = s.nk;
+    st.z0 = b == 0 ? 0 : min(s.nk, rd.head + (b - 1) * rd.piece);
+    st.z1 = b == rd.count ? s.nk : min(s.nk, rd.head + b * rd.piece);
+  }
+  return st;
 }
 
 // byte offset of row r (a multiple of 8) of K-slice sl in an exchange tile.
@@ -612,12 +663,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool job = r < nr && j < s.E;
         // a Z product: za x zb, or GM_KL's teacher za2 x zb2; the B rows are this
         // CTA's half of the 256-wide vocabulary (or row) tile
-        auto load_z = [&](bool second) {
+        auto load_z = [&](bool second, int ks0, int ks1) {
           const Pos z = locate(s, j);
           const int o = warp_uniform(outer_of(p, s, z.rp));
           const int k = z.k;
-          const int steps = second ? s.nk2 : s.nk;
-          for (int ks = 0; ok && ks < steps; ++ks) {
+          for (int ks = ks0; ok && ks < ks1; ++ks) {
             if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, ctl)) { ok = false; break; }
             const uint32_t sA = stages + stage * kStageBytes;
             const uint32_t fb = map_shared(full_bar(stage), 0);
@@ -660,20 +710,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
         };
-        if (job) load_z(false);
-        if (!ok || !consume) continue;
         const int e_lo = r > 0 ? (r - 1) * g : 0;
         const int e_end = r > 0 ? min(r * g, s.E) : 0;
-        if (r > 0) {
-          ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
-          if (!ok) break;
+        const Round rd = plan_round<kMode>(s, e_lo, e_end);
+        for (int b = 0; ok && b <= rd.count; ++b) {
+          const Step st = round_step<kMode>(s, rd, b, e_end);
+          if (job) load_z(st.second, st.z0, st.z1);
+          if (!ok || !consume) break;
+          if (b == 0 && r > 0) {
+            ok = wait_round_ready(p.ready + ring0, p.R, e_lo, e_end, lane, ctl);
+            if (!ok) break;
+            __syncwarp();
+            fence_proxy_async_global();
+          }
+          load_tiles(st.until);
         }
-        __syncwarp();
-        fence_proxy_async_global();
-        const int e_mid = split_point<kMode>(s, e_lo, e_end);
-        load_tiles(e_mid);
-        if (kMode == GM_KL && job) load_z(true);
-        load_tiles(e_end);
       }
       if (paced && s.m == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(p.pace + s.q) = kPaceDone;
       if (!ok && lane == 0) {
@@ -728,10 +779,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int r = 0; ok && r <= nr; ++r) {
           const int j = r * g + s.m;
           const bool job = r < nr && j < s.E;
-          auto z_product = [&](int steps) {
-            if (!mbar_wait_warp(zempty, zph ^ 1u, ctl)) { ok = false; return; }
-            tc_fence_after();
-            for (int ks = 0; ks < steps; ++ks) {
+          // K steps [ks0, ks1) of a Z product of `steps`
+          auto z_product = [&](int ks0, int ks1, int steps) {
+            if (ks0 == 0) {
+              if (!mbar_wait_warp(zempty, zph ^ 1u, ctl)) { ok = false; return; }
+              tc_fence_after();
+            }
+            for (int ks = ks0; ks < ks1; ++ks) {
               if (!mbar_wait_warp(full_bar(stage), phase, ctl)) { ok = false; return; }
               tc_fence_after();
               const uint32_t so = static_cast<uint32_t>(stage) * (kStageBytes >> 4);
@@ -744,8 +798,10 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
               if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            if (leader) umma_commit_pair(zfull);
-            zph ^= 1u;
+            if (ks1 == steps) {
+              if (leader) umma_commit_pair(zfull);
+              zph ^= 1u;
+            }
           };
           auto accumulate = [&](int e_to) {
             for (; ok && at.e < e_to; at.next()) {
@@ -783,14 +839,14 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           };
-          if (job) z_product(s.nk);
-          if (!ok || !consume) continue;
           const int e_lo = r > 0 ? (r - 1) * g : 0;
           const int e_end = r > 0 ? min(r * g, s.E) : 0;
-          const int e_mid = split_point<kMode>(s, e_lo, e_end);
-          accumulate(e_mid);
-          if (kMode == GM_KL && ok && job) z_product(s.nk2);
-          if (ok) accumulate(e_end);
+          const Round rd = plan_round<kMode>(s, e_lo, e_end);
+          for (int b = 0; ok && b <= rd.count; ++b) {
+            const Step st = round_step<kMode>(s, rd, b, e_end);
+            if (job && st.z1 > st.z0) z_product(st.z0, st.z1, st.steps);
+            if (ok && consume) accumulate(st.until);
+          }
         }
         // arrives once every MMA issued above has completed (bounded wait that
         // ignores the abort flag: it only waits for work already in flight)
@@ -913,10 +969,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (kMode == GM_B && s.ni == 0) {
       // no masked rows: dW is zero on this member's columns of its outer tiles
-      float acc[4][32] = {};
+      const int vecs = s.cw * (p.out_dtype == OLIVE_DTYPE_F32 ? 4 : 2) / 16;
       for (int rp = s.pg; 2 * rp < s.no; rp += s.npg) {
         const int v = outer_of(p, s, rp) * kBM + row;
-        store_output(v < p.V ? v : -1, acc);
+        if (v >= p.V) continue;
+        uint4* o = reinterpret_cast<uint4*>(static_cast<uint8_t*>(p.out) +
+                                            (p.out_dtype == OLIVE_DTYPE_F32 ? 4 : 2) *
+                                                (static_cast<size_t>(v) * p.d + s.c0));
+        for (int c = half; c < vecs; c += 2) o[c] = make_uint4(0, 0, 0, 0);
       }
     }
 
@@ -926,7 +986,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float s_coef = s.coef;
     for (int r = 0; ok && r <= nr; ++r) {
       const int j = r * g + s.m;
-      if (r < nr && j < s.E) {
+      const int e_lo = r > 0 ? (r - 1) * g : 0;
+      const int e_end = r > 0 ? min(r * g, s.E) : 0;
+      const Round rd = plan_round<kMode>(s, e_lo, e_end);
+      // the outer tiles that close before the round's last boundary, then the Z
+      // tile, then the others
+      for (int part = kMode == GM_B && rd.count > 0 ? 0 : 1; ok && part < 2; ++part) {
+      if (part == 1 && r < nr && j < s.E) {
         // ---------------------------------------------------- Z epilogue
         const Pos at = locate(s, j);
         const int k = at.k;
@@ -1170,10 +1236,10 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (kMode == GM_B) named_bar_sync(1, kEpi);
         }
       }
-      if (!consume || r == 0) continue;
+      if constexpr (!consume) break;
+      if (r == 0) continue;
       // ------------------------------------------- outer tiles completed
-      const int e_end = min(r * g, s.E);
-      for (int e = (r - 1) * g; ok && e < e_end; ++e) {
+      for (int e = part == 0 ? e_lo : rd.last; ok && e < (part == 0 ? rd.last : e_end); ++e) {
         const Pos at = locate(s, e);
         if (!closes(s, e, at.k)) continue;
         const int o = outer_of(p, s, at.rp);
@@ -1337,6 +1403,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           store_output(rw.valid ? rw.t : -1, acc);
         }
+      }
       }
     }
   }
