@@ -66,6 +66,7 @@ struct FwdWs {
   float* part_s;  // [part_rows]
   float* zy;      // [Tpad]
   float* nll;     // [Tpad]
+  uint32_t* done; // finished blocks of the finalize kernel; null when min_parts is 0
 };
 size_t fwd_ws_bytes(int64_t T, int64_t d, int min_parts = kMinParts);
 FwdWs carve_fwd(void* ws, int64_t T, int64_t d, int min_parts = kMinParts);
@@ -181,7 +182,7 @@ struct GroupArgs {
   const float* grad_loss;
   int lse_known, redo, write_fwd;
   const float* lse_in;
-  float *rref, *rmax, *part_s, *part_m, *zy, *pyb, *logp, *lse, *nll;
+  float *rref, *rmax, *part_s, *part_m, *zy, *pyb, *logp, *lse, *nll, *loss;
   uint32_t* redo_list;
   uint32_t* outer_ctr;
   void* ring;

@@ -293,7 +293,10 @@ __global__ void __launch_bounds__(128)
                         const int32_t* __restrict__ targets, int T, int V, int vt, int ctas, int min_parts,
                         const float* __restrict__ part_m, const float* __restrict__ part_s,
                         const float* __restrict__ zy, float* __restrict__ logp,
-                        float* __restrict__ lse, float* __restrict__ nll, int32_t* dev_status) {
+                        float* __restrict__ lse, float* nll, uint32_t* done, int reduction,
+                        float* __restrict__ loss, int32_t* dev_status) {
+  __shared__ double part[4];
+  __shared__ bool last;
   const int n = read_n_rows(n_rows, T, nullptr);
   const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, min_parts));
   const int lane = threadIdx.x & 31;
@@ -322,6 +325,25 @@ __global__ void __launch_bounds__(128)
     logp[t] = lp;
     lse[t] = l;
     nll[r] = -lp;
+  }
+  // the last block to finish adds the loss terms up in a fixed order
+  if (!done) return;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double acc = 0.0;
+#pragma unroll 4
+  for (int r = threadIdx.x; r < n; r += 128) acc += static_cast<double>(__ldcg(nll + r));
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    acc = (part[0] + part[1]) + (part[2] + part[3]);
+    if (reduction == OLIVE_REDUCE_MEAN) acc = n > 0 ? acc / n : 0.0;
+    *loss = static_cast<float>(acc);
   }
 }
 
@@ -454,6 +476,7 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
   q.gather(hidden, d, w.hc);
   q.fill(logp, sizeof(float) * T);
   q.fill(lse, sizeof(float) * T);
+  q.fill(w.done, sizeof(uint32_t));
   olive_status st = launch_prepare(c, q, rows, n_rows, T, dev_status);
   if (st != OLIVE_OK) return st;
 
@@ -483,12 +506,10 @@ olive_status launch_logprob_fwd(const Ctx& c, const void* hidden, const void* W,
   const int vt = (V + FwdKern::kBN - 1) / FwdKern::kBN;
   const int blocks = static_cast<int>(std::min<int64_t>(ceil_div(T, 4), c.num_sms * 16));
   fwd_finalize_kernel<<<blocks, 128, 0, c.stream>>>(n_rows, rows, targets, T, V, vt, c.num_sms, min_parts,
-                                                     w.part_m, w.part_s, w.zy, logp, lse, w.nll,
-                                                     dev_status);
+                                                     w.part_m, w.part_s, w.zy, logp, lse, w.nll, w.done,
+                                                     reduction, loss, dev_status);
   if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
-  loss_reduce_kernel<<<1, 1024, 0, c.stream>>>(n_rows, T, w.nll, reduction, loss);
-  if (cudaGetLastError() != cudaSuccess) return OLIVE_ERR_CUDA;
-  return OLIVE_OK;
+  return w.done ? OLIVE_OK : launch_loss_reduce(c, n_rows, T, w.nll, reduction, loss);
 }
 
 olive_status launch_topk_fwd(const Ctx& c, const void* hidden, const void* W, const int32_t* rows,

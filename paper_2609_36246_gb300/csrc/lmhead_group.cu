@@ -127,7 +127,8 @@ constexpr int kEpi = 32 * kEpiWarps; // epilogue threads: two per accumulator ro
 constexpr int kProducerWarp = kEpiWarps;
 constexpr int kMmaWarp = kEpiWarps + 1;
 constexpr int kSignalWarp = kEpiWarps + 2;  // posts the members' "tile copied" counts
-constexpr int kThreads = 32 * (kEpiWarps + 4);  // three whole warpgroups (warp 11 idles)
+constexpr int kLossWarp = kEpiWarps + 3;
+constexpr int kThreads = 32 * (kEpiWarps + 4);  // three whole warpgroups
 // Registers a thread: 168 at launch (65536 / 384 threads); the warpgroup of
 // the producer, MMA and signal warps hands most of its share to the two of
 // the epilogue, whose 128 held accumulator values otherwise spill (the L1 left
@@ -188,6 +189,7 @@ struct GroupParams {
   float* logp;              // [T]
   float* lse;               // [T]
   float* nll;               // [Tpad] per-row loss terms
+  float* loss;              // GM_B: their sum (or mean), null when not asked for
   uint32_t* redo_list;      // [1 + rt]: count, then row tiles
   uint32_t* outer_ctr;      // [rt] pass A group barrier (one array per GM_A launch)
   __nv_bfloat16* ring;      // [ngroups][R][128 x 256] exchange tiles (swizzled images)
@@ -756,6 +758,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       __syncwarp();
+    } else if (warp == kLossWarp) {
+      // a warp that has nothing else to do, in one CTA: the loss from pass A's
+      // per-row terms, in a fixed order (a launch of its own took 5 us and a
+      // gap at the end of every step)
+      if (kMode == GM_B && p.loss && blockIdx.x == gridDim.x - 1) {
+        double acc = 0.0;
+        for (int rc = lane; rc < s.n; rc += 32) acc += static_cast<double>(p.nll[rc]);
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (p.reduction == OLIVE_REDUCE_MEAN) acc = s.n > 0 ? acc / s.n : 0.0;
+        if (lane == 0) *p.loss = static_cast<float>(acc);
+      }
     } else if (warp == kMmaWarp) {
       // a lane of the even CTA's MMA warp issues the pair's MMAs (M = 256: 128
       // rows in each CTA's TMEM); the odd CTA's only holds its TMEM allocation
@@ -1647,6 +1660,7 @@ olive_status launch_group(const Ctx& c, int mode, const void* hc, const void* W,
   p.logp = a.logp;
   p.lse = a.lse;
   p.nll = a.nll;
+  p.loss = a.loss;
   p.redo_list = a.redo_list;
   p.outer_ctr = a.outer_ctr + (mode == GM_A && a.redo ? (T + kBM - 1) / kBM : 0);
   p.ring = static_cast<__nv_bfloat16*>(a.ring);
@@ -1756,10 +1770,11 @@ olive_status launch_loss_group(const Ctx& c, const void* hidden, const void* W,
         return st;
       a.redo = 0;
     }
+    a.loss = fwd && cb == 0 ? loss : nullptr;
     if ((st = launch_group(c, GM_B, w.hc, W, T, d, V, a, cb, ce, w.ring_ctr + 2 * rw, &mb)) != OLIVE_OK)
       return st;
   }
-  return fwd ? launch_loss_reduce(c, n_rows, T, w.nll, reduction, loss) : OLIVE_OK;
+  return OLIVE_OK;
 }
 
 }  // namespace olive

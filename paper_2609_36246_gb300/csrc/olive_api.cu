@@ -147,6 +147,7 @@ static FwdWs carve_fwd_impl(void* ws, int64_t T, int64_t d, int min_parts, size_
   w.part_s = static_cast<float*>(c.take(4ull * part_rows(Tpad, min_parts)));
   w.zy = static_cast<float*>(c.take(4ull * Tpad));
   w.nll = static_cast<float*>(c.take(4ull * Tpad));
+  w.done = min_parts > 0 ? static_cast<uint32_t*>(c.take(4)) : nullptr;
   if (total) *total = c.off;
   return w;
 }
