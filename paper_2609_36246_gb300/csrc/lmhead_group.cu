@@ -995,7 +995,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     int cur_rp = -1;            // pass A: the row pair of the running partials
     RowA ra{false, -1, -1, 0.f};
-    float run_s = 0.f, run_m = -INFINITY;  // of 2^(x - R) and of x - R
+    float run_m = -INFINITY;  // of x - R
     const float s_coef = s.coef;
     for (int r = 0; ok && r <= nr; ++r) {
       const int j = r * g + s.m;
@@ -1043,6 +1043,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!named_bar_and(1, kEpi, go && mbar_wait(zfull, zph, ctl))) { ok = false; break; }
         zph ^= 1u;
         tc_fence_after();
+        float pv_all[4][32];  // pass A: 2^(x - R) of this thread's columns
+        bool fresh = false;   // pass A: the member's first tile of the outer tile
         uint8_t* img = ring_bytes + (ring0 + slot) * static_cast<size_t>(kXTile);
         if (!OLIVE_DCHECK(p.dev_status, !consume || static_cast<int64_t>(ring0 + slot) < p.ring_tiles))
           img = nullptr;
@@ -1175,22 +1177,28 @@ __global__ void __launch_bounds__(kThreads, 1)
             put(h, gv);
           }
         } else {
-          if (at.rp != cur_rp) {
+          fresh = at.rp != cur_rp;
+          if (fresh) {
             cur_rp = at.rp;
             ra = load_row_a(p, s, o * kBM + row);
-            run_s = 0.f;
             run_m = -INFINITY;
           }
           const int v0 = k * kZN;
-#pragma unroll 1
-          for (int h = hbeg; h < hend; ++h) {
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            const int h = hbeg + b;
+            if (h >= hend) {
+#pragma unroll
+              for (int c = 0; c < 32; ++c) pv_all[b][c] = 0.f;
+              continue;
+            }
             uint32_t a[32];
             tmem_ld_32x32b_x32(zaddr + h * 32, a);
             tmem_ld_wait();
             drained(h);
-            float pv[32];
-            // two running sums and maxima of x - R: shorter chains
-            float s1 = 0.f, m1 = -INFINITY;
+            float(&pv)[32] = pv_all[b];
+            // (two running maxima of x - R: shorter chains)
+            float m1 = -INFINITY;
             if (h * 32 + 32 <= kv) {
 #pragma unroll
               for (int c = 0; c < 32; c += 2) {
@@ -1200,8 +1208,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 m1 = fmaxf(m1, x1);
                 pv[c] = fast_exp2(x0);
                 pv[c + 1] = fast_exp2(x1);
-                run_s += pv[c];
-                s1 += pv[c + 1];
               }
             } else {
 #pragma unroll
@@ -1210,10 +1216,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
                 m1 = in ? fmaxf(m1, x0) : m1;
                 pv[c] = in ? fast_exp2(x0) : 0.f;
-                s1 += pv[c];
               }
             }
-            run_s += s1;
             run_m = fmaxf(run_m, m1);
             const int yo = ra.y - (v0 + h * 32);
             if (kMode == GM_A && yo >= 0 && yo < 32) {
@@ -1237,7 +1241,6 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
           named_bar_sync(1, kEpi);
         } else {
-          if (kMode == GM_A && ra.valid) put_sums(j, at.rp, o, run_s, run_m + ra.R);
           // publish the warp's part of the tile once its copies are complete
           if (lane == 0) {
             bulk_wait();
@@ -1247,6 +1250,23 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           // the row metadata of this tile is read: the next one's may be written
           if (kMode == GM_B) named_bar_sync(1, kEpi);
+          if (kMode == GM_A) {
+            // The row's sum over this member's tiles is one chain in column
+            // order, which the first half's thread hands to the second's in
+            // shared memory.  (One sum a half rounds less where a large term
+            // stands early, but by other amounts than the target's logit does,
+            // and the mean loss, in which the two nearly cancel, was 1.5 to 1.7
+            // times as far from 64 bits.)
+            if (half) named_bar_sync(2, kEpi);
+            float sum = !half && fresh ? 0.f : meta_l[row];
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+#pragma unroll
+              for (int c = 0; c < 32; ++c) sum += pv_all[b][c];
+            meta_l[row] = sum;
+            if (!half) named_bar_arrive(2, kEpi);
+            if (ra.valid) put_sums(j, at.rp, o, half ? sum : 0.f, run_m + ra.R);
+          }
         }
       }
       if constexpr (!consume) break;

@@ -415,6 +415,10 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* addr) {
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
+// Arrival without waiting at a barrier that others of the `count` threads sync on.
+__device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
 // Barrier over `count` threads that returns the AND of every thread's `v`,
 // so a group can take one decision together.
 __device__ __forceinline__ bool named_bar_and(uint32_t id, uint32_t count, bool v) {
