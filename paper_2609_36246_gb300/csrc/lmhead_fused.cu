@@ -907,6 +907,7 @@ __global__ void __launch_bounds__(256)
 //      Where lam is out of range (|lam| < 2^-96, |A| < 2^-20) or a half tile
 //      kept its own maximum, the row is rewritten as G itself (lam = 1).
 
+constexpr int kDotRows = 4;  // dot products taken together
 constexpr int kTkCand = 24;  // most candidates taken to the exact recomputation (K <= 16)
 
 __device__ __forceinline__ float dot8(uint4 x, uint4 y, float s) {
@@ -922,27 +923,40 @@ __device__ __forceinline__ float dot8(uint4 x, uint4 y, float s) {
   return s;
 }
 
-// h . w over d8 16-byte groups, split across the warp; four groups per lane
-// in flight
-__device__ __forceinline__ float dot_row_bf16(const uint4* __restrict__ h,
-                                              const uint4* __restrict__ w, int d8, int lane) {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+// h . w[q] for N rows at once, over d8 16-byte groups split across the warp:
+// every lane has 4 (N + 1) loads in flight.  (One row at a time, with 8, a
+// masked row's 24 candidates and 16 teacher rows took 40 x 5 us one after the
+// other: the kernel is bound by that chain, one warp a row.)
+template <int N>
+__device__ __forceinline__ void dot_rows_bf16(const uint4* __restrict__ h,
+                                              const uint4* const (&w)[N], int d8, int lane,
+                                              float (&out)[N]) {
+  float s[N][4] = {};
   int c = lane;
   for (; c + 96 < d8; c += 128) {
-    const uint4 w0 = __ldg(w + c), w1 = __ldg(w + c + 32), w2 = __ldg(w + c + 64),
-                w3 = __ldg(w + c + 96);
-    const uint4 h0 = __ldg(h + c), h1 = __ldg(h + c + 32), h2 = __ldg(h + c + 64),
-                h3 = __ldg(h + c + 96);
-    s0 = dot8(h0, w0, s0);
-    s1 = dot8(h1, w1, s1);
-    s2 = dot8(h2, w2, s2);
-    s3 = dot8(h3, w3, s3);
-  }
-  for (; c < d8; c += 32) s0 = dot8(__ldg(h + c), __ldg(w + c), s0);
-  float s = (s0 + s1) + (s2 + s3);
+    uint4 wv[N][4], hv[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
+    for (int u = 0; u < 4; ++u) {
+      hv[u] = __ldg(h + c + 32 * u);
+#pragma unroll
+      for (int q = 0; q < N; ++q) wv[q][u] = __ldg(w[q] + c + 32 * u);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < N; ++q) s[q][u] = dot8(hv[u], wv[q][u], s[q][u]);
+  }
+  for (; c < d8; c += 32) {
+    const uint4 hv = __ldg(h + c);
+#pragma unroll
+    for (int q = 0; q < N; ++q) s[q][0] = dot8(hv, __ldg(w[q] + c), s[q][0]);
+  }
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    out[q] = (s[q][0] + s[q][1]) + (s[q][2] + s[q][3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) out[q] += __shfl_xor_sync(0xffffffffu, out[q], o);
+  }
 }
 
 // Inserts (v, id) into a lane-local list of N entries sorted by (value
@@ -1058,11 +1072,29 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
       tv[j] = -INFINITY;
       ti[j] = INT_MAX;
     }
-    for (int j = lane; j < a.vh; j += 32) {
-      const float mj = tmx[j];
-      own |= mj - R > kRefMax;  // the forward tiles' own test
-      lse_merge(m, sum, zm[j], zs[j]);
-      if (mj > tv[kTkCand - 1]) lane_list_insert(tv, ti, mj, j);
+    // (four half tiles a lane at a time: one at a time, the loads' latency
+    // stood 2 x 37 times in the row's chain at V = 151936)
+    for (int base = 0; base < a.vh; base += 128) {
+      float mj[4], zj[4], sj[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = base + 32 * u + lane;
+        const bool in = j < a.vh;
+        mj[u] = in ? tmx[j] : -INFINITY;
+        zj[u] = in ? zm[j] : -INFINITY;
+        sj[u] = in ? zs[j] : 0.f;
+      }
+#pragma unroll 1
+      for (int u = 0; u < 4; ++u) {
+        const int j = base + 32 * u + lane;
+        if (j >= a.vh) break;
+        const float mu = u == 0 ? mj[0] : u == 1 ? mj[1] : u == 2 ? mj[2] : mj[3];
+        const float zu = u == 0 ? zj[0] : u == 1 ? zj[1] : u == 2 ? zj[2] : zj[3];
+        const float su = u == 0 ? sj[0] : u == 1 ? sj[1] : u == 2 ? sj[2] : sj[3];
+        own |= mu - R > kRefMax;  // the forward tiles' own test
+        lse_merge(m, sum, zu, su);
+        if (mu > tv[kTkCand - 1]) lane_list_insert(tv, ti, mu, j);
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1089,9 +1121,20 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
       li[j] = INT_MAX;
     }
     __nv_bfloat16* grow = a.g + static_cast<size_t>(r) * a.ldg;
+    unsigned reach[4];
     for (int base = 0; base < a.vh; base += 32) {
-      const int j = base + lane;
-      unsigned b = __ballot_sync(0xffffffffu, j < a.vh && tmx[j] >= tau);
+      if ((base & 96) == 0) {
+        bool over[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int j = base + 32 * u + lane;
+          over[u] = j < a.vh && tmx[j] >= tau;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) reach[u] = __ballot_sync(0xffffffffu, over[u]);
+      }
+      const int u4 = (base >> 5) & 3;
+      unsigned b = u4 == 0 ? reach[0] : u4 == 1 ? reach[1] : u4 == 2 ? reach[2] : reach[3];
       while (b) {
         int js[4];
 #pragma unroll
@@ -1136,11 +1179,21 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
     // 3. exact logits of the candidates, then the K largest by rank
     const uint4* hs_in = a.h_s + static_cast<size_t>(t) * a.ds8;
     float l = -INFINITY;
-    for (int k = 0; k < C; ++k) {
-      const int u = __shfl_sync(0xffffffffu, cid, k);
-      if (u < 0) break;  // the list ends (fewer columns than candidates)
-      const float x = dot_row_bf16(hs_in, a.W_s + static_cast<size_t>(u) * a.ds8, a.ds8, lane);
-      if (lane == k) l = x * a.inv_tau - lse_s;
+    for (int k = 0; k < C; k += kDotRows) {
+      const uint4* w[kDotRows];
+      int u[kDotRows];
+#pragma unroll
+      for (int e = 0; e < kDotRows; ++e) {
+        u[e] = __shfl_sync(0xffffffffu, cid, k + e);  // (C <= 24: lanes in range)
+        if (k + e >= C) u[e] = -1;
+        w[e] = a.W_s + static_cast<size_t>(u[e] < 0 ? 0 : u[e]) * a.ds8;
+      }
+      if (u[0] < 0) break;  // the list ends (fewer columns than candidates)
+      float x[kDotRows];
+      dot_rows_bf16(hs_in, w, a.ds8, lane, x);
+#pragma unroll
+      for (int e = 0; e < kDotRows; ++e)
+        if (lane == k + e && u[e] >= 0) l = x[e] * a.inv_tau - lse_s;
     }
     int rank = 0;
     for (int k = 0; k < C; ++k) {
@@ -1165,11 +1218,21 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
     const uint4* ht = a.h_t + static_cast<size_t>(t) * a.dt8;
     const float lse_t = a.t_lse[t];
     float q = 0.f;
-    for (int j = 0; j < K; ++j) {
-      const int u = __shfl_sync(0xffffffffu, sid, j);
-      if (u < 0) continue;
-      const float x = dot_row_bf16(ht, a.W_t + static_cast<size_t>(u) * a.dt8, a.dt8, lane);
-      if (lane == j) q = x * a.inv_tau - lse_t;
+    for (int j = 0; j < K; j += kDotRows) {
+      const uint4* w[kDotRows];
+      int u[kDotRows];
+#pragma unroll
+      for (int e = 0; e < kDotRows; ++e) {
+        u[e] = __shfl_sync(0xffffffffu, sid, j + e);
+        if (j + e >= K) u[e] = -1;
+        w[e] = a.W_t + static_cast<size_t>(u[e] < 0 ? 0 : u[e]) * a.dt8;
+      }
+      if (u[0] < 0) break;  // (the ids of S come first)
+      float x[kDotRows];
+      dot_rows_bf16(ht, w, a.dt8, lane, x);
+#pragma unroll
+      for (int e = 0; e < kDotRows; ++e)
+        if (lane == j + e && u[e] >= 0) q = x[e] * a.inv_tau - lse_t;
     }
     const bool in_k = lane < K && sid >= 0;
     const float p = in_k ? expf(slp) : 0.f;
