@@ -63,7 +63,8 @@ struct OpdKern {
   static constexpr int kStages = 4;
   static constexpr int kAccBufs = 1;
   static constexpr int kEpiWarps = 8;
-  static constexpr int kEpiSmem = 0;
+  // each (row, half)'s 16th values so far and the unit they belong to
+  static constexpr int kEpiSmem = 2 * 2 * 128 * 8;
   // segments per row tile (each writes two halves)
   static __device__ int seg_cap(int n) { return split_cap((n + 127) / 128, kMinPartsOpd) / 2; }
 
@@ -115,15 +116,28 @@ struct OpdKern {
   }
 
   struct Epi {
-    int r, sg, half;
+    int r, sg, half, unit;
+    // [2]: the student list's and the teacher list's bound of this row's halves,
+    // value bits and unit number in one 64-bit word
+    volatile unsigned long long *own, *peer;
+    float bound_s, bound_t;
     float ms, ss, es, mt, st, A;
     float sv[kTopMax], sx[kTopMax], tv[kTopMax];
     int si[kTopMax], ti[kTopMax];
 
-    __device__ void init(uint8_t*, int prt) { half = prt; }
+    __device__ void init(uint8_t* smem, int prt) {
+      half = prt;
+      volatile unsigned long long* base =
+          reinterpret_cast<volatile unsigned long long*>(smem) + 2 * (threadIdx.x & 127);
+      own = base + 256 * half;
+      peer = base + 256 * (1 - half);
+      own[0] = own[1] = ~0ull;
+    }
     __device__ void begin(const Params& p, const Sched& s, int u, int row) {
       int i;
       unit_pos(p, s, u, i, sg);
+      unit = u;
+      bound_s = bound_t = -INFINITY;
       r = i * kBM + row;
       ms = mt = -INFINITY;
       ss = es = st = A = 0.f;
@@ -134,67 +148,71 @@ struct OpdKern {
       }
     }
 
+    // kFull: all 32 columns are below V
+    template <bool kFull>
     __device__ __forceinline__ void chunk(const Params& p, const uint32_t (&a)[32],
-                                          const uint32_t (&b)[32], int col0) {
-      const int nvalid = p.V - col0;
+                                          const uint32_t (&b)[32], int col0, uint32_t& cand_s,
+                                          uint32_t& cand_t) {
+      const int nvalid = kFull ? 32 : p.V - col0;
+      // raw maxima (the scale is positive), then one fma an exponent
       float cs = -INFINITY, ct = -INFINITY;
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         if (k < nvalid) {
-          cs = fmaxf(cs, __uint_as_float(a[k]) * p.scale2);
-          ct = fmaxf(ct, __uint_as_float(b[k]) * p.scale2);
+          cs = fmaxf(cs, __uint_as_float(a[k]));
+          ct = fmaxf(ct, __uint_as_float(b[k]));
         }
       }
-      const float msn = fmaxf(ms, cs);
-      const float mtn = fmaxf(mt, ct);
+      const float msn = fmaxf(ms, cs * p.scale2);
+      const float mtn = fmaxf(mt, ct * p.scale2);
       float e_s = 0.f, e_e = 0.f, e_t = 0.f, e_a = 0.f;
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
         const bool ok = k < nvalid;
-        const float xs = __uint_as_float(a[k]) * p.scale2;
-        const float xt = __uint_as_float(b[k]) * p.scale2;
-        const float qs = ok ? fast_exp2(xs - msn) : 0.f;
-        const float qt = ok ? fast_exp2(xt - mtn) : 0.f;
+        const float zs = __uint_as_float(a[k]), zt = __uint_as_float(b[k]);
+        const float qs = ok ? fast_exp2(fmaf(zs, p.scale2, -msn)) : 0.f;
+        const float qt = ok ? fast_exp2(fmaf(zt, p.scale2, -mtn)) : 0.f;
         e_s += qs;
-        e_e += qs * xs;
         e_t += qt;
-        e_a += p.reverse ? qs * (xs - xt) : qt * (xt - xs);
+        e_e = ok ? fmaf(qs, zs, e_e) : e_e;
+        e_a = ok ? fmaf(p.reverse ? qs : -qt, zs - zt, e_a) : e_a;
       }
       const float rs = fast_exp2(ms - msn);
       const float rt = fast_exp2(mt - mtn);
       ss = ss * rs + e_s;
-      es = es * rs + e_e;
+      es = es * rs + e_e * p.scale2;
       st = st * rt + e_t;
-      A = A * (p.reverse ? rs : rt) + e_a;
+      A = A * (p.reverse ? rs : rt) + e_a * p.scale2;
       ms = msn;
       mt = mtn;
       // a unit visits its ids in ascending order, so a new id is larger than
       // every listed one: values alone decide the candidates and their places
-      uint32_t cand_s = 0u, cand_t = 0u;
       const float last_s = sv[kTopMax - 1], last_t = tv[kTopMax - 1];
+      if (cs > last_s && cs >= bound_s) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const bool ok = k < nvalid;
-        if (ok && __uint_as_float(a[k]) > last_s) cand_s |= 1u << k;
-        if (ok && __uint_as_float(b[k]) > last_t) cand_t |= 1u << k;
+        for (int k = 0; k < 32; ++k) {
+          const float v = __uint_as_float(a[k]);
+          if (k < nvalid && v > last_s && v >= bound_s) cand_s |= 1u << k;
+        }
       }
-#pragma unroll 1
-      while (cand_s) {
-        const int k = __ffs(cand_s) - 1;
-        cand_s &= cand_s - 1u;
-        const float v = __uint_as_float(pick32(a, k));
-        if (v > sv[kTopMax - 1]) topk_insert3_asc(sv, si, sx, v, col0 + k, __uint_as_float(pick32(b, k)));
-      }
-#pragma unroll 1
-      while (cand_t) {
-        const int k = __ffs(cand_t) - 1;
-        cand_t &= cand_t - 1u;
-        const float w = __uint_as_float(pick32(b, k));
-        if (w > tv[kTopMax - 1]) topk_insert_asc(tv, ti, w, col0 + k);
+      if (ct > last_t && ct >= bound_t) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+          const float v = __uint_as_float(b[k]);
+          if (k < nvalid && v > last_t && v >= bound_t) cand_t |= 1u << k;
+        }
       }
     }
 
     __device__ void tile(const Params& p, const Sched&, int, int, const TileC& tc, uint32_t taddr) {
+      // The other half of the row lists 16 logits no smaller than its 16th, so
+      // what is below that cannot be among the row's 16 largest: fewer
+      // insertions, which are what this epilogue spends most of its time on.
+      // (The two halves are not in step: a bound counts only if it carries this
+      // unit's number, and a stale one is merely lower.)
+      const unsigned long long ps = peer[0], pt = peer[1];
+      if (ps >> 32 == static_cast<uint32_t>(unit)) bound_s = __uint_as_float(static_cast<uint32_t>(ps));
+      if (pt >> 32 == static_cast<uint32_t>(unit)) bound_t = __uint_as_float(static_cast<uint32_t>(pt));
 #pragma unroll 1
       for (int c = half * (kBN / 2); c < (half + 1) * (kBN / 2); c += 32) {
         const int col0 = tc.n0 + c;
@@ -203,8 +221,27 @@ struct OpdKern {
         tmem_ld_32x32b_x32(taddr + c, a);
         tmem_ld_32x32b_x32(taddr + kBN + c, b);
         tmem_ld_wait();
-        chunk(p, a, b, col0);
+        uint32_t cand_s = 0u, cand_t = 0u;
+        if (col0 + 32 <= p.V) chunk<true>(p, a, b, col0, cand_s, cand_t);
+        else chunk<false>(p, a, b, col0, cand_s, cand_t);
+#pragma unroll 1
+        while (cand_s) {
+          const int k = __ffs(cand_s) - 1;
+          cand_s &= cand_s - 1u;
+          const float v = __uint_as_float(pick32(a, k));
+          if (v > sv[kTopMax - 1]) topk_insert3_asc(sv, si, sx, v, col0 + k, __uint_as_float(pick32(b, k)));
+        }
+#pragma unroll 1
+        while (cand_t) {
+          const int k = __ffs(cand_t) - 1;
+          cand_t &= cand_t - 1u;
+          const float w = __uint_as_float(pick32(b, k));
+          if (w > tv[kTopMax - 1]) topk_insert_asc(tv, ti, w, col0 + k);
+        }
       }
+      const unsigned long long tag = static_cast<unsigned long long>(static_cast<uint32_t>(unit)) << 32;
+      own[0] = tag | __float_as_uint(sv[kTopMax - 1]);
+      own[1] = tag | __float_as_uint(tv[kTopMax - 1]);
     }
 
     __device__ void end(const Params& p, const Sched& s, int) {
