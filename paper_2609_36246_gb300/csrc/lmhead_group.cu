@@ -1365,15 +1365,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         float lse2 = rw.R, mx = -INFINITY;
         if (!p.lse_known && rw.valid) {
           float sum = 0.f;
-          for (int c = run_lo; c <= run_hi; ++c) {
-            const size_t from = split ? tail_row(c + t, 0) : rc;
-            const size_t stride = split ? 2 * kBM : Tpad;
-            const float* ps = split ? p.tail_s : p.part_s;
-            const float* pm = split ? p.tail_m : p.part_m;
-            for (int mm = 0; mm < 2 * g; ++mm) {
-              sum += __ldcg(ps + from + mm * stride);
-              mx = fmaxf(mx, __ldcg(pm + from + mm * stride));
-            }
+          // (a split row pair's slots stand one after the other)
+          const size_t from = split ? tail_row(run_lo + t, 0) : rc;
+          const size_t stride = split ? 2 * kBM : Tpad;
+          const float* ps = (split ? p.tail_s : p.part_s) + from;
+          const float* pm = (split ? p.tail_m : p.part_m) + from;
+          const int count = 2 * g * (run_hi - run_lo + 1);
+#pragma unroll 8
+          for (int e2 = 0; e2 < count; ++e2) {
+            sum += __ldcg(ps + e2 * stride);
+            mx = fmaxf(mx, __ldcg(pm + e2 * stride));
           }
           lse2 = rw.R + log2f(sum);
         }
