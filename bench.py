@@ -327,8 +327,8 @@ def run_ours(args, world, rank, local):
     # unless a row's maximum exceeds its reference by 2^64, pass B: dW).  Its
     # algorithmic work per call is the forward product plus dH and dW,
     # 6 N_mask d V; it executes 8 N_mask d V (each pass computes the logits).
-    # The call is bracketed by events on its stream, so the row gather, the
-    # memsets and the loss reduction count against it.  The call lasts tens of
+    # The call is bracketed by events on its stream, so the launch that copies
+    # the rows and fills the buffers counts against it.  The call lasts tens of
     # milliseconds, so the denominator is the burst peak.
     fb_flops = counted
     ach_fb = fb_flops / (fb_ms / 1e3) / 1e12
@@ -337,8 +337,8 @@ def run_ours(args, world, rank, local):
     # algorithmic DRAM bytes of a call: W read, hc read (once per pass), dW and
     # dH written (bf16)
     alg_bytes = 2.0 * V * d + 2 * 2.0 * N_mask * d + 2.0 * V * d + 2.0 * N_mask * d
-    # splice (scan, fill) + row gather + 4 lmhead_group_kernel + loss reduce
-    launches = 2 + 1 + 4 + 1
+    # splice fill (at most 2048 sequences) + prepare + 4 lmhead_group_kernel
+    launches = 1 + 1 + 4
 
     two_call = slab = None
     if not args.no_extra:
@@ -396,7 +396,7 @@ def run_ours(args, world, rank, local):
                      "executed_frac": 8.0 * N_mask * d * V / (fb_ms / 1e3) / 1e12 / burst,
                      "kernel_rev": rev,
                      "note": "per olive_token_loss_fwd_bwd call (its lmhead_group_kernel launches, "
-                             "timed with the gather, memsets and loss reduction around them); "
+                             "timed with the launch that prepares its buffers); "
                              "traffic is DRAM bytes of those launches from an ncu capture"},
         "two_call_path": two_call,
         "slab_path": slab,
