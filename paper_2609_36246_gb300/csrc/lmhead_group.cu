@@ -86,12 +86,15 @@
 // accumulator is taken into registers (up to 128 a thread) and handed back
 // before it is converted and stored.  With four warps that stored 16-byte
 // pieces from registers and held the accumulator until its rows were stored,
-// the training step took 3.93 ms against 3.73 ms now (1024 masked rows,
-// d = 4096, V = 151936: outer tiles of pass B last 4 inner tiles) and
-// 4.48 -> 4.04 ms with 1677 rows, d = 2560, V = 100003, fp32 gradients; the
-// divergence with two N = 128 products side by side in the Z accumulator
-// (60 % of the tensor rate) 21.8 against 18.6 ms (4096 rows, d_s = 4096,
-// d_t = 5120).  Every dependency
+// the training step took 3.93 against 3.73 ms (1024 masked rows, d = 4096,
+// V = 151936: outer tiles of pass B last 4 inner tiles; 3.4 ms now) and
+// forward call + backward call 4.48 against 4.04 ms (1677 rows, d = 2560,
+// V = 100003, fp32 gradients; 3.07 ms now); the divergence with two N = 128
+// products side by side in the Z accumulator (60 % of the tensor rate) took
+// 21.8 against 18.6 ms (4096 rows, d_s = 4096, d_t = 5120; 17.4 ms now).
+// What bounds it now: the tensor pipe and, from some thousand rows on, the
+// power cap (16384 rows: pipe 90 % active in pass A, 87 % in pass B); at a few
+// hundred rows the rounds' exchange latency.  Every dependency
 // points to a tile of an earlier round, every CTA is resident at once (the
 // grid is one CTA per SM; the host checks that the GPU holds all its
 // clusters), and every wait is bounded (OLIVE_ERR_TIMEOUT on expiry).  A
@@ -236,9 +239,9 @@ struct GroupParams {
 // a quarter of an inner tile's time at the least, so runs are at least
 // sqrt(ni / 4) long and the tail stays whole where that cost is not below ni.
 // Pass A, whole -> split: 365 rows, d = 2048, V = 151936 (2 row pairs for 8
-// pair-groups) 1580 -> 545 us; 1677 rows, d = 2560, V = 100003 (7 for 6)
-// 1910 -> 1275 us; 300 rows, d = 256, V = 4096 (2 row pairs of 16 tiles)
-// 126 -> 30 us.
+// pair-groups) 1580 -> 545 us (457 now); 1677 rows, d = 2560, V = 100003
+// (7 for 6) 1910 -> 1275 us (1046 now); 300 rows, d = 256, V = 4096 (2 row
+// pairs of 16 tiles) 126 -> 30 us.
 struct GSched {
   int n;      // masked rows
   int rank;   // 0: the pair's even CTA (issues the MMAs), 1: its peer
@@ -1005,439 +1008,439 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the outer tiles that close before the round's last boundary, then the Z
       // tile, then the others
       for (int part = kMode == GM_B && rd.count > 0 ? 0 : 1; ok && part < 2; ++part) {
-      if (part == 1 && r < nr && j < s.E) {
-        // ---------------------------------------------------- Z epilogue
-        const Pos at = locate(s, j);
-        const int k = at.k;
-        const int o = outer_of(p, s, at.rp);
-        const int slot = j % p.R;
-        const int kv = kvalid_of(s, k);
-        // 32-column blocks to read: every block of the slices the members
-        // copy, so columns >= kv are written as zeros, never left stale
-        const int hlast = 2 * slices_of(s, k);
-        const int hbeg = half * (kZN / 64);
-        const int hend = min(hlast, hbeg + kZN / 64);
-        // the slot's previous tile must have been copied by every member
-        bool go = true;
-        if (consume && lane == 0) {
-          go = wait_counter(p.cons + ring0 + slot, static_cast<uint32_t>(g * (j / p.R)), ctl);
-          fence_proxy_async_global();
-        }
-        if (kMode == GM_B) {
-          // lse2 and target of the tile's 256 masked rows (+inf / -1 beyond n)
-          for (int c = threadIdx.x; c < kZN; c += kEpi) {
-            const int rc = k * kZN + c;
-            float l2 = INFINITY;
-            int yy = -1;
+        if (part == 1 && r < nr && j < s.E) {
+          // ---------------------------------------------------- Z epilogue
+          const Pos at = locate(s, j);
+          const int k = at.k;
+          const int o = outer_of(p, s, at.rp);
+          const int slot = j % p.R;
+          const int kv = kvalid_of(s, k);
+          // 32-column blocks to read: every block of the slices the members
+          // copy, so columns >= kv are written as zeros, never left stale
+          const int hlast = 2 * slices_of(s, k);
+          const int hbeg = half * (kZN / 64);
+          const int hend = min(hlast, hbeg + kZN / 64);
+          // the slot's previous tile must have been copied by every member
+          bool go = true;
+          if (consume && lane == 0) {
+            go = wait_counter(p.cons + ring0 + slot, static_cast<uint32_t>(g * (j / p.R)), ctl);
+            fence_proxy_async_global();
+          }
+          if (kMode == GM_B) {
+            // lse2 and target of the tile's 256 masked rows (+inf / -1 beyond n)
+            for (int c = threadIdx.x; c < kZN; c += kEpi) {
+              const int rc = k * kZN + c;
+              float l2 = INFINITY;
+              int yy = -1;
+              if (rc < s.n) {
+                const int t = p.rows[rc];
+                if (t >= 0 && t < p.T) {
+                  l2 = p.lse_in[t] * kLog2e;
+                  yy = p.targets[t];
+                }
+              }
+              meta_l[c] = l2;
+              meta_y[c] = yy;
+            }
+          }
+          if (!named_bar_and(1, kEpi, go && mbar_wait(zfull, zph, ctl))) { ok = false; break; }
+          zph ^= 1u;
+          tc_fence_after();
+          float pv_all[4][32];  // pass A: 2^(x - R) of this thread's columns
+          bool fresh = false;   // pass A: the member's first tile of the outer tile
+          uint8_t* img = ring_bytes + (ring0 + slot) * static_cast<size_t>(kXTile);
+          if (!OLIVE_DCHECK(p.dev_status, !consume || static_cast<int64_t>(ring0 + slot) < p.ring_tiles))
+            img = nullptr;
+          // Two 32-column blocks at a time make a slice of this warp's 32 rows,
+          // staged in shared memory and moved to the ring by one bulk store
+          // (4 KB of whole lines).  `put` stages a block once the previous
+          // slice's copy has read the staging area, and starts the copy after
+          // the second block.  (Storing the 16-byte chunks straight from the
+          // registers writes half sectors of 32 different lines per
+          // instruction, and needed a device-wide fence by every thread of the
+          // epilogue per tile; the bulk stores need one by each warp's lane 0.)
+          auto put = [&](int h, const float (&v)[32]) {
+            if (!(h & 1)) {
+              if (lane == 0) bulk_wait_read();
+              __syncwarp();
+            }
+            stage32(staging, lane, h, v);
+            if (h & 1) {
+              fence_proxy_async_shared();
+              __syncwarp();
+              if (lane == 0 && img) {
+                bulk_store(img + img_off((warp & 3) * 32, h >> 1), staging, kWarpSlice);
+                bulk_commit();
+              }
+            }
+          };
+          // the accumulator goes back to the MMA thread once its last block is
+          // in registers
+          auto drained = [&](int h) {
+            if (h + 1 < hend) return;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(zempty_lead);
+          };
+          if (kMode != GM_KL && hbeg >= hend) drained(hend);  // no valid column in this half
+          if (kMode == GM_B) {
+            const int v = o * kBM + row;
+            // does any of this half's columns have its target in the outer tile?
+            bool hit = false;
+  #pragma unroll
+            for (int q = 0; q < 4; ++q)
+              hit = hit || static_cast<uint32_t>(meta_y[half * 128 + q * 32 + lane] - o * kBM) < kBM;
+            hit = __any_sync(0xffffffffu, hit);
+  #pragma unroll 1
+            for (int h = hbeg; h < hend; ++h) {
+              uint32_t a[32];
+              tmem_ld_32x32b_x32(zaddr + h * 32, a);
+              tmem_ld_wait();
+              drained(h);
+              float gv[32];
+  #pragma unroll
+              for (int c = 0; c < 32; ++c)
+                gv[c] = s_coef * fast_exp2(fmaf(__uint_as_float(a[c]), p.scale2, -meta_l[h * 32 + c]));
+              if (hit) {
+                // the target entry p - 1 from expm1, exact where p is near 1
+  #pragma unroll 1
+                for (int c = 0; c < 32; ++c) {
+                  if (meta_y[h * 32 + c] != v) continue;
+                  float z = 0.f;
+  #pragma unroll
+                  for (int q = 0; q < 32; ++q) z = q == c ? __uint_as_float(a[q]) : z;
+                  z = s_coef * expm1f(fmaf(z, p.scale2, -meta_l[h * 32 + c]) * kLn2);
+  #pragma unroll
+                  for (int q = 0; q < 32; ++q) gv[q] = q == c ? z : gv[q];
+                }
+              }
+              if (h * 32 + 32 > kv) {
+                // rows beyond the last one may hold anything, NaN too
+  #pragma unroll
+                for (int c = 0; c < 32; ++c) gv[c] = h * 32 + c < kv ? gv[c] : 0.f;
+              }
+              put(h, gv);
+            }
+          } else if (kMode == GM_KL) {
+            // G of the divergence for this 128 x 256 tile from both heads' fp32
+            // logits and the row's lse of each head and KL from the value sweep:
+            // reverse g inv_tau p_s (log p_s - log p_t - KL), forward
+            // g inv_tau (p_s - p_t).  The student's logits arrive first and wait
+            // in registers for the teacher's.
+            float zs_all[4][32];
+  #pragma unroll
+            for (int b = 0; b < 4; ++b)
+              tmem_ld_32x32b_x32(zaddr + (hbeg + b) * 32, reinterpret_cast<uint32_t(&)[32]>(zs_all[b]));
+            tmem_ld_wait();
+            drained(hend - 1);
+            const int rc = o * kBM + row;
+            bool valid = false;
+            float ls0 = 0.f, lt0 = 0.f, klv = 0.f, cf = 0.f;
             if (rc < s.n) {
               const int t = p.rows[rc];
               if (t >= 0 && t < p.T) {
-                l2 = p.lse_in[t] * kLog2e;
-                yy = p.targets[t];
+                valid = true;
+                ls0 = p.lse_sc[rc];
+                lt0 = p.lse_tc[rc];
+                klv = p.kl[t];
+                cf = p.grad_kl[t] * p.inv_tau;
               }
             }
-            meta_l[c] = l2;
-            meta_y[c] = yy;
-          }
-        }
-        if (!named_bar_and(1, kEpi, go && mbar_wait(zfull, zph, ctl))) { ok = false; break; }
-        zph ^= 1u;
-        tc_fence_after();
-        float pv_all[4][32];  // pass A: 2^(x - R) of this thread's columns
-        bool fresh = false;   // pass A: the member's first tile of the outer tile
-        uint8_t* img = ring_bytes + (ring0 + slot) * static_cast<size_t>(kXTile);
-        if (!OLIVE_DCHECK(p.dev_status, !consume || static_cast<int64_t>(ring0 + slot) < p.ring_tiles))
-          img = nullptr;
-        // Two 32-column blocks at a time make a slice of this warp's 32 rows,
-        // staged in shared memory and moved to the ring by one bulk store
-        // (4 KB of whole lines).  `put` stages a block once the previous
-        // slice's copy has read the staging area, and starts the copy after
-        // the second block.  (Storing the 16-byte chunks straight from the
-        // registers writes half sectors of 32 different lines per
-        // instruction, and needed a device-wide fence by every thread of the
-        // epilogue per tile; the bulk stores need one by each warp's lane 0.)
-        auto put = [&](int h, const float (&v)[32]) {
-          if (!(h & 1)) {
-            if (lane == 0) bulk_wait_read();
-            __syncwarp();
-          }
-          stage32(staging, lane, h, v);
-          if (h & 1) {
-            fence_proxy_async_shared();
-            __syncwarp();
-            if (lane == 0 && img) {
-              bulk_store(img + img_off((warp & 3) * 32, h >> 1), staging, kWarpSlice);
-              bulk_commit();
-            }
-          }
-        };
-        // the accumulator goes back to the MMA thread once its last block is
-        // in registers
-        auto drained = [&](int h) {
-          if (h + 1 < hend) return;
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(zempty_lead);
-        };
-        if (kMode != GM_KL && hbeg >= hend) drained(hend);  // no valid column in this half
-        if (kMode == GM_B) {
-          const int v = o * kBM + row;
-          // does any of this half's columns have its target in the outer tile?
-          bool hit = false;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            hit = hit || static_cast<uint32_t>(meta_y[half * 128 + q * 32 + lane] - o * kBM) < kBM;
-          hit = __any_sync(0xffffffffu, hit);
-#pragma unroll 1
-          for (int h = hbeg; h < hend; ++h) {
-            uint32_t a[32];
-            tmem_ld_32x32b_x32(zaddr + h * 32, a);
-            tmem_ld_wait();
-            drained(h);
-            float gv[32];
-#pragma unroll
-            for (int c = 0; c < 32; ++c)
-              gv[c] = s_coef * fast_exp2(fmaf(__uint_as_float(a[c]), p.scale2, -meta_l[h * 32 + c]));
-            if (hit) {
-              // the target entry p - 1 from expm1, exact where p is near 1
-#pragma unroll 1
-              for (int c = 0; c < 32; ++c) {
-                if (meta_y[h * 32 + c] != v) continue;
-                float z = 0.f;
-#pragma unroll
-                for (int q = 0; q < 32; ++q) z = q == c ? __uint_as_float(a[q]) : z;
-                z = s_coef * expm1f(fmaf(z, p.scale2, -meta_l[h * 32 + c]) * kLn2);
-#pragma unroll
-                for (int q = 0; q < 32; ++q) gv[q] = q == c ? z : gv[q];
-              }
-            }
-            if (h * 32 + 32 > kv) {
-              // rows beyond the last one may hold anything, NaN too
-#pragma unroll
-              for (int c = 0; c < 32; ++c) gv[c] = h * 32 + c < kv ? gv[c] : 0.f;
-            }
-            put(h, gv);
-          }
-        } else if (kMode == GM_KL) {
-          // G of the divergence for this 128 x 256 tile from both heads' fp32
-          // logits and the row's lse of each head and KL from the value sweep:
-          // reverse g inv_tau p_s (log p_s - log p_t - KL), forward
-          // g inv_tau (p_s - p_t).  The student's logits arrive first and wait
-          // in registers for the teacher's.
-          float zs_all[4][32];
-#pragma unroll
-          for (int b = 0; b < 4; ++b)
-            tmem_ld_32x32b_x32(zaddr + (hbeg + b) * 32, reinterpret_cast<uint32_t(&)[32]>(zs_all[b]));
-          tmem_ld_wait();
-          drained(hend - 1);
-          const int rc = o * kBM + row;
-          bool valid = false;
-          float ls0 = 0.f, lt0 = 0.f, klv = 0.f, cf = 0.f;
-          if (rc < s.n) {
-            const int t = p.rows[rc];
-            if (t >= 0 && t < p.T) {
-              valid = true;
-              ls0 = p.lse_sc[rc];
-              lt0 = p.lse_tc[rc];
-              klv = p.kl[t];
-              cf = p.grad_kl[t] * p.inv_tau;
-            }
-          }
-          if (!named_bar_and(1, kEpi, mbar_wait(zfull, zph, ctl))) { ok = false; break; }
-          zph ^= 1u;
-          tc_fence_after();
-          if (hbeg >= hend) drained(hend);
-          // log p_s - log p_t as (z_s - z_t) - (lse_s - lse_t): a teacher
-          // shifted by a constant per row cancels before the large terms meet
-          const float dl = ls0 - lt0;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int h = hbeg + b;
-            if (h >= hend) break;
-            float(&gv)[32] = zs_all[b];
-#pragma unroll
-            for (int u = 0; u < 32; u += 16) {
-              uint32_t zt_b[16];
-              tmem_ld_32x32b_x16(zaddr + h * 32 + u, zt_b);
-              tmem_ld_wait();
-              if (u) drained(h);
-#pragma unroll
-              for (int c = 0; c < 16; ++c) {
-                const float zs = gv[u + c] * p.inv_tau;
-                const float zt = __uint_as_float(zt_b[c]) * p.inv_tau;
-                const float ps = fast_exp2((zs - ls0) * kLog2e);
-                gv[u + c] = cf * (p.reverse ? ps * (((zs - zt) - dl) - klv)
-                                            : ps - fast_exp2((zt - lt0) * kLog2e));
-              }
-            }
-            if (!valid || h * 32 + 32 > kv) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c) gv[c] = valid && h * 32 + c < kv ? gv[c] : 0.f;
-            }
-            put(h, gv);
-          }
-        } else {
-          fresh = at.rp != cur_rp;
-          if (fresh) {
-            cur_rp = at.rp;
-            ra = load_row_a(p, s, o * kBM + row);
-            run_m = -INFINITY;
-          }
-          const int v0 = k * kZN;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int h = hbeg + b;
-            if (h >= hend) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c) pv_all[b][c] = 0.f;
-              continue;
-            }
-            uint32_t a[32];
-            tmem_ld_32x32b_x32(zaddr + h * 32, a);
-            tmem_ld_wait();
-            drained(h);
-            float(&pv)[32] = pv_all[b];
-            // (two running maxima of x - R: shorter chains)
-            float m1 = -INFINITY;
-            if (h * 32 + 32 <= kv) {
-#pragma unroll
-              for (int c = 0; c < 32; c += 2) {
-                const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
-                const float x1 = fmaf(__uint_as_float(a[c + 1]), p.scale2, -ra.R);
-                run_m = fmaxf(run_m, x0);
-                m1 = fmaxf(m1, x1);
-                pv[c] = fast_exp2(x0);
-                pv[c + 1] = fast_exp2(x1);
-              }
-            } else {
-#pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                const bool in = h * 32 + c < kv;
-                const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
-                m1 = in ? fmaxf(m1, x0) : m1;
-                pv[c] = in ? fast_exp2(x0) : 0.f;
-              }
-            }
-            run_m = fmaxf(run_m, m1);
-            const int yo = ra.y - (v0 + h * 32);
-            if (kMode == GM_A && yo >= 0 && yo < 32) {
-              // the target's exact logit and the bf16 value of P'_y the MMA
-              // sees: the epilogue replaces that term by p_y - 1 from the
-              // logit, so rows with p_y near 1 keep their accuracy
-#pragma unroll
-              for (int c = 0; c < 32; ++c)
-                if (c == yo) {
-                  p.zy[o * kBM + row] = __uint_as_float(a[c]) * p.inv_tau;
-                  p.pyb[o * kBM + row] = __bfloat162float(__float2bfloat16_rn(pv[c]));
+            if (!named_bar_and(1, kEpi, mbar_wait(zfull, zph, ctl))) { ok = false; break; }
+            zph ^= 1u;
+            tc_fence_after();
+            if (hbeg >= hend) drained(hend);
+            // log p_s - log p_t as (z_s - z_t) - (lse_s - lse_t): a teacher
+            // shifted by a constant per row cancels before the large terms meet
+            const float dl = ls0 - lt0;
+  #pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const int h = hbeg + b;
+              if (h >= hend) break;
+              float(&gv)[32] = zs_all[b];
+  #pragma unroll
+              for (int u = 0; u < 32; u += 16) {
+                uint32_t zt_b[16];
+                tmem_ld_32x32b_x16(zaddr + h * 32 + u, zt_b);
+                tmem_ld_wait();
+                if (u) drained(h);
+  #pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                  const float zs = gv[u + c] * p.inv_tau;
+                  const float zt = __uint_as_float(zt_b[c]) * p.inv_tau;
+                  const float ps = fast_exp2((zs - ls0) * kLog2e);
+                  gv[u + c] = cf * (p.reverse ? ps * (((zs - zt) - dl) - klv)
+                                              : ps - fast_exp2((zt - lt0) * kLog2e));
                 }
+              }
+              if (!valid || h * 32 + 32 > kv) {
+  #pragma unroll
+                for (int c = 0; c < 32; ++c) gv[c] = valid && h * 32 + c < kv ? gv[c] : 0.f;
+              }
+              put(h, gv);
             }
-            if (kMode == GM_A) put(h, pv);
+          } else {
+            fresh = at.rp != cur_rp;
+            if (fresh) {
+              cur_rp = at.rp;
+              ra = load_row_a(p, s, o * kBM + row);
+              run_m = -INFINITY;
+            }
+            const int v0 = k * kZN;
+  #pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const int h = hbeg + b;
+              if (h >= hend) {
+  #pragma unroll
+                for (int c = 0; c < 32; ++c) pv_all[b][c] = 0.f;
+                continue;
+              }
+              uint32_t a[32];
+              tmem_ld_32x32b_x32(zaddr + h * 32, a);
+              tmem_ld_wait();
+              drained(h);
+              float(&pv)[32] = pv_all[b];
+              // (two running maxima of x - R: shorter chains)
+              float m1 = -INFINITY;
+              if (h * 32 + 32 <= kv) {
+  #pragma unroll
+                for (int c = 0; c < 32; c += 2) {
+                  const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
+                  const float x1 = fmaf(__uint_as_float(a[c + 1]), p.scale2, -ra.R);
+                  run_m = fmaxf(run_m, x0);
+                  m1 = fmaxf(m1, x1);
+                  pv[c] = fast_exp2(x0);
+                  pv[c + 1] = fast_exp2(x1);
+                }
+              } else {
+  #pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                  const bool in = h * 32 + c < kv;
+                  const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
+                  m1 = in ? fmaxf(m1, x0) : m1;
+                  pv[c] = in ? fast_exp2(x0) : 0.f;
+                }
+              }
+              run_m = fmaxf(run_m, m1);
+              const int yo = ra.y - (v0 + h * 32);
+              if (kMode == GM_A && yo >= 0 && yo < 32) {
+                // the target's exact logit and the bf16 value of P'_y the MMA
+                // sees: the epilogue replaces that term by p_y - 1 from the
+                // logit, so rows with p_y near 1 keep their accuracy
+  #pragma unroll
+                for (int c = 0; c < 32; ++c)
+                  if (c == yo) {
+                    p.zy[o * kBM + row] = __uint_as_float(a[c]) * p.inv_tau;
+                    p.pyb[o * kBM + row] = __bfloat162float(__float2bfloat16_rn(pv[c]));
+                  }
+              }
+              if (kMode == GM_A) put(h, pv);
+            }
+          }
+          if (kMode == GM_REF) {
+            // the row's two column halves meet in shared memory
+            if (half) meta_l[row] = run_m;
+            named_bar_sync(1, kEpi);
+            if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
+            named_bar_sync(1, kEpi);
+          } else {
+            // publish the warp's part of the tile once its copies are complete
+            if (lane == 0) {
+              bulk_wait();
+              fence_proxy_async_global();
+              red_release_add(p.ready + ring0 + slot, 1u);
+            }
+            __syncwarp();
+            // the row metadata of this tile is read: the next one's may be written
+            if (kMode == GM_B) named_bar_sync(1, kEpi);
+            if (kMode == GM_A) {
+              // The row's sum over this member's tiles is one chain in column
+              // order, which the first half's thread hands to the second's in
+              // shared memory.  (One sum a half rounds less where a large term
+              // stands early, but by other amounts than the target's logit does,
+              // and the mean loss, in which the two nearly cancel, was 1.5 to 1.7
+              // times as far from 64 bits.)
+              if (half) named_bar_sync(2, kEpi);
+              float sum = !half && fresh ? 0.f : meta_l[row];
+  #pragma unroll
+              for (int b = 0; b < 4; ++b)
+  #pragma unroll
+                for (int c = 0; c < 32; ++c) sum += pv_all[b][c];
+              meta_l[row] = sum;
+              if (!half) named_bar_arrive(2, kEpi);
+              if (ra.valid) put_sums(j, at.rp, o, half ? sum : 0.f, run_m + ra.R);
+            }
           }
         }
-        if (kMode == GM_REF) {
-          // the row's two column halves meet in shared memory
-          if (half) meta_l[row] = run_m;
-          named_bar_sync(1, kEpi);
-          if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
-          named_bar_sync(1, kEpi);
-        } else {
-          // publish the warp's part of the tile once its copies are complete
-          if (lane == 0) {
-            bulk_wait();
-            fence_proxy_async_global();
-            red_release_add(p.ready + ring0 + slot, 1u);
-          }
-          __syncwarp();
-          // the row metadata of this tile is read: the next one's may be written
-          if (kMode == GM_B) named_bar_sync(1, kEpi);
-          if (kMode == GM_A) {
-            // The row's sum over this member's tiles is one chain in column
-            // order, which the first half's thread hands to the second's in
-            // shared memory.  (One sum a half rounds less where a large term
-            // stands early, but by other amounts than the target's logit does,
-            // and the mean loss, in which the two nearly cancel, was 1.5 to 1.7
-            // times as far from 64 bits.)
-            if (half) named_bar_sync(2, kEpi);
-            float sum = !half && fresh ? 0.f : meta_l[row];
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-#pragma unroll
-              for (int c = 0; c < 32; ++c) sum += pv_all[b][c];
-            meta_l[row] = sum;
-            if (!half) named_bar_arrive(2, kEpi);
-            if (ra.valid) put_sums(j, at.rp, o, half ? sum : 0.f, run_m + ra.R);
-          }
-        }
-      }
-      if constexpr (!consume) break;
-      if (r == 0) continue;
-      // ------------------------------------------- outer tiles completed
-      for (int e = part == 0 ? e_lo : rd.last; ok && e < (part == 0 ? rd.last : e_end); ++e) {
-        const Pos at = locate(s, e);
-        if (!closes(s, e, at.k)) continue;
-        const int o = outer_of(p, s, at.rp);
-        const bool split = s.nt > 0 && e >= s.tail0;
-        // the runs [run_lo, run_hi] of the tail that hold a part of this row pair
-        const int t = at.rp - s.rp0;
-        const int run_lo = split ? run_of(s, t * s.ni) : 0;
-        const int run_hi = split ? run_of(s, (t + 1) * s.ni - 1) : 0;
-        const int rc = o * kBM + row;
-        RowA rw{false, -1, -1, 0.f};
-        const bool whole = !phantom(s, at.rp) && OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph);
-        if (kMode == GM_A && whole) {
-          // every member's sums (and the target's z_y, P'_y from the member
-          // that met it) are published before any member reads them
-          rw = load_row_a(p, s, rc);
-          if (rw.valid && !member_has_job(s, g, e, at.k)) put_sums(e, at.rp, o, 0.f, -INFINITY);
-          __threadfence();
-          named_bar_sync(1, kEpi);
-          if (threadIdx.x == 0) red_release_add(p.outer_ctr + o, 1u);
-        }
-        float acc[4][32];
-        if (!take_output(acc)) { ok = false; break; }
-        if (split) {
-          if (!whole) continue;  // a phantom: its rows are never stored
-          // the layout is the threads' own (16 bytes of every thread side by
-          // side), so stores and loads are whole lines
-          auto part = [&](int run) {
-            return reinterpret_cast<float4*>(p.tail_acc) +
-                   (static_cast<size_t>((run + t) * 2 + s.rank) * g + s.m) * kTailVecs + threadIdx.x;
-          };
-          if (!OLIVE_DCHECK(p.dev_status, ((run_hi + t) * 2 + s.rank) * g + s.m < p.tail_parts)) {
-            ok = false;
-            break;
-          }
-          float4* out = part(s.pg);
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            if (ob + 32 * b >= oe) continue;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              out[(8 * b + q) * kEpi] =
-                  make_float4(acc[b][4 * q], acc[b][4 * q + 1], acc[b][4 * q + 2], acc[b][4 * q + 3]);
-          }
-          __threadfence();
-          named_bar_sync(1, kEpi);
-          bool last = true;
-          if (threadIdx.x == 0) {
-            last = atomicAdd(p.tail_ctr + (2 * t + s.rank) * g + s.m, 1u) ==
-                   static_cast<uint32_t>(run_hi - run_lo);
+        if constexpr (!consume) break;
+        if (r == 0) continue;
+        // ------------------------------------------- outer tiles completed
+        for (int e = part == 0 ? e_lo : rd.last; ok && e < (part == 0 ? rd.last : e_end); ++e) {
+          const Pos at = locate(s, e);
+          if (!closes(s, e, at.k)) continue;
+          const int o = outer_of(p, s, at.rp);
+          const bool split = s.nt > 0 && e >= s.tail0;
+          // the runs [run_lo, run_hi] of the tail that hold a part of this row pair
+          const int t = at.rp - s.rp0;
+          const int run_lo = split ? run_of(s, t * s.ni) : 0;
+          const int run_hi = split ? run_of(s, (t + 1) * s.ni - 1) : 0;
+          const int rc = o * kBM + row;
+          RowA rw{false, -1, -1, 0.f};
+          const bool whole = !phantom(s, at.rp) && OLIVE_DCHECK(p.dev_status, o >= 0 && o <= s.ph);
+          if (kMode == GM_A && whole) {
+            // every member's sums (and the target's z_y, P'_y from the member
+            // that met it) are published before any member reads them
+            rw = load_row_a(p, s, rc);
+            if (rw.valid && !member_has_job(s, g, e, at.k)) put_sums(e, at.rp, o, 0.f, -INFINITY);
             __threadfence();
+            named_bar_sync(1, kEpi);
+            if (threadIdx.x == 0) red_release_add(p.outer_ctr + o, 1u);
           }
-          if (!named_bar_and(1, kEpi, last)) continue;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) acc[b][c] = 0.f;
-          }
-          for (int c = run_lo; c <= run_hi; ++c) {
-            const float4* in = part(c);
-#pragma unroll
+          float acc[4][32];
+          if (!take_output(acc)) { ok = false; break; }
+          if (split) {
+            if (!whole) continue;  // a phantom: its rows are never stored
+            // the layout is the threads' own (16 bytes of every thread side by
+            // side), so stores and loads are whole lines
+            auto part = [&](int run) {
+              return reinterpret_cast<float4*>(p.tail_acc) +
+                     (static_cast<size_t>((run + t) * 2 + s.rank) * g + s.m) * kTailVecs + threadIdx.x;
+            };
+            if (!OLIVE_DCHECK(p.dev_status, ((run_hi + t) * 2 + s.rank) * g + s.m < p.tail_parts)) {
+              ok = false;
+              break;
+            }
+            float4* out = part(s.pg);
+  #pragma unroll
             for (int b = 0; b < 4; ++b) {
               if (ob + 32 * b >= oe) continue;
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const float4 v = __ldcg(in + (8 * b + q) * kEpi);
-                acc[b][4 * q] += v.x;
-                acc[b][4 * q + 1] += v.y;
-                acc[b][4 * q + 2] += v.z;
-                acc[b][4 * q + 3] += v.w;
-              }
+  #pragma unroll
+              for (int q = 0; q < 8; ++q)
+                out[(8 * b + q) * kEpi] =
+                    make_float4(acc[b][4 * q], acc[b][4 * q + 1], acc[b][4 * q + 2], acc[b][4 * q + 3]);
             }
-          }
-        }
-        if (kMode == GM_B) {
-          store_output(rc < p.V ? rc : -1, acc);
-          continue;
-        }
-        if (kMode == GM_KL) {
-          // the divergence gradient: G carried g inv_tau, so d_h_s is the sum
-          const int tr = rc < s.n ? p.rows[rc] : -1;
-          store_output(tr < p.T ? tr : -1, acc);
-          continue;
-        }
-        // pass A: merge the members' sums, then dH
-        if (whole) {
-          const uint32_t posts = static_cast<uint32_t>(g * (run_hi - run_lo + 1));
-          const bool seen = threadIdx.x == 0 ? wait_counter(p.outer_ctr + o, posts, ctl) : true;
-          if (!named_bar_and(1, kEpi, seen)) { ok = false; break; }
-        }
-        float lse2 = rw.R, mx = -INFINITY;
-        if (!p.lse_known && rw.valid) {
-          float sum = 0.f;
-          // (a split row pair's slots stand one after the other)
-          const size_t from = split ? tail_row(run_lo + t, 0) : rc;
-          const size_t stride = split ? 2 * kBM : Tpad;
-          const float* ps = (split ? p.tail_s : p.part_s) + from;
-          const float* pm = (split ? p.tail_m : p.part_m) + from;
-          const int count = 2 * g * (run_hi - run_lo + 1);
-#pragma unroll 8
-          for (int e2 = 0; e2 < count; ++e2) {
-            sum += __ldcg(ps + e2 * stride);
-            mx = fmaxf(mx, __ldcg(pm + e2 * stride));
-          }
-          lse2 = rw.R + log2f(sum);
-        }
-        // (the redo launch, with R = the rows' maxima, never flags)
-        const bool row_ok = !rw.valid || p.lse_known || p.redo ||
-                            (mx - rw.R <= kRefMax && isfinite(lse2));
-        const bool tile_ok = named_bar_and(1, kEpi, row_ok);
-        if (!tile_ok) {
-          // the reference was too low for some row: the redo launch
-          // recomputes this row tile with R = the rows' maxima
-          if (s.m == 0) {
-            if (rw.valid && !half) p.rmax[rc] = mx;
+            __threadfence();
+            named_bar_sync(1, kEpi);
+            bool last = true;
             if (threadIdx.x == 0) {
-              const uint32_t at = atomicAdd(p.redo_list, 1u);
-              p.redo_list[1 + at] = static_cast<uint32_t>(o);
+              last = atomicAdd(p.tail_ctr + (2 * t + s.rank) * g + s.m, 1u) ==
+                     static_cast<uint32_t>(run_hi - run_lo);
+              __threadfence();
             }
-          }
-        } else {
-          const bool has_y = rw.valid && rw.y >= 0 && rw.y < p.V;
-          if (s.m == 0 && rw.valid && !half) {
-            if (!has_y) atomicOr(p.dev_status, 1 << OLIVE_ERR_TOKEN_RANGE);
-            if (p.write_fwd) {
-              const float l = lse2 * kLn2;
-              const float lp = has_y ? __ldcg(p.zy + rc) - l : NAN;
-              p.lse[rw.t] = l;
-              p.logp[rw.t] = lp;
-              p.nll[rc] = -lp;
+            if (!named_bar_and(1, kEpi, last)) continue;
+  #pragma unroll
+            for (int b = 0; b < 4; ++b) {
+  #pragma unroll
+              for (int c = 0; c < 32; ++c) acc[b][c] = 0.f;
             }
-          }
-          const float scale = fast_exp2(rw.R - lse2);
-          // dH = coef (scale acc - W[y]) with the target's term taken out of
-          // acc (scale P'_y, P'_y as the MMA saw it) and put back as p_y W[y]:
-          // together coef (scale acc + corr W[y]), corr = (p_y - 1) - scale P'_y
-          float corr = 0.f;
-          if (has_y) {
-            const float lnat = p.lse_known ? p.lse_in[rw.t] : lse2 * kLn2;
-            corr = expm1f(__ldcg(p.zy + rc) - lnat) - scale * __ldcg(p.pyb + rc);
-          }
-          const uint4* wy =
-              has_y ? reinterpret_cast<const uint4*>(p.W + static_cast<size_t>(rw.y) * p.d + s.c0) : nullptr;
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int c = ob + 32 * b;
-            if (c >= oe) continue;
-            const int nv = min(32, oe - c);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint4 w4 = make_uint4(0, 0, 0, 0);
-              if (wy && 8 * q < nv) w4 = __ldg(wy + c / 8 + q);
-              const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w4);
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const float2 wf = __bfloat1622float2(w2[u]);
-                float& a0 = acc[b][8 * q + 2 * u];
-                float& a1 = acc[b][8 * q + 2 * u + 1];
-                a0 = s.coef * fmaf(scale, a0, corr * wf.x);
-                a1 = s.coef * fmaf(scale, a1, corr * wf.y);
+            for (int c = run_lo; c <= run_hi; ++c) {
+              const float4* in = part(c);
+  #pragma unroll
+              for (int b = 0; b < 4; ++b) {
+                if (ob + 32 * b >= oe) continue;
+  #pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                  const float4 v = __ldcg(in + (8 * b + q) * kEpi);
+                  acc[b][4 * q] += v.x;
+                  acc[b][4 * q + 1] += v.y;
+                  acc[b][4 * q + 2] += v.z;
+                  acc[b][4 * q + 3] += v.w;
+                }
               }
             }
           }
-          store_output(rw.valid ? rw.t : -1, acc);
+          if (kMode == GM_B) {
+            store_output(rc < p.V ? rc : -1, acc);
+            continue;
+          }
+          if (kMode == GM_KL) {
+            // the divergence gradient: G carried g inv_tau, so d_h_s is the sum
+            const int tr = rc < s.n ? p.rows[rc] : -1;
+            store_output(tr < p.T ? tr : -1, acc);
+            continue;
+          }
+          // pass A: merge the members' sums, then dH
+          if (whole) {
+            const uint32_t posts = static_cast<uint32_t>(g * (run_hi - run_lo + 1));
+            const bool seen = threadIdx.x == 0 ? wait_counter(p.outer_ctr + o, posts, ctl) : true;
+            if (!named_bar_and(1, kEpi, seen)) { ok = false; break; }
+          }
+          float lse2 = rw.R, mx = -INFINITY;
+          if (!p.lse_known && rw.valid) {
+            float sum = 0.f;
+            // (a split row pair's slots stand one after the other)
+            const size_t from = split ? tail_row(run_lo + t, 0) : rc;
+            const size_t stride = split ? 2 * kBM : Tpad;
+            const float* ps = (split ? p.tail_s : p.part_s) + from;
+            const float* pm = (split ? p.tail_m : p.part_m) + from;
+            const int count = 2 * g * (run_hi - run_lo + 1);
+  #pragma unroll 8
+            for (int e2 = 0; e2 < count; ++e2) {
+              sum += __ldcg(ps + e2 * stride);
+              mx = fmaxf(mx, __ldcg(pm + e2 * stride));
+            }
+            lse2 = rw.R + log2f(sum);
+          }
+          // (the redo launch, with R = the rows' maxima, never flags)
+          const bool row_ok = !rw.valid || p.lse_known || p.redo ||
+                              (mx - rw.R <= kRefMax && isfinite(lse2));
+          const bool tile_ok = named_bar_and(1, kEpi, row_ok);
+          if (!tile_ok) {
+            // the reference was too low for some row: the redo launch
+            // recomputes this row tile with R = the rows' maxima
+            if (s.m == 0) {
+              if (rw.valid && !half) p.rmax[rc] = mx;
+              if (threadIdx.x == 0) {
+                const uint32_t at = atomicAdd(p.redo_list, 1u);
+                p.redo_list[1 + at] = static_cast<uint32_t>(o);
+              }
+            }
+          } else {
+            const bool has_y = rw.valid && rw.y >= 0 && rw.y < p.V;
+            if (s.m == 0 && rw.valid && !half) {
+              if (!has_y) atomicOr(p.dev_status, 1 << OLIVE_ERR_TOKEN_RANGE);
+              if (p.write_fwd) {
+                const float l = lse2 * kLn2;
+                const float lp = has_y ? __ldcg(p.zy + rc) - l : NAN;
+                p.lse[rw.t] = l;
+                p.logp[rw.t] = lp;
+                p.nll[rc] = -lp;
+              }
+            }
+            const float scale = fast_exp2(rw.R - lse2);
+            // dH = coef (scale acc - W[y]) with the target's term taken out of
+            // acc (scale P'_y, P'_y as the MMA saw it) and put back as p_y W[y]:
+            // together coef (scale acc + corr W[y]), corr = (p_y - 1) - scale P'_y
+            float corr = 0.f;
+            if (has_y) {
+              const float lnat = p.lse_known ? p.lse_in[rw.t] : lse2 * kLn2;
+              corr = expm1f(__ldcg(p.zy + rc) - lnat) - scale * __ldcg(p.pyb + rc);
+            }
+            const uint4* wy =
+                has_y ? reinterpret_cast<const uint4*>(p.W + static_cast<size_t>(rw.y) * p.d + s.c0) : nullptr;
+  #pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              const int c = ob + 32 * b;
+              if (c >= oe) continue;
+              const int nv = min(32, oe - c);
+  #pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                uint4 w4 = make_uint4(0, 0, 0, 0);
+                if (wy && 8 * q < nv) w4 = __ldg(wy + c / 8 + q);
+                const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w4);
+  #pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const float2 wf = __bfloat1622float2(w2[u]);
+                  float& a0 = acc[b][8 * q + 2 * u];
+                  float& a1 = acc[b][8 * q + 2 * u + 1];
+                  a0 = s.coef * fmaf(scale, a0, corr * wf.x);
+                  a1 = s.coef * fmaf(scale, a1, corr * wf.y);
+                }
+              }
+            }
+            store_output(rw.valid ? rw.t : -1, acc);
+          }
         }
-      }
       }
     }
   }
