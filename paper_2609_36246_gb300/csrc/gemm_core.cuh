@@ -25,8 +25,11 @@
 //   kBMn, kDual, kStages, kEpiWarps, Sched, make_sched(p) (one whole warp; may
 //   read device counters such as n_rows), num_units(p,s), unit_len(p,s,u),
 //   tile(p,s,u,t), kEpiSmem (bytes of shared-memory scratch for the epilogue)
-//   and Epi with init(smem, part), begin(p,s,u,row), tile(p,s,u,t,tc,taddr),
-//   end(p,s,u).  Every wait of the epilogue ends in one decision of all its
+//   and Epi with init(smem, part), begin(p,s,u,row), end(p,s,u) and
+//   tile(p,s,u,t,tc,taddr,release), which calls release() once, after its last
+//   read of the accumulator.  With kFirst (dual policies) first(p,tc,taddr)
+//   runs before it, as soon as the first product is complete, while the second
+//   one's MMAs run.  Every wait of the epilogue ends in one decision of all its
 //   warps, so Epi::end may synchronise them (named barrier 2).
 #pragma once
 
@@ -69,8 +72,8 @@ struct CoreLayout {
   static constexpr int B_BYTES = Kern::kBN * kBK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int RING_BYTES = STAGE_BYTES * Kern::kStages;
-  // barriers: full[S], empty[S], tfull[2], tempty[2], drain
-  static constexpr int BAR_BYTES = 8 * (2 * Kern::kStages + 5);
+  // barriers: full[S], empty[S], tfull[2], tempty[2], drain, first
+  static constexpr int BAR_BYTES = 8 * (2 * Kern::kStages + 6);
   static constexpr int MISC_BYTES = 64;
   static constexpr int EPI_BYTES = Kern::kEpiSmem;  // scratch for the epilogue policy
   static constexpr int SMEM_BYTES =
@@ -80,6 +83,7 @@ struct CoreLayout {
   static constexpr uint32_t TMEM_COLS = ACC_BUFS * ACC_COLS;
   static_assert(ACC_BUFS == 1 || ACC_BUFS == 2, "one or two accumulators");
   static_assert(TMEM_COLS <= 512, "the accumulators must fit in TMEM");
+  static_assert(!Kern::kFirst || (Kern::kDual && ACC_BUFS == 1), "one barrier for the first products");
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
 };
 
@@ -104,6 +108,7 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
   auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * Kern::kStages + b); };
   auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * Kern::kStages + 2 + b); };
   const uint32_t drain_bar = bar0 + 8u * (2 * Kern::kStages + 4);
+  const uint32_t first_bar = bar0 + 8u * (2 * Kern::kStages + 5);
   uint8_t* misc = gbase + L::RING_BYTES + L::BAR_BYTES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
@@ -123,6 +128,7 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
       mbar_init(tempty_bar(b), CT::kEpi);
     }
     mbar_init(drain_bar, 1);
+    mbar_init(first_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -240,6 +246,7 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
             for (int kk = 0; kk < kBK / 16; ++kk)
               umma_bf16(dt, dA + (so + kk * kStepA), dB + (so + kk * kStepB), idesc, kk > 0 ? 1u : acc0);
             umma_commit(empty_bar(stage));
+            if (Kern::kFirst && k == tc.nk - 1) umma_commit(first_bar);
           }
           if (++stage == Kern::kStages) { stage = 0; phase ^= 1u; }
         }
@@ -271,13 +278,21 @@ __global__ void __launch_bounds__(CoreThreads<Kern>::kAll, 1)
       epi.begin(p, sched, u, row);
       for (int t = 0; t < nt; ++t) {
         const TileC tc = Kern::tile(p, sched, u, t);
+        const uint32_t taddr = lane_addr + static_cast<uint32_t>(buf * L::ACC_COLS);
         // one decision for all epilogue threads: tcgen05.ld below is a warp
         // collective and Epi::end may synchronise the epilogue warps
+        if constexpr (Kern::kFirst) {
+          if (!named_bar_and(1, CT::kEpi, mbar_wait(first_bar, aphase, ctl))) { ok = false; break; }
+          tc_fence_after();
+          epi.first(p, tc, taddr);
+        }
         if (!named_bar_and(1, CT::kEpi, mbar_wait(tfull_bar(buf), aphase, ctl))) { ok = false; break; }
         tc_fence_after();
-        epi.tile(p, sched, u, t, tc, lane_addr + static_cast<uint32_t>(buf * L::ACC_COLS));
-        tc_fence_before();
-        mbar_arrive(tempty_bar(buf));
+        const uint32_t tempty = tempty_bar(buf);
+        epi.tile(p, sched, u, t, tc, taddr, [&] {
+          tc_fence_before();
+          mbar_arrive(tempty);
+        });
         if (++buf == L::ACC_BUFS) { buf = 0; aphase ^= 1u; }
       }
       if (!ok) break;

@@ -37,6 +37,7 @@ struct FwdKernT {
   static constexpr bool kAMn = false;
   static constexpr bool kBMn = false;
   static constexpr bool kDual = false;
+  static constexpr bool kFirst = false;
   static constexpr int kStages = 4;
   static constexpr int kAccBufs = 2;
   static constexpr int kEpiWarps = 4;
@@ -202,7 +203,9 @@ struct FwdKernT {
       m = mn;
     }
 
-    __device__ void tile(const Params& p, const Sched&, int, int, const TileC& tc, uint32_t taddr) {
+    template <class Release>
+    __device__ void tile(const Params& p, const Sched&, int, int, const TileC& tc, uint32_t taddr,
+                         const Release& release) {
 #pragma unroll 1
       for (int c = 0; c < kBN; c += 64) {
         const int col0 = tc.n0 + c;
@@ -214,6 +217,7 @@ struct FwdKernT {
         chunk(p, a, col0);
         if (col0 + 32 < p.V) chunk(p, b, col0 + 32);
       }
+      release();
     }
 
     __device__ void end(const Params& p, const Sched& sc, int) {

@@ -43,6 +43,7 @@ struct KlFwdKern {
   static constexpr bool kAMn = false;
   static constexpr bool kBMn = false;
   static constexpr bool kDual = true;
+  static constexpr bool kFirst = false;
   static constexpr int kStages = 4;
   static constexpr int kAccBufs = 1;
   static constexpr int kEpiWarps = 8;
@@ -137,7 +138,9 @@ struct KlFwdKern {
       mp = mpn;
       mq = mqn;
     }
-    __device__ void tile(const Params& p, const Sched&, int, int, const TileC& tc, uint32_t taddr) {
+    template <class Release>
+    __device__ void tile(const Params& p, const Sched&, int, int, const TileC& tc, uint32_t taddr,
+                         const Release& release) {
 #pragma unroll 1
       for (int c = part * (kBN / 2); c < (part + 1) * (kBN / 2); c += 32) {
         const int col0 = tc.n0 + c;
@@ -148,6 +151,7 @@ struct KlFwdKern {
         tmem_ld_wait();
         chunk(p, a, b, col0);
       }
+      release();
     }
     // (m, s, a) + (m2, s2, a2) in base 2; an empty side (m = -inf) adds nothing
     static __device__ __forceinline__ void merge3(float& m, float& s, float& a, float m2, float s2,

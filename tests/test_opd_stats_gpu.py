@@ -82,6 +82,21 @@ def test_small_shapes(T, ds, dt, V, K, inv_tau, direction):
     _check_against_oracle(hs, Ws, ht, Wt, rows, K, inv_tau, direction, g)
 
 
+@pytest.mark.parametrize("V", [40, 100, 128, 257, 384, 389, 1000])
+@pytest.mark.parametrize("direction", ["reverse", "forward"])
+def test_ragged_half_tiles(V, direction):
+    """Tiles whose second 128 columns are missing, whole or cut, with logits
+    that grow along the vocabulary: every tile replaces entries of the student's
+    list, whose teacher logits are looked up after the teacher's product."""
+    rng = np.random.default_rng(V)
+    hs, Ws, ht, Wt = _models(rng, 140, 64, 96, V)
+    grow = torch.linspace(0.25, 1.0, V).unsqueeze(1)
+    Ws, Wt = (Ws.float() * grow).to(torch.bfloat16), (Wt.float() * grow).to(torch.bfloat16)
+    rows = np.arange(1, 140)
+    g = _gpu(hs, Ws, ht, Wt, rows, 16, 1.0, direction)
+    _check_against_oracle(hs, Ws, ht, Wt, rows, 16, 1.0, direction, g)
+
+
 def test_full_set_and_identical_models():
     """K = V = 16: overlap 1 and the truncated KL is the full KL; identical
     heads: KL 0, overlap 1."""
