@@ -774,6 +774,18 @@ __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2
   m = mn;
 }
 
+// 2^y, y <= 0, as two factors for a product with e up to 2^117 (a half tile's
+// stored exponentials, kOwnShift): (e a) b leaves fp32's normal range only
+// where the whole product does.  2^y alone is 0 or subnormal from y = -127 on,
+// and a half tile 17 below lse2 has y = -110 - 17.  b is 1 for y >= -100.
+struct Pow2 {
+  float a, b;
+};
+__device__ __forceinline__ Pow2 pow2_split(float y) {
+  const float h = fmaxf(y, -100.f);
+  return Pow2{exp2f(h), exp2f(y - h)};
+}
+
 // One warp per row tile row of the slab, after ZSAVE tiles with a row
 // reference R (base 2): the row's stored e' = 2^(x - R) give G = coef s e'
 // off the target, with coef = g inv_tau (/ N_mask) and s = 2^(R - lse2) per
@@ -851,13 +863,14 @@ __global__ void __launch_bounds__(256)
       uint4* grow = reinterpret_cast<uint4*>(g + static_cast<size_t>(r) * ldg);
       for (int idx = lane; idx < nvec; idx += 32) {
         uint4 v = grow[idx];
-        const float sc = fast_exp2(zm[idx >> 4] - lse2);  // 16 vectors per half tile
+        const Pow2 sc = pow2_split(zm[idx >> 4] - lse2);  // 16 vectors per half tile
         __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&v);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float2 u = __bfloat1622float2(h2[e]);
           const int c = idx * 8 + 2 * e;
-          h2[e] = __floats2bfloat162_rn(c < V ? u.x * sc : 0.f, c + 1 < V ? u.y * sc : 0.f);
+          h2[e] = __floats2bfloat162_rn(c < V ? (u.x * sc.a) * sc.b : 0.f,
+                                        c + 1 < V ? (u.y * sc.a) * sc.b : 0.f);
         }
         grow[idx] = v;
       }
@@ -1272,15 +1285,15 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
       uint4* g4 = reinterpret_cast<uint4*>(grow);
       for (int idx = lane; idx < nvec; idx += 32) {
         uint4 v = g4[idx];
-        const float sc = fast_exp2(zm[idx >> 4] - lse2);  // 16 vectors per half tile
+        const Pow2 sc = pow2_split(zm[idx >> 4] - lse2);  // 16 vectors per half tile
         __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&v);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const float2 u = __bfloat1622float2(h2[e]);
           const int c = idx * 8 + 2 * e;
           // p = e' 2^(ref - lse2) first, then the row coefficient
-          h2[e] = __floats2bfloat162_rn(c < a.V ? (u.x * sc) * cf : 0.f,
-                                        c + 1 < a.V ? (u.y * sc) * cf : 0.f);
+          h2[e] = __floats2bfloat162_rn(c < a.V ? (u.x * sc.a) * sc.b * cf : 0.f,
+                                        c + 1 < a.V ? (u.y * sc.a) * sc.b * cf : 0.f);
         }
         g4[idx] = v;
       }

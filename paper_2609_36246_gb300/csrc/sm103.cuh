@@ -452,11 +452,11 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* addr, uint32_t targ
 }
 
 // ---------------------------------------------------------------- helpers ---
-// 2^x in one instruction (largest relative error 2^-22 by the PTX ISA, the
-// unit exp2f uses too); results below 2^-126 are 0, -inf gives 0, NaN stays.
-// exp2f's range check for subnormal results costs four more instructions an
-// element, and no sum or product here can hold such a term: every 2^x meets a
-// sum of at least 1 (or its row's total) in 24 bits.
+// 2^x in one instruction: largest relative error 2^-22 by the PTX ISA, results
+// below 2^-126 are 0, -inf gives 0, NaN stays.  For terms that meet a sum of at
+// least 1 (or their row's total) in 24 bits, where what is flushed cannot show.
+// A factor that is multiplied by something large, and an exponential that is
+// used by itself, take exp2f.
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -341,3 +341,25 @@ def test_split_row_pairs(n, V, d, redo):
         h[::2, 0] = 8.0
         W[V // 2, 0] = 8.0
     _full_check(b, h, W, grad_loss=0.7, grad_dtype=torch.float32)
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_small_probabilities_beside_a_far_maximum(form):
+    """Ids 256 to 511 lie 59 (base 2) above every row's reference, the largest
+    logit 131 above it: the slab form stores theirs as 2^59 and scales by
+    2^-131, and their p of about 2^-72 make up the whole dW rows of the ids that
+    are no targets."""
+    rng = np.random.default_rng(92)
+    V = 1000
+    b = synth.batch_from_lengths(rng, [2], [60], V)
+    h = synth.normal_bf16(rng, (b.T, 64), 1.0)
+    h[:, 0] = 8.0
+    W = synth.normal_bf16(rng, (V, 64), 0.05)
+    W[:, 0] = 0.0
+    W[256:512, 0] = 5.125
+    W[700, 0] = 11.375
+    _, _, dw = _full_check(b, h, W, grad_dtype=torch.float32, form=form)
+    o = oracle_pack(b)
+    _, rdw = oracle.token_loss_bwd(to_f64(h), to_f64(W), o["targets"], o["rows"])
+    ids = np.setdiff1d(np.arange(256, 512), o["targets"])
+    assert rel_frob(dw[ids], rdw[ids]) <= 1e-2

@@ -220,6 +220,34 @@ def test_rows_far_above_their_first_tile(spike):
     _full_check(hs, Ws, ht, Wt, rows, K, g, 1.0)
 
 
+def test_flat_rest_far_above_the_first_tile():
+    """Half of the rows have their first 256 logits at 0, one id at 82 nats and
+    the other 151679 around 69: every half tile past the first is stored 110
+    (base 2) below its own maximum, which lies 16 to 19 below lse, and together
+    they hold a quarter of the row's mass, so the factor that turns what is
+    stored into probabilities is below 2^-126 for almost all of them."""
+    rng = np.random.default_rng(90)
+    T, d, V, K = 24, 64, 151936, 8
+    hs = synth.normal_bf16(rng, (T, d), 1.0)
+    hs[:, :2] = 0.0
+    hs[::2, :2] = 8.0
+    Ws = synth.normal_bf16(rng, (V, d), 0.05)
+    Ws[:, 0], Ws[:, 1] = 8.625, 0.0
+    Ws[:256, 0] = 0.0
+    # (in a direction of its own: what G has there and in the rest adds up to 0)
+    Ws[70001, 0], Ws[70001, 1] = 0.0, 10.25
+    ht = synth.normal_bf16(rng, (T, d), 1.0)
+    Wt = synth.normal_bf16(rng, (V, d), 0.3)
+    z = oracle.logits(to_f64(hs), to_f64(Ws), 1.0)[::2]
+    lse = np.logaddexp.reduce(z, axis=1)
+    # (in base 2; the last tile is whole, so every column belongs to a half tile of 128)
+    below = (lse[:, None] - z[:, 256:].reshape(len(z), -1, 128).max(axis=2)) / np.log(2)
+    assert (below > 16).mean() > 0.8 and np.exp(z[:, :256].max(axis=1) - lse).max() < 2.0 ** -100
+    rows = _decided_rows(hs, Ws, ht, Wt, np.arange(T), K, 1.0)
+    g = rng.uniform(0.5, 2.0, size=T)
+    _full_check(hs, Ws, ht, Wt, rows, K, g, 1.0)
+
+
 def test_tiny_weights_take_the_rewritten_form():
     """Rows with g_t = 1e-30 put the row scale below 2^-96, so their G is
     written out in full; each such row still matches on its own."""
