@@ -360,7 +360,12 @@ __device__ void epi_grad(const FusedParams& p, const Plan& pl, const Unit& x, in
 
 // forward tile of the fused forward + backward: per row the tile's max and
 // sum of 2^(x - max) in base-2 units, e = 2^(x - max) stored in bf16 at the
-// row's G slab columns (zeros on padding rows), and the exact target logit
+// row's G slab columns (zeros on padding rows), and the exact target logit.
+// kList: the top-K candidates are taken from e itself, so what fast_exp2 would
+// flush is kept down to 2^-133, as far as bf16 goes (exp2f in the cross-entropy
+// step too cost it 4 % at d = 256 and 512, where this epilogue bounds it: 317 ->
+// 329 us for 16384 rows, V = 4096).
+template <bool kList>
 __device__ void epi_zsave(const FusedParams& p, const Plan& pl, const Unit& x, int row, int part,
                           uint32_t taddr) {
   const int r_local = x.i * kBM + row;
@@ -397,7 +402,7 @@ __device__ void epi_zsave(const FusedParams& p, const Plan& pl, const Unit& x, i
   // else the half tile's own maximum (kOwnShift below it when the true maxima
   // are kept for a top-K selection)
   float ref = tm;
-  if (p.zref) ref = !(tm - R > kRefMax) ? R : (p.part_tm ? tm - kOwnShift : tm);
+  if (p.zref) ref = !(tm - R > kRefMax) ? R : (kList ? tm - kOwnShift : tm);
   __nv_bfloat16* grow = p.g + static_cast<size_t>(r_local) * p.ldg;
   float ts = 0.f;
 #pragma unroll 1
@@ -411,7 +416,8 @@ __device__ void epi_zsave(const FusedParams& p, const Plan& pl, const Unit& x, i
     float e[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
-      e[k] = (valid && k < nv) ? fast_exp2(__uint_as_float(a[k]) * p.scale2 - ref) : 0.f;
+      const float x = __uint_as_float(a[k]) * p.scale2 - ref;
+      e[k] = (valid && k < nv) ? (kList ? exp2f(x) : fast_exp2(x)) : 0.f;
       ts += e[k];
     }
     store_row32(grow, col0, OLIVE_DTYPE_BF16, nv, e);
@@ -420,7 +426,7 @@ __device__ void epi_zsave(const FusedParams& p, const Plan& pl, const Unit& x, i
     const size_t o = static_cast<size_t>(r_local) * pl.vh + 2 * x.j + part;
     p.part_zm[o] = ref;
     p.part_zs[o] = ts;
-    if (p.part_tm) p.part_tm[o] = tm;
+    if (kList) p.part_tm[o] = tm;
   }
 }
 
@@ -728,7 +734,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
       }
       switch (x.kind) {
         case K_GRAD: epi_grad(p, pl, x, row, part, taddr); break;
-        case K_ZSAVE: epi_zsave(p, pl, x, row, part, taddr); break;
+        case K_ZSAVE:
+          if (p.part_tm) epi_zsave<true>(p, pl, x, row, part, taddr);
+          else epi_zsave<false>(p, pl, x, row, part, taddr);
+          break;
         case K_ZREF: epi_zref(p, x, row, part, taddr); break;
         case K_DH: epi_dh(p, x, row, part, taddr); break;
         case K_DW: epi_dw(p, pl, x, row, part, taddr, nk); break;

@@ -248,6 +248,31 @@ def test_flat_rest_far_above_the_first_tile():
     _full_check(hs, Ws, ht, Wt, rows, K, g, 1.0)
 
 
+def test_selection_far_below_the_reference():
+    """One id about 88 nats above all others: the rest of the row's top K lies
+    126 to 129 (base 2) below its reference, where the stored 2^(x - R) is
+    subnormal in bf16; the row still lists K ids, the right ones."""
+    rng = np.random.default_rng(91)
+    T, d, V, K = 40, 64, 4000, 16
+    hs = synth.normal_bf16(rng, (T, d), 1.0)
+    hs[:, 0] = 8.0
+    Ws = synth.normal_bf16(rng, (V, d), 0.127)
+    Ws[:, 0] = -11.4375
+    Ws[3] = 0.0
+    ht = synth.normal_bf16(rng, (T, d), 1.0)
+    Wt = synth.normal_bf16(rng, (V, d), 0.3)
+    z = oracle.logits(to_f64(hs), to_f64(Ws), 1.0)
+    kth = (np.sort(z, axis=1)[:, V - K] - z.max(axis=1)) / np.log(2)
+    assert kth.max() < -126 and kth.min() > -130
+    rows = _decided_rows(hs, Ws, ht, Wt, np.arange(T), K, 1.0)
+    o = _gpu(hs, Ws, ht, Wt, rows, K, rng.uniform(0.5, 2.0, size=T))
+    _, _, lp, ids = oracle.token_topk(to_f64(hs), to_f64(Ws), rows, K)
+    assert np.array_equal(np.sort(o["s_ids"][rows], axis=1), np.sort(ids[rows], axis=1))
+    assert_close_logp(o["s_logp"][rows], lp[rows], "s_logp")
+    # (with p = 1 at one id the gradient is what 1 - p leaves: nothing to compare)
+    assert not o["d_h_s"][rows].any() or np.abs(o["d_h_s"][rows]).max() < 1e-4
+
+
 def test_tiny_weights_take_the_rewritten_form():
     """Rows with g_t = 1e-30 put the row scale below 2^-96, so their G is
     written out in full; each such row still matches on its own."""
