@@ -1406,6 +1406,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 p.logp[rw.t] = lp;
                 p.nll[rc] = -lp;
               }
+            } else if (s.m == 0 && p.write_fwd && !half && rc < s.n) {
+              p.nll[rc] = 0.f;  // an index outside the batch: reported, and no term of the loss
             }
             const float scale = fast_exp2(rw.R - lse2);
             // dH = coef (scale acc - W[y]) with the target's term taken out of

@@ -363,3 +363,34 @@ def test_small_probabilities_beside_a_far_maximum(form):
     _, rdw = oracle.token_loss_bwd(to_f64(h), to_f64(W), o["targets"], o["rows"])
     ids = np.setdiff1d(np.arange(256, 512), o["targets"])
     assert rel_frob(dw[ids], rdw[ids]) <= 1e-2
+
+
+@pytest.mark.parametrize("reduction", ["sum", "mean"])
+def test_loss_with_row_indices_outside_the_batch(reduction):
+    """Row indices outside [0, T) are reported and add nothing to the loss,
+    whatever the workspace held; on every form of the step and on the forward
+    call alone."""
+    b, h, W = synth.random_case(93, 4, 900, 64, max_prefix=30, max_cont=80, std_w=0.1)
+    g = gpu_pack(b)
+    n = int(g["n_rows"].item())
+    rows = g["rows"].clone()
+    rows[2], rows[n - 1] = b.T + 5, -1
+    o = oracle_pack(b)
+    keep = np.delete(o["rows"], [2, n - 1])
+    _, _, want = oracle.token_logprob(to_f64(h), to_f64(W), o["targets"], keep, 1.0, "sum")
+    want = want / n if reduction == "mean" else want
+    hc, Wc = h.cuda(), W.cuda()
+    one = torch.ones(1, dtype=torch.float32, device="cuda")
+    for fill in (0x00, 0x7f, 0xff):
+        for op in ("logprob_fwd", "loss_fwd_bwd", "loss_fwd_bwd_slab"):
+            ws = B.workspace(B.olive_workspace_size(op, b.T, 64, 900)).fill_(fill)
+            st = B.new_status()
+            if op == "logprob_fwd":
+                loss = B.olive_token_logprob_fwd(hc, Wc, g["targets"], rows, g["n_rows"], 1.0, reduction,
+                                                 ws=ws, dev_status=st)[2]
+            else:
+                loss = B.olive_token_loss_fwd_bwd(hc, Wc, g["targets"], rows, g["n_rows"], one, 1.0,
+                                                  reduction, ws=ws, dev_status=st,
+                                                  slab=op == "loss_fwd_bwd_slab")[2]
+            assert B.status_bits(st) == ["OLIVE_ERR_OFFSETS"]
+            assert_close_loss(loss.item(), want)
