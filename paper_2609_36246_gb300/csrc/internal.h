@@ -65,7 +65,7 @@ struct FwdWs {
   float* part_m;  // [part_rows]: segment, row (row tiles x 128 to a segment)
   float* part_s;  // [part_rows]
   float* zy;      // [Tpad]
-  float* nll;     // [Tpad]
+  float* nll;     // [Tpad] loss terms of the rows, or with `done` of blocks of them (doubles)
   uint32_t* done; // finished blocks of the finalize kernel; null when min_parts is 0
 };
 size_t fwd_ws_bytes(int64_t T, int64_t d, int min_parts = kMinParts);

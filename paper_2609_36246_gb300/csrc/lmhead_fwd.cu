@@ -4,8 +4,9 @@
 // entropy and the K largest log-probs (Appendix A: OPD reads the student's
 // top-16 log-probs).
 //
-//   gather      hc[r] = hidden[rows[r]]  (compacts the masked rows so TMA can
-//               stream 128-row tiles; the last tile is zero-padded)
+//   prepare     hc[r] = hidden[rows[r]]  (compacts the masked rows so TMA can
+//               stream 128-row tiles; the last tile is zero-padded), outputs
+//               and counters filled
 //   fwd tiles   persistent tcgen05 GEMM, 128 x 256 tiles of z = hc . W^T in
 //               TMEM; each epilogue thread owns one row and folds 256 logits
 //               per tile into a running (max, sum) in registers, catching
@@ -15,8 +16,8 @@
 //               per-thread shared-memory buffer and are merged into a
 //               16-entry register list by a compare-swap network
 //   finalize    merges the per-segment partials, writes lse and
-//               logp = z_y - lse (or entropy and top-K) on the packed rows
-//   loss        one block sums -logp in a fixed order (deterministic)
+//               logp = z_y - lse (or entropy and top-K) on the packed rows, and
+//               sums -logp in a fixed order (deterministic)
 #include <algorithm>
 #include <climits>
 #include <cmath>
@@ -292,12 +293,19 @@ __global__ void __launch_bounds__(256)
 
 // One warp a row, its lanes over the row's segments.  (One thread a row walked
 // up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
+//
+// `done` given: a block adds its rows' loss terms up itself and leaves one sum
+// in `terms` (a double a block, no more room than a float a row takes), and the
+// last block adds those: a fixed order, whatever block is last.  (Scoring 131072
+// rows, d = 64, V = 512: 125 us; with the last block of 128 threads over all of
+// the rows' terms 252, with a launch of 1024 threads for them 175.)
+// Null: the rows' terms, for launch_loss_reduce.
 __global__ void __launch_bounds__(128)
     fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
                         const int32_t* __restrict__ targets, int T, int V, int vt, int ctas, int min_parts,
                         const float* __restrict__ part_m, const float* __restrict__ part_s,
                         const float* __restrict__ zy, float* __restrict__ logp,
-                        float* __restrict__ lse, float* nll, uint32_t* done, int reduction,
+                        float* __restrict__ lse, void* terms, uint32_t* done, int reduction,
                         float* __restrict__ loss, int32_t* dev_status) {
   __shared__ double part[4];
   __shared__ bool last;
@@ -306,6 +314,7 @@ __global__ void __launch_bounds__(128)
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
   const int warps = gridDim.x * 4;
+  double acc = 0.0;
   for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
     float M = -INFINITY, S = 0.f;
     for (int s = lane; s < sp.sv; s += 32) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
@@ -314,38 +323,42 @@ __global__ void __launch_bounds__(128)
     if (lane) continue;
     const float l = (M + log2f(S)) * kLn2;
     const int t = rows[r];
-    if (t < 0 || t >= T) {
-      nll[r] = 0.f;
-      continue;  // reported by the gather kernel
+    float lp = 0.f;
+    if (t >= 0 && t < T) {
+      const int y = targets[t];
+      if (y >= 0 && y < V) {
+        lp = zy[r] - l;
+      } else {
+        atomicOr(dev_status, 1 << OLIVE_ERR_TOKEN_RANGE);
+        lp = NAN;
+      }
+      logp[t] = lp;
+      lse[t] = l;
     }
-    const int y = targets[t];
-    float lp;
-    if (y < 0 || y >= V) {
-      atomicOr(dev_status, 1 << OLIVE_ERR_TOKEN_RANGE);
-      lp = NAN;
-    } else {
-      lp = zy[r] - l;
-    }
-    logp[t] = lp;
-    lse[t] = l;
-    nll[r] = -lp;
+    if (done) acc -= static_cast<double>(lp);
+    else static_cast<float*>(terms)[r] = -lp;
   }
-  // the last block to finish adds the loss terms up in a fixed order
   if (!done) return;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  auto block_sum = [&](double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    return (part[0] + part[1]) + (part[2] + part[3]);
+  };
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) {
+    __stcg(static_cast<double*>(terms) + blockIdx.x, acc);
+    __threadfence();
+    last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
   __syncthreads();
   if (!last) return;
-  __threadfence();
-  double acc = 0.0;
-#pragma unroll 4
-  for (int r = threadIdx.x; r < n; r += 128) acc += static_cast<double>(__ldcg(nll + r));
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) part[threadIdx.x >> 5] = acc;
-  __syncthreads();
+  acc = 0.0;
+  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += 128)
+    acc += __ldcg(static_cast<const double*>(terms) + b);
+  acc = block_sum(acc);
   if (threadIdx.x == 0) {
-    acc = (part[0] + part[1]) + (part[2] + part[3]);
     if (reduction == OLIVE_REDUCE_MEAN) acc = n > 0 ? acc / n : 0.0;
     *loss = static_cast<float>(acc);
   }

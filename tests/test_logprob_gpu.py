@@ -255,3 +255,26 @@ def test_few_rows_many_segments(n):
     for ids in (ti[r], opd["s_topk_ids"][r]):
         assert torch.equal(ids.long()[sure], want_i[sure])
     close(opd["t_logp_s"][r][sure], lt.gather(1, want_i)[sure])
+
+
+@pytest.mark.parametrize("n", [1, 5, 131, 2433, 9729, 40000])
+@pytest.mark.parametrize("reduction", ["sum", "mean"])
+def test_loss_over_blocks_of_rows(n, reduction):
+    """The loss is the sum of the blocks' sums, one block to many (and many rows
+    a warp): equal to the fp64 sum of the call's own log-probs, again on a
+    workspace that holds anything, and the same with no workspace."""
+    rng = np.random.default_rng(n)
+    V, d = 300, 16
+    b = synth.batch_from_lengths(rng, [2], [n], V)
+    h = synth.normal_bf16(rng, (b.T, d), 1.0).cuda()
+    W = synth.normal_bf16(rng, (V, d), 0.3).cuda()
+    g = gpu_pack(b)
+    args = (h, W, g["targets"], g["rows"], g["n_rows"], 1.0, reduction)
+    for fill in (0, 0xff):
+        ws = B.workspace(B.olive_workspace_size("logprob_fwd", b.T, d, V)).fill_(fill)
+        logp, _, loss = B.olive_token_logprob_fwd(*args, ws=ws)
+        want = -logp.double().sum().item() / (n if reduction == "mean" else 1)
+        # the terms are fp32 and their sum fp64: one rounding to fp32
+        assert abs(loss.item() - want) <= 2.0 ** -23 * abs(want)
+    logp2, _, loss2 = B.olive_token_logprob_fwd_noalloc(*args)
+    assert torch.equal(logp2, logp) and abs(loss2.item() - want) <= 2.0 ** -23 * abs(want)
