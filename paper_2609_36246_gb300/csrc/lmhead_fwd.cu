@@ -380,14 +380,14 @@ __global__ void __launch_bounds__(128)
   const int warps = gridDim.x * 4;
   for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
     const int t = rows[r];
-    if (t < 0 || t >= T) continue;  // reported by the gather kernel
+    if (t < 0 || t >= T) continue;  // reported by prepare_kernel
     float M = -INFINITY, S = 0.f, A = 0.f;
     for (int s = lane; s < sp.sv; s += 32) {
       float f[2];
       merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r], f);
       A = A * f[0] + part_a[s * ld + r] * f[1];
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = merge_lanes(sp.sv) / 2; o > 0; o >>= 1) {
       float f[2];
       const float m2 = __shfl_xor_sync(0xffffffffu, M, o);
       const float s2 = __shfl_xor_sync(0xffffffffu, S, o);
@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(128)
       merge_ms(M, S, m2, s2, f);
       A = A * f[0] + a2 * f[1];
     }
-    const float l2 = M + log2f(S);
-    const float l = l2 * kLn2;
+    const float l2 = M + log2f(S);  // (lane 0's)
+    const float l = __shfl_sync(0xffffffffu, l2 * kLn2, 0);
     if (lane == 0) {
       lse[t] = l;
       entropy[t] = kLn2 * (l2 - A / S);  // lse - E_p[z] in natural units
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(128)
     float tv;
     int ti;
     size_t at;
-    warp_top_merge(part_tv, part_ti, sp.sv, ld, r, K, lane, tv, ti, at);
+    warp_top_merge(part_tv, part_ti, sp.sv, ld, r, lane, tv, ti, at);
     if (lane < K) {
       topk_logp[static_cast<size_t>(t) * K + lane] = tv * inv_tau - l;
       topk_ids[static_cast<size_t>(t) * K + lane] = ti;

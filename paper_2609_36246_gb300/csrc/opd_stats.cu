@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(128)
   const int warps = gridDim.x * 4;
   for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
     const int t = rows[r];
-    if (t < 0 || t >= T) continue;  // reported by the gather kernel
+    if (t < 0 || t >= T) continue;  // reported by prepare_kernel
     float Ms = -INFINITY, Mt = -INFINITY, Ss = 0.f, Es = 0.f, St = 0.f, A = 0.f;
     float fs[2], ft[2];
     for (int s = lane; s < nsv; s += 32) {
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(128)
       Es = Es * fs[0] + part[2 * plane + o] * fs[1];
       A = reverse ? A * fs[0] + part[5 * plane + o] * fs[1] : A * ft[0] + part[5 * plane + o] * ft[1];
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = merge_lanes(nsv) / 2; o > 0; o >>= 1) {
       const float ms2 = __shfl_xor_sync(0xffffffffu, Ms, o), ss2 = __shfl_xor_sync(0xffffffffu, Ss, o);
       const float mt2 = __shfl_xor_sync(0xffffffffu, Mt, o), st2 = __shfl_xor_sync(0xffffffffu, St, o);
       const float es2 = __shfl_xor_sync(0xffffffffu, Es, o), a2 = __shfl_xor_sync(0xffffffffu, A, o);
@@ -382,9 +382,9 @@ __global__ void __launch_bounds__(128)
       Es = Es * fs[0] + es2 * fs[1];
       A = reverse ? A * fs[0] + a2 * fs[1] : A * ft[0] + a2 * ft[1];
     }
-    const float l2s = Ms + log2f(Ss);
+    const float l2s = Ms + log2f(Ss);  // (lane 0's)
     const float l2t = Mt + log2f(St);
-    const float ls = l2s * kLn2, lt = l2t * kLn2;
+    const float ls = __shfl_sync(0xffffffffu, l2s * kLn2, 0), lt = __shfl_sync(0xffffffffu, l2t * kLn2, 0);
     if (lane == 0) {
       // KL = ln2 A / S_p - lse_p + lse_q
       if (out.kl) out.kl[t] = reverse ? kLn2 * (A / Ss) - ls + lt : kLn2 * (A / St) - lt + ls;
@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(128)
     float sv, tv;
     int si, ti;
     size_t at;
-    warp_top_merge(part_tv, part_ti, nsv, ld, r, K, lane, tv, ti, at);
-    warp_top_merge(part_sv, part_si, nsv, ld, r, K, lane, sv, si, at);
+    warp_top_merge(part_tv, part_ti, nsv, ld, r, lane, tv, ti, at);
+    warp_top_merge(part_sv, part_si, nsv, ld, r, lane, sv, si, at);
     bool hit = false;
     for (int q = 0; q < K; ++q) hit |= __shfl_sync(0xffffffffu, ti, q) == si;
     const int common = __popc(__ballot_sync(0xffffffffu, lane < K && hit));

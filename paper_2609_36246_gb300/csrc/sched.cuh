@@ -97,6 +97,14 @@ __device__ inline int read_n_rows(const int32_t* n_rows, int T, int32_t* dev_sta
   return n;
 }
 
+// Lanes of a warp that share a row's sv segments when partials are merged: a
+// power of two, one segment each where 32 are enough.
+__device__ __forceinline__ int merge_lanes(int sv) {
+  int l = 1;
+  while (l < sv && l < 32) l *= 2;
+  return l;
+}
+
 // (m, s) + (m2, s2): a base-2 maximum and the sum of 2^(x - m); an empty side
 // (m = -inf) adds nothing.  w receives the factors applied to each side.
 __device__ __forceinline__ void merge_ms(float& m, float& s, float m2, float s2, float* w = nullptr) {

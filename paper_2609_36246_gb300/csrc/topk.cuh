@@ -43,70 +43,74 @@ __device__ __forceinline__ void topk_insert3_asc(float (&tv)[kTopMax], int (&ti)
   }
 }
 
-// Every lane of a warp: the K largest entries of row r over nsv lists of
+// An entry of a sorted list of 16 that a half warp holds, entry j in its lane j:
+// value, id, and where it came from (list * 16 + entry).
+struct TopEntry {
+  float v;
+  int id, from;
+};
+__device__ __forceinline__ bool top_before(float av, int ai, float bv, int bi) {
+  return av > bv || (av == bv && ai < bi);
+}
+// Sorts a bitonic sequence of 16 (the larger halves of two sorted lists, one of
+// them reversed), best first, in every half warp.
+__device__ __forceinline__ void top_sort16(TopEntry& e, int lane) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const float v = __shfl_xor_sync(0xffffffffu, e.v, o);
+    const int id = __shfl_xor_sync(0xffffffffu, e.id, o);
+    const int from = __shfl_xor_sync(0xffffffffu, e.from, o);
+    if (lane & o ? top_before(e.v, e.id, v, id) : top_before(v, id, e.v, e.id)) e = TopEntry{v, id, from};
+  }
+}
+
+// Every lane of a warp: the 16 largest entries of row r over nsv lists of
 // kTopMax entries each, sorted by value descending, then id ascending (list s
-// at (s ld + r) kTopMax of tv, ti).  Lane j < K ends with the j-th entry and
-// the place `at` it came from.  A lane keeps the best head of every 32nd list;
-// the warp takes the best of the 32 heads K times, and only the lane it came
-// from looks at its lists again.  (One thread a row inserted up to 64 lists of
-// 16 one entry after the other: 130 us for 2048 rows, 296 us for 2900 rows of
-// the OPD sweep's two lists.)
+// at (s ld + r) kTopMax of tv, ti).  Lane j < 16 ends with the j-th entry and
+// the place `at` it came from.  The half warps take every other list: a list
+// comes in reversed, the better of each pair of entries are the 16 best of both,
+// four exchanges sort them, and a list of which no entry gets in costs its two
+// loads and one vote; eight lists' loads are in flight.  (The best of the
+// lists' heads taken 16 times over the warp, five exchanges and a dependent load
+// each, cost as much for one list as for 64: the top-16 call took 650 us for
+// 131072 rows, d = 64, V = 512, and takes 278.  One thread a row, inserting up to
+// 64 lists of 16 one entry after the other, took 294 there and 130 us of its own
+// for 2048 rows.)
 __device__ __forceinline__ void warp_top_merge(const float* __restrict__ tv,
                                                const int32_t* __restrict__ ti, int nsv, size_t ld,
-                                               int r, int K, int lane, float& v_out, int& i_out,
+                                               int r, int lane, float& v_out, int& i_out,
                                                size_t& at_out) {
-  uint64_t heads = 0;  // entries taken from each of this lane's lists, 5 bits each (at most 10 lists)
-  float v;
-  int id, list;
-  size_t at;
-  auto look = [&]() {
-    v = -INFINITY;
-    id = INT_MAX;
-    at = 0;
-    list = 0;
-    for (int s = lane, q = 0; s < nsv; s += 32, ++q) {
-      const int h = static_cast<int>(heads >> (5 * q)) & 31;
-      if (h >= kTopMax) continue;
-      const size_t o = (static_cast<size_t>(s) * ld + r) * kTopMax + h;
-      const float cv = __ldg(tv + o);
-      const int ci = __ldg(ti + o);
-      if (cv > v || (cv == v && ci < id)) {
-        v = cv;
-        id = ci;
-        at = o;
-        list = q;
-      }
+  constexpr int kAhead = 4;  // lists a half warp loads at a time
+  const int half = lane >> 4, sub = lane & 15;
+  TopEntry e{-INFINITY, INT_MAX, 0};
+  for (int s0 = 0; s0 < nsv; s0 += 2 * kAhead) {
+    float v[kAhead];
+    int id[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int s = s0 + 2 * u + half;
+      const size_t o = (static_cast<size_t>(s) * ld + r) * kTopMax + (kTopMax - 1 - sub);
+      v[u] = s < nsv ? __ldg(tv + o) : -INFINITY;
+      id[u] = s < nsv ? __ldg(ti + o) : INT_MAX;
     }
-  };
-  look();
-  v_out = -INFINITY;
-  i_out = INT_MAX;
-  at_out = 0;
-  for (int j = 0; j < K; ++j) {
-    float bv = v;
-    int bi = id, bl = lane;
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      const int ol = __shfl_xor_sync(0xffffffffu, bl, o);
-      if (ov > bv || (ov == bv && (oi < bi || (oi == bi && ol < bl)))) {
-        bv = ov;
-        bi = oi;
-        bl = ol;
-      }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const bool in = top_before(v[u], id[u], e.v, e.id);
+      if (!__any_sync(0xffffffffu, in)) continue;
+      if (in) e = TopEntry{v[u], id[u], (s0 + 2 * u + half) * kTopMax + kTopMax - 1 - sub};
+      top_sort16(e, lane);
     }
-    const unsigned long long ba = __shfl_sync(0xffffffffu, static_cast<unsigned long long>(at), bl);
-    if (lane == j) {
-      v_out = bv;
-      i_out = bi;
-      at_out = static_cast<size_t>(ba);
-    }
-    if (lane == bl && id != INT_MAX) {
-      heads += 1ull << (5 * list);
-      look();
-    }
-    __syncwarp();
   }
+  if (nsv > 1) {  // the two halves' lists: the other one's, reversed
+    const float v = __shfl_xor_sync(0xffffffffu, e.v, 31);
+    const int id = __shfl_xor_sync(0xffffffffu, e.id, 31);
+    const int from = __shfl_xor_sync(0xffffffffu, e.from, 31);
+    if (top_before(v, id, e.v, e.id)) e = TopEntry{v, id, from};
+    top_sort16(e, lane);
+  }
+  v_out = e.v;
+  i_out = e.id;
+  at_out = (static_cast<size_t>(e.from / kTopMax) * ld + r) * kTopMax + e.from % kTopMax;
 }
 
 }  // namespace olive

@@ -95,6 +95,29 @@ def test_uniform_logits_ties_take_smallest_ids():
     assert np.array_equal(ti, np.tile(np.arange(K), (T, 1)))
 
 
+@pytest.mark.parametrize("T,V,K", [(20000, 300, 16), (20000, 300, 1), (30000, 900, 5), (2500, 1300, 16),
+                                   (700, 4097, 11)])
+def test_many_rows_few_lists(T, V, K):
+    """One list a row up to some tens: the merge's one-sided, odd and full
+    batches of lists, against torch on the same fp32 logits' scale."""
+    rng = np.random.default_rng(V + K)
+    h = synth.normal_bf16(rng, (T, 32), 1.0)
+    W = synth.normal_bf16(rng, (V, 32), 0.4)
+    lse, H, tv, ti = _gpu(h, W, np.arange(T), K)
+    z = h.cuda().double() @ W.cuda().double().t()
+    l = torch.log_softmax(z, 1)
+    want, ids = (x.cpu().numpy() for x in l.topk(K + 1, 1))
+    # fp32 sums of 32 products and of V exponentials: 2e-5 of a value near 10
+    assert np.abs(lse - z.logsumexp(1).cpu().numpy()).max() <= 2e-4
+    assert np.abs(H + (l.exp() * l).sum(1).cpu().numpy()).max() <= 2e-4
+    assert np.abs(tv - want[:, :K]).max() <= 2e-4
+    # ids where neighbours are further apart than that
+    gap = want[:, :-1] - want[:, 1:] > 1e-3
+    sure = gap.copy()
+    sure[:, 1:] &= gap[:, :-1]
+    assert sure.mean() > 0.5 and np.array_equal(ti[sure], ids[:, :K][sure])
+
+
 @pytest.mark.slow
 def test_scoring_workload_sampled_rows():
     """2 x (4096 + 4096) tokens, d = 2048, V = 151936, K = 16: sampled rows."""
