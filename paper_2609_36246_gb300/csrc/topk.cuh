@@ -10,18 +10,20 @@ constexpr int kTopMax = 16;  // list length kept per row
 // the last entry falls off.  For a sweep that visits ids in ascending order
 // within the list's lifetime: the new id is larger than every id already
 // listed, so among equal values it belongs last, and the value alone decides
-// its place (no id comparisons).
+// its place (no id comparisons).  Every entry below that place moves by one:
+// all are compared with the new value, and none with its neighbour, which an
+// equal value would let past.
 __device__ __forceinline__ void topk_insert_asc(float (&tv)[kTopMax], int (&ti)[kTopMax], float cv,
                                                 int ci) {
 #pragma unroll
-  for (int j = 0; j < kTopMax; ++j) {
-    const bool before = cv > tv[j];
-    const float v = tv[j];
-    const int i = ti[j];
-    tv[j] = before ? cv : v;
-    ti[j] = before ? ci : i;
-    cv = before ? v : cv;
-    ci = before ? i : ci;
+  for (int j = kTopMax - 1; j > 0; --j) {
+    const bool at = cv > tv[j], above = cv > tv[j - 1];
+    ti[j] = above ? ti[j - 1] : at ? ci : ti[j];
+    tv[j] = above ? tv[j - 1] : at ? cv : tv[j];
+  }
+  if (cv > tv[0]) {
+    tv[0] = cv;
+    ti[0] = ci;
   }
 }
 
@@ -29,17 +31,16 @@ __device__ __forceinline__ void topk_insert_asc(float (&tv)[kTopMax], int (&ti)[
 __device__ __forceinline__ void topk_insert3_asc(float (&tv)[kTopMax], int (&ti)[kTopMax],
                                                  float (&tx)[kTopMax], float cv, int ci, float cx) {
 #pragma unroll
-  for (int j = 0; j < kTopMax; ++j) {
-    const bool before = cv > tv[j];
-    const float v = tv[j];
-    const int i = ti[j];
-    const float x = tx[j];
-    tv[j] = before ? cv : v;
-    ti[j] = before ? ci : i;
-    tx[j] = before ? cx : x;
-    cv = before ? v : cv;
-    ci = before ? i : ci;
-    cx = before ? x : cx;
+  for (int j = kTopMax - 1; j > 0; --j) {
+    const bool at = cv > tv[j], above = cv > tv[j - 1];
+    tx[j] = above ? tx[j - 1] : at ? cx : tx[j];
+    ti[j] = above ? ti[j - 1] : at ? ci : ti[j];
+    tv[j] = above ? tv[j - 1] : at ? cv : tv[j];
+  }
+  if (cv > tv[0]) {
+    tv[0] = cv;
+    ti[0] = ci;
+    tx[0] = cx;
   }
 }
 

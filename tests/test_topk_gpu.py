@@ -118,6 +118,28 @@ def test_many_rows_few_lists(T, V, K):
     assert sure.mean() > 0.5 and np.array_equal(ti[sure], ids[:, :K][sure])
 
 
+@pytest.mark.parametrize("V,first,larger", [(300, 1.0, 5), (300, 1.0, 16), (3000, 0.5, 9), (700, 1.0, 1)])
+def test_ties_below_later_larger_values(V, first, larger):
+    """Equal logits first, then a few larger ones: of the equal ones the
+    smallest ids stay, in ascending order, whatever is put in before them."""
+    T, K = 140, 16
+    h = torch.zeros(T, 64, dtype=torch.bfloat16)
+    h[:, 0] = 1.0
+    W = torch.zeros(V, 64, dtype=torch.bfloat16)
+    W[:, 0] = first
+    W[V - larger:, 0] = first + 1.0 + torch.arange(larger) % 3
+    z = to_f64(W)[:, 0]
+    want = np.lexsort((np.arange(V), -z))[:K]
+    _, _, tv, ti = _gpu(h, W, np.arange(T), K)
+    assert np.array_equal(ti, np.tile(want, (T, 1)))
+    r = torch.arange(T, dtype=torch.int32, device="cuda")
+    n = torch.tensor([T], dtype=torch.int32, device="cuda")
+    c = lambda x: x.cuda()
+    o = B.olive_opd_token_stats(c(h), c(W), c(h), c(W), r, n, K)
+    assert np.array_equal(o["s_topk_ids"].cpu().numpy(), np.tile(want, (T, 1)))
+    assert (o["overlap"] == 1.0).all()
+
+
 @pytest.mark.slow
 def test_scoring_workload_sampled_rows():
     """2 x (4096 + 4096) tokens, d = 2048, V = 151936, K = 16: sampled rows."""
