@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// One warp a row, its lanes over the row's segments.  (One thread a row walked
-// up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
+// As many lanes a row as it has segments (merge_lanes).  (One thread a row
+// walked up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
 //
 // `done` given: a block adds its rows' loss terms up itself and leaves one sum
 // in `terms` (a double a block, no more room than a float a row takes), and the
@@ -313,14 +313,17 @@ __global__ void __launch_bounds__(128)
   const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, min_parts));
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
-  const int warps = gridDim.x * 4;
+  const int per = merge_lanes(sp.sv), sub = lane & (per - 1);
+  const int step = 32 / per;  // rows of a warp
   double acc = 0.0;
-  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
+  for (int r0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * step; r0 < n; r0 += gridDim.x * 4 * step) {
+    const int r = r0 + lane / per;
     float M = -INFINITY, S = 0.f;
-    for (int s = lane; s < sp.sv; s += 32) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
-    for (int o = 16; o > 0; o >>= 1)
+    if (r < n)
+      for (int s = sub; s < sp.sv; s += per) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
+    for (int o = per / 2; o > 0; o >>= 1)
       merge_ms(M, S, __shfl_xor_sync(0xffffffffu, M, o), __shfl_xor_sync(0xffffffffu, S, o));
-    if (lane) continue;
+    if (r >= n || sub) continue;
     const float l = (M + log2f(S)) * kLn2;
     const int t = rows[r];
     float lp = 0.f;

@@ -199,7 +199,7 @@ struct KlFwdKern {
 
 // kl[t] per masked row; with lse_p / lse_q non-null also both heads' lse per
 // compact row (p the primary head: the student for the reverse KL)
-// (one warp a row, its lanes over the row's segments)
+// (as many lanes a row as it has segments: merge_lanes)
 __global__ void __launch_bounds__(128)
     kl_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
                        int vt, int ctas, size_t plane, const float* __restrict__ part,
@@ -209,17 +209,21 @@ __global__ void __launch_bounds__(128)
   const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
-  const int warps = gridDim.x * 4;
-  for (int r = blockIdx.x * 4 + (threadIdx.x >> 5); r < n; r += warps) {
+  const int per = merge_lanes(sp.sv), sub = lane & (per - 1);
+  const int step = 32 / per;  // rows of a warp
+  for (int r0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * step; r0 < n; r0 += gridDim.x * 4 * step) {
+    const int r = r0 + lane / per;
     float Mp = -INFINITY, Mq = -INFINITY, Sp = 0.f, Sq = 0.f, A = 0.f;
     float f[2];
-    for (int s = lane; s < sp.sv; s += 32) {
-      const size_t o = s * ld + r;
-      merge_ms(Mp, Sp, part[0 * plane + o], part[1 * plane + o], f);
-      A = A * f[0] + part[4 * plane + o] * f[1];
-      merge_ms(Mq, Sq, part[2 * plane + o], part[3 * plane + o]);
+    if (r < n) {
+      for (int s = sub; s < sp.sv; s += per) {
+        const size_t o = s * ld + r;
+        merge_ms(Mp, Sp, part[0 * plane + o], part[1 * plane + o], f);
+        A = A * f[0] + part[4 * plane + o] * f[1];
+        merge_ms(Mq, Sq, part[2 * plane + o], part[3 * plane + o]);
+      }
     }
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = per / 2; o > 0; o >>= 1) {
       const float mp2 = __shfl_xor_sync(0xffffffffu, Mp, o), sp2 = __shfl_xor_sync(0xffffffffu, Sp, o);
       const float mq2 = __shfl_xor_sync(0xffffffffu, Mq, o), sq2 = __shfl_xor_sync(0xffffffffu, Sq, o);
       const float a2 = __shfl_xor_sync(0xffffffffu, A, o);
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(128)
       A = A * f[0] + a2 * f[1];
       merge_ms(Mq, Sq, mq2, sq2);
     }
-    if (lane) continue;
+    if (r >= n || sub) continue;
     const float lse_p = (Mp + log2f(Sp)) * kLn2;
     const float lse_q = (Mq + log2f(Sq)) * kLn2;
     const int t = rows[r];
