@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(128)
     float tv;
     int ti;
     size_t at;
-    warp_top_merge(part_tv, part_ti, sp.sv, ld, r, lane, tv, ti, at);
+    warp_top_merge(part_tv, part_ti, sp.sv, ld, r, K, lane, tv, ti, at);
     if (lane < K) {
       topk_logp[static_cast<size_t>(t) * K + lane] = tv * inv_tau - l;
       topk_ids[static_cast<size_t>(t) * K + lane] = ti;

@@ -395,8 +395,8 @@ __global__ void __launch_bounds__(128)
     float sv, tv;
     int si, ti;
     size_t at;
-    warp_top_merge(part_tv, part_ti, nsv, ld, r, lane, tv, ti, at);
-    warp_top_merge(part_sv, part_si, nsv, ld, r, lane, sv, si, at);
+    warp_top_merge(part_tv, part_ti, nsv, ld, r, K, lane, tv, ti, at);
+    warp_top_merge(part_sv, part_si, nsv, ld, r, K, lane, sv, si, at);
     bool hit = false;
     for (int q = 0; q < K; ++q) hit |= __shfl_sync(0xffffffffu, ti, q) == si;
     const int common = __popc(__ballot_sync(0xffffffffu, lane < K && hit));
