@@ -291,42 +291,49 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// As many lanes a row as it has segments (merge_lanes).  (One thread a row
-// walked up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
+// Merges the rows' partials, writes lse and logp and, with `done` given, the
+// loss: the last block adds the terms up in a fixed order (null: the rows' terms
+// for launch_loss_reduce).  One of two forms, kMany beyond kManyRows rows.
 //
-// `done` given: a block adds its rows' loss terms up itself and leaves one sum
-// in `terms` (a double a block, no more room than a float a row takes), and the
-// last block adds those: a fixed order, whatever block is last.  (Scoring 131072
-// rows, d = 64, V = 512: 125 us; with the last block of 128 threads over all of
-// the rows' terms 252, with a launch of 1024 threads for them 175.)
-// Null: the rows' terms, for launch_loss_reduce.
-__global__ void __launch_bounds__(128)
-    fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
-                        const int32_t* __restrict__ targets, int T, int V, int vt, int ctas, int min_parts,
-                        const float* __restrict__ part_m, const float* __restrict__ part_s,
-                        const float* __restrict__ zy, float* __restrict__ logp,
-                        float* __restrict__ lse, void* terms, uint32_t* done, int reduction,
-                        float* __restrict__ loss, int32_t* dev_status) {
+// kMany false: one warp a row, its lanes over the row's segments, and the loss
+// from the rows' own terms (a float a row in `terms`).  (One thread a row walked
+// up to 64 segments twice, a dependent load each: 29 to 50 us a call.)
+// kMany true: as many lanes a row as it has segments (merge_lanes), and each block
+// adds its rows' terms up first and leaves one sum (a double a block, no more
+// room than the floats take).  Scoring 131072 rows, d = 64, V = 512: 81 us; with
+// the first form 252 (its last block of 128 threads reads all of the terms);
+// 16384 rows, d = 256, V = 4096: 67 and 83 us.
+// So short a kernel waits for its code to come from memory, so the first form
+// stands apart: 96 rows of d = 4096 over V = 151936 took 215 us, and 217 with the
+// second.
+template <bool kMany>
+__device__ __forceinline__ void fwd_finalize(int n, const int32_t* __restrict__ rows,
+                                             const int32_t* __restrict__ targets, int T, int V, int vt,
+                                             int ctas, int min_parts, const float* __restrict__ part_m,
+                                             const float* __restrict__ part_s,
+                                             const float* __restrict__ zy, float* __restrict__ logp,
+                                             float* __restrict__ lse, void* terms, uint32_t* done,
+                                             int reduction, float* __restrict__ loss,
+                                             int32_t* dev_status) {
   __shared__ double part[4];
   __shared__ bool last;
-  const int n = read_n_rows(n_rows, T, nullptr);
   const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, min_parts));
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
-  const int per = merge_lanes(sp.sv), sub = lane & (per - 1);
+  const int per = kMany ? merge_lanes(sp.sv) : 32, sub = lane & (per - 1);
   const int step = 32 / per;  // rows of a warp
   double acc = 0.0;
   for (int r0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * step; r0 < n; r0 += gridDim.x * 4 * step) {
     const int r = r0 + lane / per;
     float M = -INFINITY, S = 0.f;
-    if (r < n)
-      for (int s = sub; s < sp.sv; s += per) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
+    if (r < n)  // (fewer lanes than 32 have no second segment)
+      for (int s = sub; s < sp.sv; s += 32) merge_ms(M, S, part_m[s * ld + r], part_s[s * ld + r]);
     for (int o = per / 2; o > 0; o >>= 1)
       merge_ms(M, S, __shfl_xor_sync(0xffffffffu, M, o), __shfl_xor_sync(0xffffffffu, S, o));
     if (r >= n || sub) continue;
     const float l = (M + log2f(S)) * kLn2;
     const int t = rows[r];
-    float lp = 0.f;
+    float lp = 0.f;  // (an index outside the batch is reported by prepare_kernel)
     if (t >= 0 && t < T) {
       const int y = targets[t];
       if (y >= 0 && y < V) {
@@ -338,7 +345,7 @@ __global__ void __launch_bounds__(128)
       logp[t] = lp;
       lse[t] = l;
     }
-    if (done) acc -= static_cast<double>(lp);
+    if (kMany && done) acc -= static_cast<double>(lp);
     else static_cast<float*>(terms)[r] = -lp;
   }
   if (!done) return;
@@ -348,23 +355,42 @@ __global__ void __launch_bounds__(128)
     __syncthreads();
     return (part[0] + part[1]) + (part[2] + part[3]);
   };
-  acc = block_sum(acc);
-  if (threadIdx.x == 0) {
-    __stcg(static_cast<double*>(terms) + blockIdx.x, acc);
-    __threadfence();
-    last = atomicAdd(done, 1u) == gridDim.x - 1;
-    __threadfence();
+  if (kMany) {
+    acc = block_sum(acc);
+    if (threadIdx.x == 0) __stcg(static_cast<double*>(terms) + blockIdx.x, acc);
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
+  __threadfence();
   acc = 0.0;
-  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += 128)
-    acc += __ldcg(static_cast<const double*>(terms) + b);
+  const int count = kMany ? static_cast<int>(gridDim.x) : n;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < count; i += 128)
+    acc += kMany ? __ldcg(static_cast<const double*>(terms) + i)
+                 : static_cast<double>(__ldcg(static_cast<const float*>(terms) + i));
   acc = block_sum(acc);
   if (threadIdx.x == 0) {
     if (reduction == OLIVE_REDUCE_MEAN) acc = n > 0 ? acc / n : 0.0;
     *loss = static_cast<float>(acc);
   }
+}
+__global__ void __launch_bounds__(128)
+    fwd_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows,
+                        const int32_t* __restrict__ targets, int T, int V, int vt, int ctas, int min_parts,
+                        const float* __restrict__ part_m, const float* __restrict__ part_s,
+                        const float* __restrict__ zy, float* __restrict__ logp,
+                        float* __restrict__ lse, void* terms, uint32_t* done, int reduction,
+                        float* __restrict__ loss, int32_t* dev_status) {
+  const int n = read_n_rows(n_rows, T, nullptr);
+  if (n <= kManyRows)
+    fwd_finalize<false>(n, rows, targets, T, V, vt, ctas, min_parts, part_m, part_s, zy, logp, lse, terms,
+                        done, reduction, loss, dev_status);
+  else
+    fwd_finalize<true>(n, rows, targets, T, V, vt, ctas, min_parts, part_m, part_s, zy, logp, lse, terms,
+                       done, reduction, loss, dev_status);
 }
 
 // One warp a row: lanes share the segments' sums and merge their top lists

@@ -198,25 +198,24 @@ struct KlFwdKern {
 };
 
 // kl[t] per masked row; with lse_p / lse_q non-null also both heads' lse per
-// compact row (p the primary head: the student for the reverse KL)
-// (as many lanes a row as it has segments: merge_lanes)
-__global__ void __launch_bounds__(128)
-    kl_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
-                       int vt, int ctas, size_t plane, const float* __restrict__ part,
-                       float* __restrict__ kl, float* __restrict__ lse_p_out,
-                       float* __restrict__ lse_q_out) {
-  const int n = read_n_rows(n_rows, T, nullptr);
+// compact row (p the primary head: the student for the reverse KL).  kMany beyond
+// kManyRows rows: as many lanes a row as it has segments, else a warp.
+template <bool kMany>
+__device__ __forceinline__ void kl_finalize(int n, const int32_t* __restrict__ rows, int T, int vt,
+                                            int ctas, size_t plane, const float* __restrict__ part,
+                                            float* __restrict__ kl, float* __restrict__ lse_p_out,
+                                            float* __restrict__ lse_q_out) {
   const Split sp = choose_split(n, vt, ctas, split_cap((n + 127) / 128, kMinParts));
   const int lane = threadIdx.x & 31;
   const size_t ld = static_cast<size_t>(sp.rt) * 128;
-  const int per = merge_lanes(sp.sv), sub = lane & (per - 1);
+  const int per = kMany ? merge_lanes(sp.sv) : 32, sub = lane & (per - 1);
   const int step = 32 / per;  // rows of a warp
   for (int r0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * step; r0 < n; r0 += gridDim.x * 4 * step) {
     const int r = r0 + lane / per;
     float Mp = -INFINITY, Mq = -INFINITY, Sp = 0.f, Sq = 0.f, A = 0.f;
     float f[2];
     if (r < n) {
-      for (int s = sub; s < sp.sv; s += per) {
+      for (int s = sub; s < sp.sv; s += 32) {  // (fewer lanes than 32 have no second segment)
         const size_t o = s * ld + r;
         merge_ms(Mp, Sp, part[0 * plane + o], part[1 * plane + o], f);
         A = A * f[0] + part[4 * plane + o] * f[1];
@@ -241,6 +240,15 @@ __global__ void __launch_bounds__(128)
       lse_q_out[r] = lse_q;
     }
   }
+}
+__global__ void __launch_bounds__(128)
+    kl_finalize_kernel(const int32_t* __restrict__ n_rows, const int32_t* __restrict__ rows, int T,
+                       int vt, int ctas, size_t plane, const float* __restrict__ part,
+                       float* __restrict__ kl, float* __restrict__ lse_p_out,
+                       float* __restrict__ lse_q_out) {
+  const int n = read_n_rows(n_rows, T, nullptr);
+  if (n <= kManyRows) kl_finalize<false>(n, rows, T, vt, ctas, plane, part, kl, lse_p_out, lse_q_out);
+  else kl_finalize<true>(n, rows, T, vt, ctas, plane, part, kl, lse_p_out, lse_q_out);
 }
 
 template <class K>

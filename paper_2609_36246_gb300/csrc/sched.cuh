@@ -97,8 +97,12 @@ __device__ inline int read_n_rows(const int32_t* n_rows, int T, int32_t* dev_sta
   return n;
 }
 
-// Lanes of a warp that share a row's sv segments when partials are merged: a
-// power of two, one segment each where 32 are enough.
+// Rows beyond which a merge of the sweeps' partials gives a row no more lanes than
+// it has segments (merge_lanes): a warp a row is quicker at few rows, which are
+// cut into many segments, and its code is shorter.
+constexpr int kManyRows = 1024;
+// Lanes of a warp that share a row's sv segments: a power of two, one segment
+// each where 32 are enough.
 __device__ __forceinline__ int merge_lanes(int sv) {
   int l = 1;
   while (l < sv && l < 32) l *= 2;

@@ -257,7 +257,7 @@ def test_few_rows_many_segments(n):
     close(opd["t_logp_s"][r][sure], lt.gather(1, want_i)[sure])
 
 
-@pytest.mark.parametrize("n", [1, 5, 131, 2433, 9729, 40000])
+@pytest.mark.parametrize("n", [1, 5, 131, 1024, 1025, 9729, 40000])
 @pytest.mark.parametrize("reduction", ["sum", "mean"])
 def test_loss_over_blocks_of_rows(n, reduction):
     """The loss is the sum of the blocks' sums, one block to many (and many rows
