@@ -394,3 +394,57 @@ def test_loss_with_row_indices_outside_the_batch(reduction):
                                                   slab=op == "loss_fwd_bwd_slab")[2]
             assert B.status_bits(st) == ["OLIVE_ERR_OFFSETS"]
             assert_close_loss(loss.item(), want)
+
+
+@pytest.mark.parametrize("grad_dtype", [torch.bfloat16, torch.float32])
+def test_gradient_written_over_its_input(grad_dtype):
+    """d_hidden in the memory of hidden (bf16), or in fp32 over the second half of
+    it: the rows are copied before the gradient's buffer is cleared, so the
+    results are those of separate buffers bit for bit."""
+    b, h, W = synth.random_case(94, 5, 900, 64, max_prefix=40, max_cont=90, std_w=0.1)
+    g = gpu_pack(b)
+    T, d = h.shape
+    Wc = W.cuda()
+    one = torch.ones(1, dtype=torch.float32, device="cuda")
+    wide = grad_dtype == torch.float32
+    at = T // 2 * d if wide else 0  # the gradient's first element, in bf16 elements
+
+    def buffers(apart):
+        mem = torch.zeros(at + T * d * (2 if wide else 1), dtype=torch.bfloat16, device="cuda")
+        hid = mem[: T * d].view(T, d)
+        hid.copy_(h)
+        dh = mem[at:].view(grad_dtype).view(T, d)
+        return hid, torch.empty_like(dh) if apart else dh
+
+    def call(op, apart):
+        hid, dh = buffers(apart)
+        st = B.new_status()
+        dw = torch.empty(900, d, dtype=grad_dtype, device="cuda")
+        f = lambda n: torch.empty(n, dtype=torch.float32, device="cuda")
+        if op == "bwd":
+            lse = torch.from_numpy(lse0).cuda()
+            out = B.olive_token_loss_bwd(hid, Wc, g["targets"], g["rows"], g["n_rows"], lse, one,
+                                         grad_dtype=grad_dtype, dev_status=st, out=(dh, dw))
+        elif op == "kl":
+            kl = f(T)
+            ws = B.workspace(B.olive_workspace_size("divergence", T, d, 900, d_t=d))
+            B._check(B.lib().olive_token_divergence(
+                B._ptr(hid), B._ptr(Wc), d, B._ptr(ht), B._ptr(Wc), d, B._ptr(g["rows"]),
+                B._ptr(g["n_rows"]), T, 900, 1.0, B.DIRECTION["reverse"], B._ptr(kl), B._ptr(weight),
+                B._ptr(dh), B.DTYPE[grad_dtype], B._ptr(ws), ws.numel(), B._ptr(st), B._stream()), op)
+            out = (kl, dh)
+        else:
+            out = B.olive_token_loss_fwd_bwd(hid, Wc, g["targets"], g["rows"], g["n_rows"], one,
+                                             grad_dtype=grad_dtype, dev_status=st, slab=op == "slab",
+                                             out=(f(T), f(T), f(1), dh, dw))
+        torch.cuda.synchronize()
+        assert B.status_bits(st) == []
+        return [x.clone() for x in out]
+
+    ht = h.flip(0).contiguous().cuda()
+    weight = torch.rand(T, device="cuda") + 0.5
+    lse0 = call("onchip", True)[1].cpu().numpy()
+    for op in ("onchip", "slab", "bwd", "kl"):
+        for x, y in zip(call(op, True), call(op, False)):
+            assert torch.equal(x, y), op
+        assert call(op, False)[-1 if op == "kl" else 0].any()
