@@ -48,10 +48,7 @@ struct TileC {
 
 constexpr int kBM = 128;
 constexpr int kBK = 64;
-constexpr int kThreads = 192;
 constexpr int kEpiThreads = 128;
-constexpr int kProducerWarp = 4;
-constexpr int kMmaWarp = 5;
 constexpr int kStatusTimeoutBit = 1 << 6;  // (1 << OLIVE_ERR_TIMEOUT)
 
 // Thread layout of a policy's CTA.
@@ -60,7 +57,6 @@ struct CoreThreads {
   static constexpr int kEpiWarps = Kern::kEpiWarps;
   static_assert(kEpiWarps == 4 || kEpiWarps == 8, "4 or 8 epilogue warps");
   static constexpr int kEpi = 32 * kEpiWarps;   // epilogue threads
-  static constexpr int kParts = kEpiWarps / 4;  // threads per accumulator row
   static constexpr int kProducer = kEpiWarps;
   static constexpr int kMma = kEpiWarps + 1;
   static constexpr int kAll = 32 * (kEpiWarps + 2);

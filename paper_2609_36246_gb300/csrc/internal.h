@@ -150,8 +150,8 @@ struct GroupWs {
   float* zy;         // [Tpad] target logits
   float* pyb;        // [Tpad] the targets' bf16 exchange-tile entries
   float* nll;        // [Tpad] per-row loss terms
-  float* part_s;     // [2 g_max, Tpad] partial sums per member and column half
-  float* part_m;     // [2 g_max, Tpad] partial maxima
+  float* part_s;     // [2 g_max, Tpad] partial sums per member (in its second row; the first is 0)
+  float* part_m;     // [2 g_max, Tpad] partial maxima per member and column half
   void* ring;        // group_ring_bytes(T, d, V)
   float* tail_acc;   // group_tail_bytes(T, d, V): partial accumulators of split row pairs
   float* tail_s;     // group_tail_sums(T, d, V): their row sums

@@ -831,7 +831,7 @@ __global__ void __launch_bounds__(256)
     const int t = r < in_s ? rows[row0 + r] : -1;
     uint4* hrow = hs + static_cast<size_t>(row0 + r) * d8;
     if (t < 0 || t >= T) {
-      // reported by the gather (masked rows); the G row is zero
+      // reported by prepare_kernel (masked rows); the G row is zero
       if (lane == 0) {
         lam[r] = 0.f;
         if (r < in_s) nll[row0 + r] = 0.f;
@@ -1073,7 +1073,7 @@ __global__ void __launch_bounds__(256) topk_kl_rows_kernel(const TopkKlRows a) {
     const int t = r < in_s ? a.rows[row0 + r] : -1;
     uint4* hrow = a.hs + static_cast<size_t>(row0 + r) * a.ds8;
     if (t < 0 || t >= a.T) {
-      // reported by the gather (masked rows); the G row is zero
+      // reported by prepare_kernel (masked rows); the G row is zero
       if (lane == 0) a.lam[r] = 0.f;
       for (int c = lane; c < a.ds8; c += 32) hrow[c] = make_uint4(0u, 0u, 0u, 0u);
       continue;

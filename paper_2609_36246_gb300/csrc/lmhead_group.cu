@@ -94,11 +94,27 @@
 // 21.8 against 18.6 ms (4096 rows, d_s = 4096, d_t = 5120; 17.4 ms now).
 // What bounds it now: the tensor pipe and, from some thousand rows on, the
 // power cap (16384 rows: pipe 90 % active in pass A, 87 % in pass B); at a few
-// hundred rows the rounds' exchange latency.  Every dependency
-// points to a tile of an earlier round, every CTA is resident at once (the
-// grid is one CTA per SM; the host checks that the GPU holds all its
-// clusters), and every wait is bounded (OLIVE_ERR_TIMEOUT on expiry).  A
-// pacing hint keeps the groups within a round of one another, so that one
+// hundred rows the rounds' exchange latency.
+//
+// Why the waits end: every CTA is resident at once (the grid is one CTA per SM;
+// the host checks that the GPU holds all its clusters), and each wait is for
+// work that does not wait for the waiter.
+//   - Within a pair-group a wait for an exchange tile (`ready`) or its slot
+//     (`cons`) is for work of an earlier round.
+//   - Pass A's merge of an outer tile's sums waits for the posts of all members
+//     that hold a part of it.  A member posts, takes its output accumulator out
+//     and hands it back before it waits, and its Z tile of the round is
+//     published by then, so the members of its own pair-group reach their posts
+//     of the same round without it.
+//   - Where a row pair of the tail is split between pair-groups, only the last
+//     member to arrive for its columns waits, for the posts of the row pair's
+//     other runs.  A run goes through its row pairs in ascending order, so what
+//     can keep it from its post is a wait on the row pair before, which in turn
+//     waits on runs of that one only: the chain ends at the tail's first row
+//     pair.  Passes B and the divergence add partials up without waiting.
+// Each is bounded all the same (OLIVE_ERR_TIMEOUT on expiry).
+//
+// A pacing hint keeps the groups within a round of one another, so that one
 // DRAM fetch of an inner operand tile (W in pass A, hc in pass B) can serve
 // every group from the L2 (how often it does depends on what else the L2
 // holds: the call reads the streamed operand several times over).
@@ -132,12 +148,12 @@ constexpr int kMmaWarp = kEpiWarps + 1;
 constexpr int kSignalWarp = kEpiWarps + 2;  // posts the members' "tile copied" counts
 constexpr int kLossWarp = kEpiWarps + 3;
 constexpr int kThreads = 32 * (kEpiWarps + 4);  // three whole warpgroups
+constexpr int kPieceMax = 4;  // K steps (~2000 cycles) of a Z product at an outer tile's boundary
 // Registers a thread: 168 at launch (65536 / 384 threads); the warpgroup of
 // the producer, MMA and signal warps hands most of its share to the two of
 // the epilogue, whose 128 held accumulator values otherwise spill (the L1 left
 // beside 227 KB of shared memory is too small for 384 stacks: spilled, a
 // 32-column block took ~5500 cycles).  2 x 216 + 72 = 3 x 168.
-constexpr int kPieceMax = 4;  // K steps (~2000 cycles) of a Z product at an outer tile's boundary
 constexpr int kEpiRegs = 216;
 constexpr int kOtherRegs = 72;
 constexpr int kStatusTimeoutBit = 1 << OLIVE_ERR_TIMEOUT;
@@ -185,7 +201,8 @@ struct GroupParams {
   const float* lse_in;      // [T] natural lse per packed row (GM_A lse_known, GM_B)
   float* rref;              // [Tpad] base-2 reference per compact row (GM_REF writes)
   float* rmax;              // [Tpad] base-2 row maximum (GM_A writes for redo rows)
-  float* part_s;            // [2 g][Tpad] sums of 2^(x - R) per member and column half
+  // per member, two rows of [Tpad] for the two column halves of its Z tiles
+  float* part_s;            // [2 g][Tpad] sums of 2^(x - R): the second's; the first's are 0
   float* part_m;            // [2 g][Tpad] the logits' maxima (base 2)
   float* zy;                // [Tpad] target logit z_y (natural units)
   float* pyb;               // [Tpad] P'_y as rounded to bf16 in the exchange tile
@@ -201,7 +218,7 @@ struct GroupParams {
   uint32_t* pace;           // [ngroups] rounds each group has begun (a pacing hint)
   // split row pairs (see GSched): partial accumulators [slot][2][g] of
   // kTailVecs float4 (in the order of the epilogue's threads), GM_A's partial
-  // sums and maxima [slot][2 g][2 x 128], and how many runs have left their
+  // sums (as in part_s) and maxima [slot][2 g][2 x 128], and how many runs have left their
   // partial per row tile and member
   float* tail_acc;
   float *tail_s, *tail_m;
@@ -1087,36 +1104,36 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int v = o * kBM + row;
             // does any of this half's columns have its target in the outer tile?
             bool hit = false;
-  #pragma unroll
+#pragma unroll
             for (int q = 0; q < 4; ++q)
               hit = hit || static_cast<uint32_t>(meta_y[half * 128 + q * 32 + lane] - o * kBM) < kBM;
             hit = __any_sync(0xffffffffu, hit);
-  #pragma unroll 1
+#pragma unroll 1
             for (int h = hbeg; h < hend; ++h) {
               uint32_t a[32];
               tmem_ld_32x32b_x32(zaddr + h * 32, a);
               tmem_ld_wait();
               drained(h);
               float gv[32];
-  #pragma unroll
+#pragma unroll
               for (int c = 0; c < 32; ++c)
                 gv[c] = s_coef * fast_exp2(fmaf(__uint_as_float(a[c]), p.scale2, -meta_l[h * 32 + c]));
               if (hit) {
                 // the target entry p - 1 from expm1, exact where p is near 1
-  #pragma unroll 1
+#pragma unroll 1
                 for (int c = 0; c < 32; ++c) {
                   if (meta_y[h * 32 + c] != v) continue;
                   float z = 0.f;
-  #pragma unroll
+#pragma unroll
                   for (int q = 0; q < 32; ++q) z = q == c ? __uint_as_float(a[q]) : z;
                   z = s_coef * expm1f(fmaf(z, p.scale2, -meta_l[h * 32 + c]) * kLn2);
-  #pragma unroll
+#pragma unroll
                   for (int q = 0; q < 32; ++q) gv[q] = q == c ? z : gv[q];
                 }
               }
               if (h * 32 + 32 > kv) {
                 // rows beyond the last one may hold anything, NaN too
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c) gv[c] = h * 32 + c < kv ? gv[c] : 0.f;
               }
               put(h, gv);
@@ -1128,7 +1145,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // g inv_tau (p_s - p_t).  The student's logits arrive first and wait
             // in registers for the teacher's.
             float zs_all[4][32];
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b)
               tmem_ld_32x32b_x32(zaddr + (hbeg + b) * 32, reinterpret_cast<uint32_t(&)[32]>(zs_all[b]));
             tmem_ld_wait();
@@ -1153,18 +1170,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             // log p_s - log p_t as (z_s - z_t) - (lse_s - lse_t): a teacher
             // shifted by a constant per row cancels before the large terms meet
             const float dl = ls0 - lt0;
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b) {
               const int h = hbeg + b;
               if (h >= hend) break;
               float(&gv)[32] = zs_all[b];
-  #pragma unroll
+#pragma unroll
               for (int u = 0; u < 32; u += 16) {
                 uint32_t zt_b[16];
                 tmem_ld_32x32b_x16(zaddr + h * 32 + u, zt_b);
                 tmem_ld_wait();
                 if (u) drained(h);
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 16; ++c) {
                   const float zs = gv[u + c] * p.inv_tau;
                   const float zt = __uint_as_float(zt_b[c]) * p.inv_tau;
@@ -1174,7 +1191,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
               }
               if (!valid || h * 32 + 32 > kv) {
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c) gv[c] = valid && h * 32 + c < kv ? gv[c] : 0.f;
               }
               put(h, gv);
@@ -1187,11 +1204,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               run_m = -INFINITY;
             }
             const int v0 = k * kZN;
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b) {
               const int h = hbeg + b;
               if (h >= hend) {
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c) pv_all[b][c] = 0.f;
                 continue;
               }
@@ -1203,7 +1220,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               // (two running maxima of x - R: shorter chains)
               float m1 = -INFINITY;
               if (h * 32 + 32 <= kv) {
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; c += 2) {
                   const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
                   const float x1 = fmaf(__uint_as_float(a[c + 1]), p.scale2, -ra.R);
@@ -1213,7 +1230,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   pv[c + 1] = fast_exp2(x1);
                 }
               } else {
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c) {
                   const bool in = h * 32 + c < kv;
                   const float x0 = fmaf(__uint_as_float(a[c]), p.scale2, -ra.R);
@@ -1227,7 +1244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // the target's exact logit and the bf16 value of P'_y the MMA
                 // sees: the epilogue replaces that term by p_y - 1 from the
                 // logit, so rows with p_y near 1 keep their accuracy
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c)
                   if (c == yo) {
                     p.zy[o * kBM + row] = __uint_as_float(a[c]) * p.inv_tau;
@@ -1262,9 +1279,9 @@ __global__ void __launch_bounds__(kThreads, 1)
               // times as far from 64 bits.)
               if (half) named_bar_sync(2, kEpi);
               float sum = !half && fresh ? 0.f : meta_l[row];
-  #pragma unroll
+#pragma unroll
               for (int b = 0; b < 4; ++b)
-  #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; ++c) sum += pv_all[b][c];
               meta_l[row] = sum;
               if (!half) named_bar_arrive(2, kEpi);
@@ -1311,10 +1328,10 @@ __global__ void __launch_bounds__(kThreads, 1)
               break;
             }
             float4* out = part(s.pg);
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b) {
               if (ob + 32 * b >= oe) continue;
-  #pragma unroll
+#pragma unroll
               for (int q = 0; q < 8; ++q)
                 out[(8 * b + q) * kEpi] =
                     make_float4(acc[b][4 * q], acc[b][4 * q + 1], acc[b][4 * q + 2], acc[b][4 * q + 3]);
@@ -1328,17 +1345,17 @@ __global__ void __launch_bounds__(kThreads, 1)
               __threadfence();
             }
             if (!named_bar_and(1, kEpi, last)) continue;
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b) {
-  #pragma unroll
+#pragma unroll
               for (int c = 0; c < 32; ++c) acc[b][c] = 0.f;
             }
             for (int c = run_lo; c <= run_hi; ++c) {
               const float4* in = part(c);
-  #pragma unroll
+#pragma unroll
               for (int b = 0; b < 4; ++b) {
                 if (ob + 32 * b >= oe) continue;
-  #pragma unroll
+#pragma unroll
                 for (int q = 0; q < 8; ++q) {
                   const float4 v = __ldcg(in + (8 * b + q) * kEpi);
                   acc[b][4 * q] += v.x;
@@ -1374,7 +1391,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float* ps = (split ? p.tail_s : p.part_s) + from;
             const float* pm = (split ? p.tail_m : p.part_m) + from;
             const int count = 2 * g * (run_hi - run_lo + 1);
-  #pragma unroll 8
+#pragma unroll 8
             for (int e2 = 0; e2 < count; ++e2) {
               sum += __ldcg(ps + e2 * stride);
               mx = fmaxf(mx, __ldcg(pm + e2 * stride));
@@ -1420,17 +1437,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const uint4* wy =
                 has_y ? reinterpret_cast<const uint4*>(p.W + static_cast<size_t>(rw.y) * p.d + s.c0) : nullptr;
-  #pragma unroll
+#pragma unroll
             for (int b = 0; b < 4; ++b) {
               const int c = ob + 32 * b;
               if (c >= oe) continue;
               const int nv = min(32, oe - c);
-  #pragma unroll
+#pragma unroll
               for (int q = 0; q < 4; ++q) {
                 uint4 w4 = make_uint4(0, 0, 0, 0);
                 if (wy && 8 * q < nv) w4 = __ldg(wy + c / 8 + q);
                 const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&w4);
-  #pragma unroll
+#pragma unroll
                 for (int u = 0; u < 4; ++u) {
                   const float2 wf = __bfloat1622float2(w2[u]);
                   float& a0 = acc[b][8 * q + 2 * u];

@@ -53,7 +53,7 @@ __global__ void topk_compare_kernel(const uint4* __restrict__ h_t, const uint4* 
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
     const int t = rows[r];
-    if (t < 0 || t >= T) continue;  // reported by the callers' gathers
+    if (t < 0 || t >= T) continue;  // reported where the lists were made
     const bool in_k = lane < K;
     const int sid = in_k ? s_ids[static_cast<size_t>(t) * K + lane] : -1;
     const float slp = in_k ? s_logp[static_cast<size_t>(t) * K + lane] : 0.f;
@@ -112,7 +112,7 @@ __global__ void topk_kl_prep_kernel(const int32_t* __restrict__ rows,
   const int n = read_n_rows(n_rows, T, dev_status);
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     const int t = rows[r];
-    if (t < 0 || t >= T) continue;  // reported by the backward's gather
+    if (t < 0 || t >= T) continue;  // reported by prepare_kernel
     const size_t o = static_cast<size_t>(t) * K;
     const float g = grad_kl[t] * inv_tau;
     float P = 0.f;
