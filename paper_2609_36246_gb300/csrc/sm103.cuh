@@ -442,7 +442,9 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* addr, uint32_t targ
 // below 2^-126 are 0, -inf gives 0, NaN stays.  For terms that meet a sum of at
 // least 1 (or their row's total) in 24 bits, where what is flushed cannot show.
 // A factor that is multiplied by something large, and an exponential that is
-// used by itself, take exp2f.
+// used by itself, take exp2f.  (exp2f in its place everywhere: the same results
+// bit for bit in seven cases, 300 rows of d = 256 97 -> 100 us, the divergence
+// gradient and the OPD statistics 1 % slower, the other calls level.)
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
