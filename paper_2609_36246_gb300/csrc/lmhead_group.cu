@@ -532,7 +532,9 @@ __device__ __forceinline__ RowA load_row_a(const GroupParams& p, const GSched& s
       if (p.mode == GM_A) {
         if (p.lse_known) a.R = p.lse_in[t] * kLog2e;
         else if (p.redo) a.R = p.rmax[rc];
-        else a.R = p.rref[rc];
+        // (a first tile of -inf logits alone is no reference: 0 finds the row's
+        // maximum, which the redo launch takes where it is out of range)
+        else a.R = p.rref[rc] == -INFINITY ? 0.f : p.rref[rc];
       }
     }
   }

@@ -448,3 +448,30 @@ def test_gradient_written_over_its_input(grad_dtype):
         for x, y in zip(call(op, True), call(op, False)):
             assert torch.equal(x, y), op
         assert call(op, False)[-1 if op == "kl" else 0].any()
+
+
+@pytest.mark.parametrize("level", [0.0, 90.0, -200.0])
+def test_first_tile_out_of_range(level):
+    """The first 256 logits (each row's reference) near the lowest fp32 value, whose
+    base-2 form is -inf, the others around `level`: in range of a reference of 0,
+    above it, and below."""
+    rng = np.random.default_rng(95)
+    V = 700
+    b = synth.batch_from_lengths(rng, [2, 3], [200, 90], V)
+    b.cont_ids[:] = 256 + b.cont_ids % (V - 256)
+    h = synth.normal_bf16(rng, (b.T, 64), 1.0)
+    h[:, 0] = 1.0
+    W = synth.normal_bf16(rng, (V, 64), 0.1)
+    W[:, 0] = level
+    W[:256, 0] = -3.3e38
+    logp, lse, loss, dh, dw = _gpu(b, h, W, grad_dtype=torch.float32)
+    o = oracle_pack(b)
+    args = (to_f64(h), to_f64(W), o["targets"], o["rows"])
+    rl, rlse, rloss = oracle.token_logprob(*args)
+    assert_close_logp(logp, rl)
+    assert_close_logp(lse, rlse, "lse")
+    assert_close_loss(loss, rloss)
+    rdh, rdw = oracle.token_loss_bwd(*args)
+    # (column 0 of dH is level * (sum p - 1): what rounding leaves of nothing)
+    assert_close_grad(dh[:, 1:], rdh[:, 1:], "dH")
+    assert_close_grad(dw, rdw, "dW")
