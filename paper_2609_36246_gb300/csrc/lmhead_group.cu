@@ -532,9 +532,7 @@ __device__ __forceinline__ RowA load_row_a(const GroupParams& p, const GSched& s
       if (p.mode == GM_A) {
         if (p.lse_known) a.R = p.lse_in[t] * kLog2e;
         else if (p.redo) a.R = p.rmax[rc];
-        // (a first tile of -inf logits alone is no reference: 0 finds the row's
-        // maximum, which the redo launch takes where it is out of range)
-        else a.R = p.rref[rc] == -INFINITY ? 0.f : p.rref[rc];
+        else a.R = p.rref[rc];
       }
     }
   }
@@ -1260,7 +1258,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // the row's two column halves meet in shared memory
             if (half) meta_l[row] = run_m;
             named_bar_sync(1, kEpi);
-            if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = fmaxf(run_m, meta_l[row]);
+            const float ref = fmaxf(run_m, meta_l[row]);
+            // (a tile of -inf logits alone is no reference: 0 finds the row's maximum,
+            // which the redo launch takes where it is out of range)
+            if (!half && o * kBM + row < s.n) p.rref[o * kBM + row] = ref == -INFINITY ? 0.f : ref;
             named_bar_sync(1, kEpi);
           } else {
             // publish the warp's part of the tile once its copies are complete
